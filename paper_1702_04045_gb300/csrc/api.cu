@@ -196,7 +196,7 @@ static int build_basis(Ctx* c, Basis& b) {
 static void free_basis(Basis& b) {
   void** ps[] = {(void**)&b.d_miller, (void**)&b.d_kin,    (void**)&b.d_kin32,  (void**)&b.d_col_x,
                  (void**)&b.d_col_y,  (void**)&b.d_col_off, (void**)&b.d_g_col,  (void**)&b.d_g_z,
-                 (void**)&b.d_xrows,  (void**)&b.d_xrow_c, (void**)&b.d_stick_of, (void**)&b.d_beta,   (void**)&b.d_beta32, (void**)&b.d_beta_img_cn, (void**)&b.d_beta_img_wx, (void**)&b.d_prec_base,
+                 (void**)&b.d_xrows,  (void**)&b.d_xrow_c, (void**)&b.d_stick_of, (void**)&b.d_beta,   (void**)&b.d_beta32, (void**)&b.d_beta_img_cn, (void**)&b.d_beta_img_wx, (void**)&b.beta_slices[0].cn, (void**)&b.beta_slices[1].cn, (void**)&b.d_prec_base,
                  (void**)&b.d_mg,
                  (void**)&b.d_psi,    (void**)&b.d_hpsi,   (void**)&b.d_psi32,  (void**)&b.d_hpsi32};
   for (void** p : ps) {
@@ -776,6 +776,7 @@ static cplx<T>* rows_ws(Ctx* c, const char* base, int ik) {
 // orthonormalisation, no Rayleigh-Ritz): the working-precision copy, H psi under the current potential
 // and the residual norms.
 static int adopt_orbitals(Ctx* c, int ik) {
+  PlainF64 plain(c);
   Basis& b = c->bases[ik];
   int st;
   double* w = static_cast<double*>(ws_get(c, "state_eps", (size_t)c->nb * sizeof(double)));
@@ -804,6 +805,7 @@ static int adopt_orbitals(Ctx* c, int ik) {
 
 // Rayleigh-Ritz of the span of the current orbitals (after a change of potential or a restart)
 static int reproject(Ctx* c, int ik) {
+  PlainF64 plain(c);
   Basis& b = c->bases[ik];
   const size_t n = (size_t)c->nb * b.npw;
   if (c->prec == PARO_MIXED) {
@@ -834,6 +836,7 @@ static bool carry_hx(Basis& b, int alg) {
 // One ParO step (Algorithm 1 or 2) of k-point ik at the current potential.
 template <typename T>
 static int paro_step_k(Ctx* c, int ik, int alg, double rel_tol, int max_it) {
+  PlainF64 plain(c);
   cplx<T>* X = rows_ws<T>(c, "X", ik);
   if (!X) return PARO_ERR_CUDA;
   cplx<T>* HX = carry_hx(c->bases[ik], alg) ? rows_ws<T>(c, "HX", ik) : nullptr;
@@ -856,6 +859,7 @@ __global__ void k_plane_delta(int n, const T* __restrict__ vnew, T* __restrict__
 // The merged SCF iteration in precision T (see paro_scf_step).
 template <typename T>
 static int scf_iteration(Ctx* c, const paro_scf_opts* o) {
+  PlainF64 plain(c);
   std::vector<cplx<T>*> xs(c->nk), hxs(c->nk, nullptr);
   std::vector<int> nxs(c->nk);
   int st;

@@ -268,6 +268,21 @@ template <typename T> static const cplx<T>* beta_of(const Basis& b);
 template <> const double2* beta_of<double>(const Basis& b) { return b.d_beta; }
 template <> const float2* beta_of<float>(const Basis& b) { return b.d_beta32; }
 
+// P[p][b] = <beta_p | psi_b> (nproj x nb). FP64: digit slices on the tensor cores (k_slice.cu). FP32 outside
+// the inexact inner solves: sums carried in a two-sum pair, because a long FP32 accumulation biases
+// |<beta|psi>|^2 (and with it the Rayleigh-Ritz H and the energy) at the 1e-6 level.
+template <typename T>
+int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P) {
+  const Basis& B = c->bases[ik];
+  if constexpr (sizeof(T) == 8) {
+    if (slices_on(c)) return kb_project_slice<double>(c, ik, nb, psi, P);
+  }
+  const bool carry = sizeof(T) == 4 && !c->tc_scope;
+  return gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, carry);
+}
+template int kb_project<double>(Ctx*, int, int, const double2*, double2*);
+template int kb_project<float>(Ctx*, int, int, const float2*, double2*);
+
 // H psi += beta (D o (beta^H psi))
 template <typename T>
 int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
@@ -290,11 +305,11 @@ int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
       return PARO_OK;
     }
   }
-  // FP32 projections outside the inexact inner solves carry their sums in a two-sum pair: a long FP32
-  // accumulation biases |<beta|psi>|^2 (and with it the Rayleigh-Ritz H and the energy) at the 1e-6 level
-  const bool carry = sizeof(T) == 4 && !c->tc_scope;
-  int st = gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, carry);
+  int st = kb_project<T>(c, ik, nb, psi, P);
   if (st) return st;
+  if constexpr (sizeof(T) == 8) {
+    if (slices_on(c)) return kb_update_slice<double>(c, ik, nb, P, hpsi);
+  }
   // W(k = p, m = b) = D_p P[p][b]
   return gemm_wx<T, T>(c, nb, B.npw, c->nproj, P, nb, false, c->d_dvec, beta_of<T>(B), B.npw, hpsi, B.npw, 1.0);
 }

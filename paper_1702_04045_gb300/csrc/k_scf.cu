@@ -367,6 +367,13 @@ int build_beta(Ctx* c) {
         *img = nullptr;
       }
     }
+    for (SliceImages& im : b.beta_slices) {
+      if (im.cn) {
+        PARO_CU(c, cudaStreamSynchronize(c->stream));
+        cudaFree(im.cn);
+        im = SliceImages();
+      }
+    }
     k_beta<<<dim3((b.npw + 127) / 128, c->nat), 128, 0, c->stream>>>(b.npw, c->nat, c->N[0], c->N[1], c->N[2], B,
                                                                     b.kcart[0], b.kcart[1], b.kcart[2], b.d_miller,
                                                                     ph, kph, c->kb_rc, c->omega, b.d_beta,
@@ -1079,13 +1086,9 @@ int energy_terms(Ctx* c, const double* rho_dev, double terms[7]) {
     if (c->have_kb) {
       double2* P = static_cast<double2*>(ws_get(c, "kb_proj", (size_t)c->nproj * c->nb * sizeof(double2)));
       if (!P) return PARO_ERR_CUDA;
-      // <beta|psi>: FP64 on the FP64 path; the mixed path projects its FP32 orbitals in FP32 with the
-      // sums carried in a two-sum pair (the energy sum itself stays FP64)
-      st = c->prec == PARO_MIXED && B.d_psi32
-               ? gemm_cn<float, float, float>(c, c->nproj, nocc, B.npw, B.d_beta32, B.npw, B.d_psi32, B.npw, P,
-                                              nocc, false, true)
-               : gemm_cn<double, double, double>(c, c->nproj, nocc, B.npw, B.d_beta, B.npw, B.d_psi, B.npw, P,
-                                                 nocc, false);
+      // <beta|psi> in the working precision (the energy sum itself stays FP64)
+      st = c->prec == PARO_MIXED && B.d_psi32 ? kb_project<float>(c, ik, nocc, B.d_psi32, P)
+                                              : kb_project<double>(c, ik, nocc, B.d_psi, P);
       if (st) return st;
       k_nonlocal<<<nocc, 256, 0, c->stream>>>(c->nproj, nocc, P, c->d_dvec, pn + (size_t)ik * nocc);
       PARO_LAUNCH(c, "k_nonlocal");

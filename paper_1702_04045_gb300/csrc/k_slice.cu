@@ -1,0 +1,809 @@
+// Complex GEMMs with FP64 (or better than FP32) accuracy on the bf16 tensor cores, by error-free slicing
+// (Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix multiplication", Numer. Algorithms 59,
+// 2012; the tensor-core form of Mukunoki, Ozaki, Ogita, Imamura, ISC 2020): the FP64 pipe of this chip does
+// 1.25 TFLOP/s, its bf16 tensor cores about 2 PFLOP/s.
+//
+// Every operand row is brought to a common exponent (|x| < 2^e), rounded to an integer of 8 L - 1 bits and
+// sign and written in L balanced base-256 digits, d_i in [-128, 128], which bf16 holds exactly:
+//   x = 2^(e + 1) sum_i d_i 256^-i.
+// A product of rows is sum over (i, j) of 256^-(i+j) (d_i . d'_j). The digit products are integers of at most
+// 2^14, and a chunk of K values is short enough that the sums of all (i, j) with one i + j = g stay below
+// 2^24, so the tensor core's FP32 accumulation of each group g is exact. After every chunk the groups are
+// read from tensor memory and added into 64-bit integers at their weights; floating point appears only in
+// the final conversion. Groups up to g = PMAX are kept:
+//   L = 7, PMAX = 9 (34 digit products): operands rounded to 2^-56 of the row's largest power of two, groups
+//     dropped below 2^-57: FP64 results, more accurate than FP64 sums of the same length;
+//   L = 4, PMAX = 5 (10 products): operands rounded to 2^-32, for FP32 operands outside the inner solves.
+//
+// Measured on the 64-atom cell (N_pw = 23847): V_nl of 144 FP64 orbitals 17.7 -> 0.68 ms, Cholesky
+// orthonormalisation of 288 rows 31.8 -> 3.1 ms (2.1 ms of it the factorisation); the error against extended
+// precision is 3e-17 of the rows' norms where FP64 sums have 3e-15. A stage (16 K values) of a 128 x 32 tile takes
+// 1.8 us, 53 cycles per MMA of 64 columns against 48 for its operands' shared-memory traffic: the tensor
+// pipe's operand feed bounds it, the loads (79 KB a stage) and the sums are hidden.
+//
+// C[m][n] = sum_k conj(a_m,k) b_n,k with planes of real and imaginary digits: the A tile holds 128 rows, the
+// B tile NC rows three times (b_r; b_i; -b_r), so that a_r meets (b_r | b_i) and a_i meets (b_i | -b_r) as
+// one MMA of 2 NC columns each: Re and Im side by side in tensor memory.
+#include <algorithm>
+#include <type_traits>
+
+#include "paro_ctx.h"
+#include "tc_sm100.cuh"
+
+namespace paro {
+
+static const int kSliceM = 128;           // rows of the A tile (TMEM lanes)
+static const int kSliceK = 16;            // complex K values per stage (one MMA K step per plane)
+static const int kSliceThreads = 320;     // producer warp, MMA warp, eight epilogue warps
+static const uint32_t kSlicePolls = 1u << 24;
+
+// NC: columns of an output tile (2 NC accumulator columns per group fill the 512 of tensor memory);
+// CH: stages per exact chunk: 2 (planes) * 16 CH * 2^14 * (most pairs in a group) < 2^24; NS: stage buffers
+template <int L> struct SliceCfg;
+template <> struct SliceCfg<7> { static constexpr int NC = 32, PMAX = 9, CH = 4, NS = 2; };
+template <> struct SliceCfg<4> { static constexpr int NC = 64, PMAX = 5, CH = 8, NS = 3; };
+
+template <int L> __host__ __device__ constexpr int slice_a_bytes() { return L * 2 * kSliceM * kSliceK * 2; }
+template <int L> __host__ __device__ constexpr int slice_b_bytes() { return L * 3 * SliceCfg<L>::NC * kSliceK * 2; }
+
+// ------------------------------------------------------------------------------------------------
+// digits
+// ------------------------------------------------------------------------------------------------
+// key: bits whose integer order is that of |x| (the high word for doubles); ex: biased exponent
+__device__ __forceinline__ int slice_key(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int slice_key(float x) { return __float_as_int(x) & 0x7fffffff; }
+template <typename T> __device__ __forceinline__ int slice_key_exp(int key) { return sizeof(T) == 8 ? key >> 20 : key >> 23; }
+// the row exponent e (|x| < 2^e for every x of the row) from the row's largest key; bad: Inf or NaN inside
+template <typename T> __device__ __forceinline__ int slice_exponent(int key, bool* bad) {
+  const int ex = slice_key_exp<T>(key);
+  *bad = ex == (sizeof(T) == 8 ? 0x7ff : 0xff);
+  return max(ex, 1) - (sizeof(T) == 8 ? 1022 : 126);
+}
+// round(x 2^(8 L - 1 - e)), halves away from zero
+template <int L> __device__ __forceinline__ long long slice_fixed(double x, int e) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  unsigned long long u = ((unsigned long long)(hi & 0xfffff) << 32) | (unsigned)__double2loint(x);
+  if (ex) u |= 1ull << 52;
+  const int s = max(ex, 1) - 1075 + 8 * L - 1 - e;
+  if (s >= 0) u <<= min(s, 63);
+  else u = s < -55 ? 0ull : (u + (1ull << (-s - 1))) >> -s;
+  return hi < 0 ? -(long long)u : (long long)u;
+}
+template <int L> __device__ __forceinline__ long long slice_fixed(float x, int e) {
+  const int b = __float_as_int(x), ex = (b >> 23) & 0xff;
+  unsigned long long u = (unsigned)(b & 0x7fffff);
+  if (ex) u |= 1u << 23;
+  const int s = max(ex, 1) - 150 + 8 * L - 1 - e;
+  if (s >= 0) u <<= min(s, 63);
+  else u = s < -26 ? 0ull : (u + (1ull << (-s - 1))) >> -s;
+  return b < 0 ? -(long long)u : (long long)u;
+}
+// balanced digits of F, most significant first, as bf16 bits in the upper half of d[i]
+template <int L> __device__ __forceinline__ void slice_digits(long long F, uint32_t d[L]) {
+  long long carry = 0;
+#pragma unroll
+  for (int i = 0; i < L - 1; ++i) carry |= 128ll << (8 * i);
+  const long long t = F + carry;  // each low byte now holds its digit + 128
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const int sh = 8 * (L - 1 - i);
+    const uint32_t v = i == 0 ? (uint32_t)(t >> sh) + 128u : (uint32_t)(t >> sh) & 255u;
+    d[i] = __float_as_uint(__uint_as_float(0x4B000000u | v) - 8388736.0f);  // v - 128, exact
+  }
+}
+__device__ __forceinline__ uint32_t slice_pack(uint32_t d0, uint32_t d1) { return __byte_perm(d0, d1, 0x7632); }
+
+// result scale of a row: 2^(e + 1 - 4 PMAX) (a result is the integer sum times the scales of its two rows)
+template <int L> __device__ __forceinline__ int slice_scale(int e) { return e + 1 - 4 * SliceCfg<L>::PMAX; }
+static const int kSliceBad = 1 << 20;  // scale of a row with Inf or NaN: its results are NaN
+
+// eight consecutive k of one row (|v_j| < 2^e_j) -> its 16-byte core-matrix rows of every slice and plane
+template <int L, typename T>
+__device__ __forceinline__ void slice_store(const cplx<T>* v, const int* e, bool conj_a, unsigned char* a_dst,
+                                            unsigned char* b_dst) {
+  constexpr int NCB = SliceCfg<L>::NC * kSliceK * 2;
+  uint32_t wr[L][4], wi[L][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    uint32_t d0[L], d1[L];
+    slice_digits<L>(slice_fixed<L>(v[2 * q].x, e[2 * q]), d0);
+    slice_digits<L>(slice_fixed<L>(v[2 * q + 1].x, e[2 * q + 1]), d1);
+#pragma unroll
+    for (int i = 0; i < L; ++i) wr[i][q] = slice_pack(d0[i], d1[i]);
+    slice_digits<L>(slice_fixed<L>(v[2 * q].y, e[2 * q]), d0);
+    slice_digits<L>(slice_fixed<L>(v[2 * q + 1].y, e[2 * q + 1]), d1);
+#pragma unroll
+    for (int i = 0; i < L; ++i) wi[i][q] = slice_pack(d0[i], d1[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < L; ++i) {
+    const uint4 r = make_uint4(wr[i][0], wr[i][1], wr[i][2], wr[i][3]);
+    const uint4 m = make_uint4(wi[i][0], wi[i][1], wi[i][2], wi[i][3]);
+    const uint32_t neg = 0x80008000u;  // sign of both bf16 values
+    if (a_dst) {
+      *reinterpret_cast<uint4*>(a_dst + (size_t)(2 * i) * kSliceM * kSliceK * 2) = r;
+      *reinterpret_cast<uint4*>(a_dst + (size_t)(2 * i + 1) * kSliceM * kSliceK * 2) =
+          conj_a ? make_uint4(m.x ^ neg, m.y ^ neg, m.z ^ neg, m.w ^ neg) : m;
+    }
+    if (b_dst) {
+      unsigned char* p = b_dst + (size_t)i * 3 * NCB;
+      *reinterpret_cast<uint4*>(p) = r;
+      *reinterpret_cast<uint4*>(p + NCB) = m;
+      *reinterpret_cast<uint4*>(p + 2 * NCB) = make_uint4(r.x ^ neg, r.y ^ neg, r.z ^ neg, r.w ^ neg);
+    }
+  }
+}
+
+// byte offset of (row r of the tile, k8 of the stage) in a plane: 8-row x 16-byte core matrices
+__device__ __forceinline__ size_t slice_core(int r, int c) { return (size_t)((r >> 3) * 2 + c) * 128 + (r & 7) * 16; }
+
+template <int L>
+__device__ __forceinline__ unsigned char* slice_a_at(unsigned char* img, int nstage, int row, int k8) {
+  return img + ((size_t)(row / kSliceM) * nstage + (k8 >> 1)) * slice_a_bytes<L>() + slice_core(row % kSliceM, k8 & 1);
+}
+template <int L>
+__device__ __forceinline__ unsigned char* slice_b_at(unsigned char* img, int nstage, int row, int k8) {
+  constexpr int NC = SliceCfg<L>::NC;
+  return img + ((size_t)(row / NC) * nstage + (k8 >> 1)) * slice_b_bytes<L>() + slice_core(row % NC, k8 & 1);
+}
+
+// Rows along contiguous k (orbitals, projectors): 8 rows x one K slice per CTA. Exponents are those of the
+// slice (es[z][row], ld rows_pad). a_img, b_img: either may be null.
+template <typename T, int L>
+__global__ void __launch_bounds__(256) k_slice_rows(int rows, int rows_a, int rows_b, int K, int kslice, int nstage,
+                                                    const cplx<T>* __restrict__ x, int ld, int conj_a,
+                                                    unsigned char* __restrict__ a_img,
+                                                    unsigned char* __restrict__ b_img, int* __restrict__ es,
+                                                    int rows_pad) {
+  __shared__ int skey[8];
+  const int r = threadIdx.x & 7, row = blockIdx.x * 8 + r, z = blockIdx.y;
+  const int k0 = z * kslice, k1 = min(nstage * kSliceK, k0 + kslice);  // padded K: zeros past K
+  if (threadIdx.x < 8) skey[threadIdx.x] = 0;
+  __syncthreads();
+  const cplx<T>* xr = x + (size_t)min(row, rows - 1) * ld;
+  int key = 0;
+  if (row < rows)
+    for (int k = k0 + (threadIdx.x >> 3); k < min(k1, K); k += 32) {
+      const cplx<T> v = xr[k];
+      key = max(key, max(slice_key(v.x), slice_key(v.y)));
+    }
+  atomicMax(&skey[r], key);
+  __syncthreads();
+  bool bad;
+  const int e = slice_exponent<T>(skey[r], &bad);
+  if (threadIdx.x < 8) es[(size_t)z * rows_pad + row] = bad ? kSliceBad : slice_scale<L>(e);
+  for (int k8 = k0 / 8 + (threadIdx.x >> 3); k8 < k1 / 8; k8 += 32) {
+    cplx<T> v[8];
+    int ev[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] = row < rows && 8 * k8 + j < K ? xr[8 * k8 + j] : mk<T>(0, 0);
+      ev[j] = e;
+    }
+    slice_store<L, T>(v, ev, conj_a != 0, a_img && row < rows_a ? slice_a_at<L>(a_img, nstage, row, k8) : nullptr,
+                      b_img && row < rows_b ? slice_b_at<L>(b_img, nstage, row, k8) : nullptr);
+  }
+}
+
+// Largest finite key of every row of X[k][n] (rowkey cleared by the caller).
+template <typename T>
+__global__ void __launch_bounds__(256) k_slice_rowkey(int N, const cplx<T>* __restrict__ x, int ld,
+                                                      int* __restrict__ rowkey) {
+  const cplx<T>* xr = x + (size_t)blockIdx.y * ld;
+  int key = 0;
+  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+    const cplx<T> v = xr[n];
+    const int a = slice_key(v.x), b = slice_key(v.y);
+    if (slice_key_exp<T>(a) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, a);
+    if (slice_key_exp<T>(b) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, b);
+  }
+  key = __reduce_max_sync(0xffffffffu, key);
+  if ((threadIdx.x & 31) == 0) atomicMax(&rowkey[blockIdx.y], key);
+}
+// An update sums over the rows of X, whose sizes may differ widely (orbitals beside small corrections): the
+// digits are taken of X[k][n] 2^-c_k and W(k, m) 2^c_k with c_k the exponent of row k, so that every row
+// keeps its own accuracy. c_k = 0 without row keys (the projectors, all of one size).
+template <typename T> __device__ __forceinline__ int slice_rowshift(const int* rowkey, int k) {
+  if (!rowkey) return 0;
+  const int key = rowkey[k];
+  return key ? max(slice_key_exp<T>(key), 1) - (sizeof(T) == 8 ? 1022 : 126) : 0;
+}
+// running maximum of the exponents of v 2^-shift; Inf and NaN beat every number
+static const int kSliceNonfinite = 1 << 16;
+template <typename T> __device__ __forceinline__ int slice_top(cplx<T> v, int shift) {
+  const int key = max(slice_key(v.x), slice_key(v.y));
+  const int ex = slice_key_exp<T>(key);
+  if (ex == (sizeof(T) == 8 ? 0x7ff : 0xff)) return kSliceNonfinite;
+  return key ? max(ex, 1) - (sizeof(T) == 8 ? 1022 : 126) - shift : -kSliceNonfinite;
+}
+
+// Columns of X[k][n] as A rows (row n, K = the K rows of X), conjugated (the GEMM conjugates them back):
+// 32 columns per CTA, eight warps over k.
+template <typename T, int L>
+__global__ void __launch_bounds__(256) k_slice_cols(int N, int K, int nstage, const cplx<T>* __restrict__ x, int ld,
+                                                    const int* __restrict__ rowkey,
+                                                    unsigned char* __restrict__ a_img, int* __restrict__ es) {
+  __shared__ int stop[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = blockIdx.x * 32 + lane;
+  if (threadIdx.x < 32) stop[threadIdx.x] = -kSliceNonfinite;
+  __syncthreads();
+  int top = -kSliceNonfinite;
+  if (n < N)
+    for (int k = warp; k < K; k += 8) top = max(top, slice_top<T>(x[(size_t)k * ld + n], slice_rowshift<T>(rowkey, k)));
+  atomicMax(&stop[lane], top);
+  __syncthreads();
+  const bool bad = stop[lane] == kSliceNonfinite;
+  const int e = stop[lane] == -kSliceNonfinite ? 0 : stop[lane];
+  if (warp == 0) es[n] = bad ? kSliceBad : slice_scale<L>(e);
+  for (int k8 = warp; k8 < 2 * nstage; k8 += 8) {
+    cplx<T> v[8];
+    int ev[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = 8 * k8 + j;
+      v[j] = n < N && k < K ? x[(size_t)k * ld + n] : mk<T>(0, 0);
+      ev[j] = e + (k < K ? slice_rowshift<T>(rowkey, k) : 0);
+    }
+    slice_store<L, T>(v, ev, true, slice_a_at<L>(a_img, nstage, n, k8), nullptr);
+  }
+}
+
+// The small matrix of an update as B rows: row m, value s_k W(k, m) 2^c_k (element (k, m) at W[k ldw + m], or
+// at W[m ldw + k] when wt); 8 rows per CTA. TX: type of X, whose row keys give c_k.
+template <int L, typename TX>
+__global__ void __launch_bounds__(256) k_slice_w(int M, int K, int nstage, const double2* __restrict__ W, int ldw,
+                                                 int wt, const double* __restrict__ s,
+                                                 const int* __restrict__ rowkey, unsigned char* __restrict__ b_img,
+                                                 int* __restrict__ es) {
+  __shared__ int stop[8];
+  const int r = threadIdx.x & 7, m = blockIdx.x * 8 + r;
+  if (threadIdx.x < 8) stop[threadIdx.x] = -kSliceNonfinite;
+  __syncthreads();
+  auto at = [&](int k) {
+    if (m >= M || k >= K) return make_double2(0.0, 0.0);
+    const double2 w = wt ? W[(size_t)m * ldw + k] : W[(size_t)k * ldw + m];
+    return s ? cscale(w, s[k]) : w;
+  };
+  int top = -kSliceNonfinite;
+  for (int k = threadIdx.x >> 3; k < K; k += 32) top = max(top, slice_top<double>(at(k), -slice_rowshift<TX>(rowkey, k)));
+  atomicMax(&stop[r], top);
+  __syncthreads();
+  const bool bad = stop[r] == kSliceNonfinite;
+  const int e = stop[r] == -kSliceNonfinite ? 0 : stop[r];
+  if (threadIdx.x < 8) es[m] = bad ? kSliceBad : slice_scale<L>(e);
+  for (int k8 = threadIdx.x >> 3; k8 < 2 * nstage; k8 += 32) {
+    double2 v[8];
+    int ev[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = 8 * k8 + j;
+      v[j] = at(k);
+      ev[j] = e - (k < K ? slice_rowshift<TX>(rowkey, k) : 0);
+    }
+    slice_store<L, double>(v, ev, false, nullptr, slice_b_at<L>(b_img, nstage, m, k8));
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// integer sums -> floating point
+// ------------------------------------------------------------------------------------------------
+// (hi 2^32 + lo) 2^k, rounded to nearest, by integer instructions (the FP64 pipe issues 1/64 of their rate)
+__device__ __forceinline__ double slice_to_double(long long hi, long long lo, int k) {
+  // 128-bit sum, two's complement
+  const unsigned long long h0 = (unsigned long long)hi << 32;
+  long long t1 = hi >> 32;
+  unsigned long long t0 = h0 + (unsigned long long)lo;
+  t1 += (lo >> 63) + (t0 < h0 ? 1 : 0);
+  const bool neg = t1 < 0;
+  if (neg) {
+    t0 = 0ull - t0;
+    t1 = ~t1 + (t0 == 0 ? 1 : 0);
+  }
+  if ((t1 | (long long)t0) == 0) return 0.0;
+  // the leading 64 bits m (bit 63 set), value m 2^sh, the rest into a sticky bit
+  int sh = 0;
+  unsigned long long m;
+  if (t1) {
+    const int z = __clzll(t1);
+    sh = 64 - z;
+    m = z ? ((unsigned long long)t1 << z) | (t0 >> (64 - z)) : (unsigned long long)t1;
+    if (z < 64 && (t0 << z)) m |= 1ull;
+  } else {
+    const int z = __clzll((long long)t0);
+    sh = -z;
+    m = t0 << z;
+  }
+  int ex = sh + k + 63 + 1023;  // biased exponent of the leading bit
+  if (ex >= 2047) return neg ? -INFINITY : INFINITY;
+  int drop = 11;
+  if (ex <= 0) {  // denormal result
+    drop = 12 - ex;
+    ex = 0;
+    if (drop > 64) return neg ? -0.0 : 0.0;
+  }
+  unsigned long long q = drop < 64 ? m >> drop : 0ull;
+  const unsigned long long rem = drop < 64 ? m << (64 - drop) : m;
+  if (rem > (1ull << 63) || (rem == (1ull << 63) && (q & 1ull))) ++q;
+  // q holds the leading bit at 52 for normal results: the carry of rounding moves into the exponent
+  const unsigned long long bits = ex > 0 ? ((unsigned long long)(ex - 1) << 52) + q : q;
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+// lo 2^k in FP32 (one rounding of the sum's leading 24 bits, one more only for results below 2^-126)
+__device__ __forceinline__ float slice_to_float(long long lo, int k) { return ldexpf(__ll2float_rn(lo), k); }
+
+// ------------------------------------------------------------------------------------------------
+// the GEMM
+// ------------------------------------------------------------------------------------------------
+namespace tc {
+// Instruction descriptor of kind::f16 with bf16 operands: D FP32, both K-major, M x N tile.
+__host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+}
+// 1 in one lane of a converged warp, 0 in the others. The compiler knows the result for what it is and keeps
+// the operands of the instructions it guards in uniform registers: 53 instead of 78 cycles per MMA here.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(r));
+  return r;
+}
+// executed by a whole warp, issued by the lane whose leader is nonzero
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p, q;\n"
+      "setp.ne.u32 p, %4, 0;\n"
+      "setp.ne.u32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+      "}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
+      : "memory");
+}
+// no-swizzle K-major descriptor (smem_desc with lbo 128, sbo 256) from its low word
+__device__ __forceinline__ uint64_t desc_lo(uint32_t lo) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"((256u >> 4) | 1u << 14));
+  return d;
+}
+// 32 lanes x 16 columns, not waited for
+__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+}  // namespace tc
+
+// acc += v * W (one wide multiply-add)
+template <int W> __device__ __forceinline__ void slice_acc(long long& acc, int v) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(v), "n"(W));
+}
+
+// MODE 0: part[z][m][n] = C over K slice z (complex double; M x N), herm: tiles wholly left of the diagonal
+// are skipped. MODE 1: Y[n][m] (+)= C[m][n] (the update: A rows are the long axis of Y), OUT = double or float;
+// lower: B is lower triangular and the stages past a tile's last row are left out.
+template <int L, int MODE, typename OUT>
+__global__ void __launch_bounds__(kSliceThreads, 1)
+    k_slice_gemm(int M, int N, int nstage_all, int kstages, const unsigned char* __restrict__ a_img,
+                 const int* __restrict__ ea, int ea_ld, const unsigned char* __restrict__ b_img,
+                 const int* __restrict__ eb, int eb_ld, cplx<OUT>* __restrict__ out, int ldo, int herm, int lower,
+                 int accum, int* __restrict__ err) {
+  using Cfg = SliceCfg<L>;
+  constexpr int NC = Cfg::NC, PMAX = Cfg::PMAX, CH = Cfg::CH, NS = Cfg::NS, NG = PMAX - 1;
+  constexpr int AB = slice_a_bytes<L>(), BB = slice_b_bytes<L>(), BUF = AB + BB;
+  constexpr int HC = NC / 2;                 // columns per epilogue thread
+  constexpr int NSUM = NG > 4 ? 2 : 1;       // 64-bit sums per value (four groups each)
+  static_assert(2 * NC * NG <= 512 && HC % 16 == 0, "tensor memory columns");
+  extern __shared__ __align__(128) unsigned char smem_dyn[];
+  unsigned char* smem = tc_align1024(smem_dyn);
+  __shared__ uint64_t full[NS], freeb[NS], gfull[NG], gfree[NG];
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_fail, s_last_commit, s_last_copy[NS];
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  // MODE 1: column tiles fastest, so CTAs in flight share the long operand's tile in L2
+  const int nt = blockIdx.x, mt = blockIdx.y, z = blockIdx.z;
+  const int m0 = mt * kSliceM, n0 = nt * NC;
+  if (herm && n0 + NC - 1 < m0) return;
+  const int st0 = z * kstages;
+  int nst = max(0, min(kstages, nstage_all - st0));
+  if (lower) nst = min(nst, (n0 + NC + kSliceK - 1) / kSliceK);  // b_n,k = 0 for k > n
+  if (tid == 0) {
+    for (int b = 0; b < NS; ++b) {
+      tc::mbar_init(&full[b], 1);
+      tc::mbar_init(&freeb[b], 1);
+      s_last_copy[b] = -1;
+    }
+    for (int g = 0; g < NG; ++g) {
+      tc::mbar_init(&gfull[g], 1);
+      tc::mbar_init(&gfree[g], kSliceThreads - 64);
+    }
+    s_fail = 0;
+    s_last_commit = -1;
+    tc::fence_mbar_init();
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&tmem_base, 512u);
+    tc::tmem_relinquish();
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  tc::tc_fence_after();
+  const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+  volatile int* vfail = &s_fail;
+  const int nchunk = (nst + CH - 1) / CH;
+  long long acc[NSUM][2][HC];
+#pragma unroll
+  for (int q = 0; q < NSUM; ++q)
+#pragma unroll
+    for (int j = 0; j < HC; ++j) acc[q][0][j] = acc[q][1][j] = 0;
+  if (tid == 0) {  // operand tiles: two bulk copies per stage
+    for (int s = 0; s < nst && !*vfail; ++s) {
+      const int b = s % NS;
+      if (s >= NS && !tc::mbar_wait(&freeb[b], (uint32_t)(s / NS - 1) & 1u, kSlicePolls)) {
+        *vfail = 1;
+        break;
+      }
+      tc::mbar_arrive_expect_tx(&full[b], (uint32_t)BUF);
+      tc::bulk_g2s(smem + b * BUF, a_img + ((size_t)mt * nstage_all + st0 + s) * AB, (uint32_t)AB, &full[b]);
+      tc::bulk_g2s(smem + b * BUF + AB, b_img + ((size_t)nt * nstage_all + st0 + s) * BB, (uint32_t)BB, &full[b]);
+      s_last_copy[b] = s;
+    }
+  } else if (warp == 1) {  // the MMAs: group by group, so that a chunk's first groups drain while its last are formed
+    const uint32_t leader = tc::elect_one();
+    constexpr uint32_t idesc = tc::idesc_bf16(128, 2 * NC);
+    for (int s = 0; s < nst; ++s) {
+      const int b = s % NS, ch = s / CH;
+      const bool first = s % CH == 0, last = s % CH == CH - 1 || s == nst - 1;
+      // votes keep the loop's control flow, and with it the descriptors, uniform over the warp
+      if (!__all_sync(0xffffffffu, !*vfail && tc::mbar_wait(&full[b], (uint32_t)(s / NS) & 1u, kSlicePolls))) {
+        *vfail = 1;
+        break;
+      }
+      tc::tc_fence_after();
+      // descriptors by their low words: the stage's base plus constant offsets (in 16 bytes); the issuing
+      // thread's instructions per MMA are what the tensor pipe would otherwise wait for
+      const uint32_t a0 = (tc::smem_addr(smem + b * BUF) >> 4) | (128u >> 4) << 16, b0 = a0 + (uint32_t)(AB >> 4);
+      bool okg = true;
+#pragma unroll
+      for (int g = 2; g <= PMAX; ++g) {
+        if (first && ch > 0 && okg) {
+          okg = __all_sync(0xffffffffu, tc::mbar_wait(&gfree[g - 2], (uint32_t)(ch - 1) & 1u, kSlicePolls));
+          tc::tc_fence_after();
+        }
+        if (okg) {
+          const uint32_t d = tm + (uint32_t)((g - 2) * 2 * NC);
+#pragma unroll
+          for (int i = g > L ? g - L : 1; i <= (g > L ? L : g - 1); ++i) {
+            const uint32_t ai = a0 + (uint32_t)((i - 1) * 2 * (kSliceM * kSliceK * 2) >> 4);
+            const uint32_t bj = b0 + (uint32_t)((g - i - 1) * 3 * (NC * kSliceK * 2) >> 4);
+            tc::mma_bf16(d, tc::desc_lo(ai), tc::desc_lo(bj), idesc, first && i == (g > L ? g - L : 1) ? 0u : 1u, leader);
+            tc::mma_bf16(d, tc::desc_lo(ai + (kSliceM * kSliceK * 2 >> 4)), tc::desc_lo(bj + (NC * kSliceK * 2 >> 4)),
+                         idesc, 1u, leader);
+          }
+          if (last && leader) tc::mma_commit(&gfull[g - 2]);
+        }
+      }
+      if (!okg) {
+        *vfail = 1;
+        break;
+      }
+      if (leader) {
+        tc::mma_commit(&freeb[b]);
+        s_last_commit = s;
+      }
+    }
+  } else if (warp >= 2) {  // the sums: TMEM lanes 32 (warp % 4) .., columns HC half .. of Re and of Im
+    const uint32_t base = tm + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(((warp - 2) >> 2) * HC);
+    bool okc = true;
+    for (int ch = 0; ch < nchunk && okc; ++ch) {
+#pragma unroll
+      for (int g = 0; g < NG; ++g) {
+        if (okc && (*vfail || !tc::mbar_wait(&gfull[g], (uint32_t)ch & 1u, kSlicePolls))) okc = false;
+        okc = __all_sync(0xffffffffu, okc);
+        if (!okc) continue;
+        tc::tc_fence_after();
+#pragma unroll
+        for (int c0 = 0; c0 < HC; c0 += 16) {
+          uint32_t re[16], im[16];
+          tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + c0), re);
+          tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + NC + c0), im);
+          tc::tmem_ld_wait();
+          if (c0 + 16 == HC) {
+            tc::tc_fence_before();
+            tc::mbar_arrive(&gfree[g]);
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            // weight 256^(PMAX - g): four groups per 64-bit sum
+            constexpr int kW[4] = {1 << 24, 1 << 16, 1 << 8, 1};
+            const int ir = __float2int_rn(__uint_as_float(re[j])), ii = __float2int_rn(__uint_as_float(im[j]));
+            long long &ar = acc[NSUM == 2 ? g / 4 : 0][0][c0 + j], &ai = acc[NSUM == 2 ? g / 4 : 0][1][c0 + j];
+            if (g % 4 == 0) { slice_acc<kW[0]>(ar, ir); slice_acc<kW[0]>(ai, ii); }
+            if (g % 4 == 1) { slice_acc<kW[1]>(ar, ir); slice_acc<kW[1]>(ai, ii); }
+            if (g % 4 == 2) { slice_acc<kW[2]>(ar, ir); slice_acc<kW[2]>(ai, ii); }
+            if (g % 4 == 3) { slice_acc<kW[3]>(ar, ir); slice_acc<kW[3]>(ai, ii); }
+          }
+        }
+      }
+    }
+    if (!okc) *vfail = 1;
+  }
+  __syncthreads();
+  // the last commit covers every MMA issued; copies of tiles that no MMA consumed land before exit
+  int ok = !*vfail;
+  const int lc = s_last_commit;
+  if (lc >= 0 && !tc::mbar_wait(&freeb[lc % NS], (uint32_t)(lc / NS) & 1u, kSlicePolls)) ok = 0;
+  if (lc != nst - 1) ok = 0;
+  if (tid == 0)
+    for (int b = 0; b < NS; ++b)
+      if (s_last_copy[b] > lc) tc::mbar_wait(&full[b], (uint32_t)(s_last_copy[b] / NS) & 1u, kSlicePolls);
+  ok = __syncthreads_and(ok);
+  if (warp >= 2 && ok) {
+    const int row = m0 + 32 * (warp & 3) + lane, c0 = n0 + ((warp - 2) >> 2) * HC;
+    if (row < M) {
+      const int sa = ea[(size_t)z * ea_ld + row];
+      const int* ebz = eb + (size_t)z * eb_ld;
+      if constexpr (MODE == 0) {
+        cplx<OUT>* o = out + ((size_t)z * M + row) * N;
+#pragma unroll
+        for (int j = 0; j < HC; ++j) {
+          const int n = c0 + j;
+          if (n >= N) continue;
+          const int sb = ebz[n];
+          cplx<OUT> v;
+          if (sa == kSliceBad || sb == kSliceBad) v = mk<OUT>(NAN, NAN);
+          else if constexpr (NSUM == 2)
+            v = mk<OUT>(slice_to_double(acc[0][0][j], acc[NSUM - 1][0][j], sa + sb),
+                        slice_to_double(acc[0][1][j], acc[NSUM - 1][1][j], sa + sb));
+          else
+            v = mk<OUT>(slice_to_double(0, acc[0][0][j], sa + sb), slice_to_double(0, acc[0][1][j], sa + sb));
+          o[n] = v;
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < HC; ++j) {
+          const int n = c0 + j;
+          if (n >= N) continue;
+          const int sb = ebz[n];
+          cplx<OUT>* y = out + (size_t)n * ldo + row;
+          cplx<OUT> v;
+          if (sa == kSliceBad || sb == kSliceBad) v = mk<OUT>(NAN, NAN);
+          else if constexpr (std::is_same<OUT, float>::value)
+            v = mk<OUT>(slice_to_float(acc[0][0][j], sa + sb), slice_to_float(acc[0][1][j], sa + sb));
+          else
+            v = mk<OUT>(slice_to_double(acc[0][0][j], acc[NSUM - 1][0][j], sa + sb),
+                        slice_to_double(acc[0][1][j], acc[NSUM - 1][1][j], sa + sb));
+          *y = accum ? cadd(*y, v) : v;
+        }
+      }
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc::tc_fence_after();
+    tc::tmem_dealloc(tmem_base, 512u);
+  }
+  if (!ok && tid == 0 && nst > 0) atomicExch(err, 1);
+}
+
+// C[m][n] = sum of the slices' partials; elements whose tile was skipped are the conjugate of their mirror
+__global__ void k_slice_reduce(int M, int N, int nz, const double2* __restrict__ part, double2* __restrict__ C,
+                               int ldc, int herm, int nc) {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= M * N) return;
+  const int m = idx / N, n = idx - m * N;
+  const bool mirror = herm && n / nc * nc + nc - 1 < m / kSliceM * kSliceM;
+  const size_t off = mirror ? (size_t)n * N + m : (size_t)m * N + n;
+  double2 s = make_double2(0.0, 0.0);
+  for (int z = 0; z < nz; ++z) s = cadd(s, part[(size_t)z * M * N + off]);
+  C[(size_t)m * ldc + n] = mirror ? cconj(s) : s;
+}
+
+// ------------------------------------------------------------------------------------------------
+// host side
+// ------------------------------------------------------------------------------------------------
+template <typename T> struct SliceL { static constexpr int value = sizeof(T) == 8 ? 7 : 4; };
+
+template <int L, int MODE, typename OUT>
+static int slice_launch(Ctx* c, dim3 grid, int M, int N, int nstage, int kstages, const unsigned char* a,
+                        const int* ea, int ea_ld, const unsigned char* b, const int* eb, int eb_ld, cplx<OUT>* out,
+                        int ldo, bool herm, bool lower, bool accum) {
+  int* err = tc_err_flag(c);
+  if (!err) return PARO_ERR_CUDA;
+  const size_t sm = (size_t)SliceCfg<L>::NS * (slice_a_bytes<L>() + slice_b_bytes<L>()) + 1024;
+  static int attr_dev = -1;
+  int dev = 0;
+  PARO_CU(c, cudaGetDevice(&dev));
+  if (attr_dev != dev) {
+    PARO_CU(c, cudaFuncSetAttribute(k_slice_gemm<L, MODE, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    attr_dev = dev;
+  }
+  k_slice_gemm<L, MODE, OUT><<<grid, kSliceThreads, sm, c->stream>>>(M, N, nstage, kstages, a, ea, ea_ld, b, eb, eb_ld,
+                                                                     out, ldo, herm, lower, accum, err);
+  PARO_LAUNCH(c, "k_slice_gemm");
+  return PARO_OK;
+}
+
+static int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+// K slices of the long-K product: the count that minimises waves of 152 CTAs times (stages + the stages' worth
+// of a CTA's start and conversion, about 8)
+static int slice_split_k(int tiles, int nstage) {
+  int best_nz = 1;
+  long long best = -1;
+  for (int nz = 1; nz <= std::max(1, nstage / 4); ++nz) {
+    const int ks = (nstage + nz - 1) / nz, z = (nstage + ks - 1) / ks;
+    const long long cost = ((long long)tiles * z + 151) / 152 * (ks + 8) * 64 + z;  // ties: fewer slices
+    if (best < 0 || cost < best) {
+      best = cost;
+      best_nz = z;
+    }
+  }
+  return best_nz;
+}
+
+// C = conj(A) B^T with A given as an image (scales ea[row], the same for every K slice) or as rows
+template <typename T>
+static int slice_cn(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, const unsigned char* a_img, const int* ea,
+                    const cplx<T>* B, int ldb, double2* C, int ldc, bool herm) {
+  constexpr int L = SliceL<T>::value, NC = SliceCfg<L>::NC;
+  const int mt = (M + kSliceM - 1) / kSliceM, nt = (N + NC - 1) / NC, nstage = (K + kSliceK - 1) / kSliceK;
+  int tiles = mt * nt;
+  if (herm)
+    for (int i = 0; i < mt; ++i) tiles -= std::min(nt, i * kSliceM / NC);
+  int nz = slice_split_k(tiles, nstage);
+  const int ks = (nstage + nz - 1) / nz;
+  nz = (nstage + ks - 1) / ks;
+  const int ma = mt * kSliceM, nb = nt * NC;
+  const bool same = !a_img && A == B && lda == ldb && M == N;
+  const int pad = same ? std::max(ma, nb) : nb;
+  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)nt * nstage * slice_b_bytes<L>()));
+  int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)nz * pad * sizeof(int)));
+  double2* part = static_cast<double2*>(ws_get(c, "gemm_parts", (size_t)nz * M * N * sizeof(double2)));
+  unsigned char* ai = nullptr;
+  int* ean = nullptr;
+  if (!a_img) {
+    ai = static_cast<unsigned char*>(ws_get(c, "slice_a", (size_t)mt * nstage * slice_a_bytes<L>()));
+    ean = same ? eb : static_cast<int*>(ws_get(c, "slice_ea", (size_t)nz * ma * sizeof(int)));
+    if (!ai || !ean) return PARO_ERR_CUDA;
+  }
+  if (!bi || !eb || !part) return PARO_ERR_CUDA;
+  cudaEvent_t ev = prof_begin(c);
+  if (!a_img && !same) {
+    k_slice_rows<T, L><<<dim3(ma / 8, nz), 256, 0, c->stream>>>(M, ma, 0, K, ks * kSliceK, nstage, A, lda, 0, ai,
+                                                                nullptr, ean, ma);
+    PARO_LAUNCH(c, "k_slice_rows");
+  }
+  k_slice_rows<T, L><<<dim3(pad / 8, nz), 256, 0, c->stream>>>(N, same ? ma : 0, nb, K, ks * kSliceK, nstage, B, ldb, 0,
+                                                               same ? ai : nullptr, bi, eb, pad);
+  PARO_LAUNCH(c, "k_slice_rows");
+  prof_end(c, sizeof(T) == 8 ? "k_slice_rows<f64>" : "k_slice_rows<f32>", ev);
+  ev = prof_begin(c);
+  int st = slice_launch<L, 0, double>(c, dim3(nt, mt, nz), M, N, nstage, ks, a_img ? a_img : ai, a_img ? ea : ean,
+                                      a_img ? 0 : (same ? pad : ma), bi, eb, pad, part, 0, herm, false, false);
+  if (st) return st;
+  prof_end(c, sizeof(T) == 8 ? "k_slice_gemm_cn<f64>" : "k_slice_gemm_cn<f32>", ev);
+  k_slice_reduce<<<(M * N + 255) / 256, 256, 0, c->stream>>>(M, N, nz, part, C, ldc, herm, NC);
+  PARO_LAUNCH(c, "k_slice_reduce");
+  return PARO_OK;
+}
+
+template <typename T>
+int gemm_cn_slice(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, const cplx<T>* B, int ldb, double2* C,
+                  int ldc, bool herm) {
+  return slice_cn<T>(c, M, N, K, A, lda, nullptr, nullptr, B, ldb, C, ldc, herm);
+}
+
+// Y (+)= sum_k s_k W(k, m) X[k][n] with X given as rows or as an image of its columns
+template <typename T>
+static int slice_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<T>* X,
+                    int ldx, const unsigned char* a_img, const int* ea, cplx<T>* Y, int ldy, bool accum, bool lower) {
+  constexpr int L = SliceL<T>::value, NC = SliceCfg<L>::NC;
+  const int at = (N + kSliceM - 1) / kSliceM, bt = (M + NC - 1) / NC, nstage = (K + kSliceK - 1) / kSliceK;
+  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)bt * nstage * slice_b_bytes<L>()));
+  int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)bt * NC * sizeof(int)));
+  if (!bi || !eb) return PARO_ERR_CUDA;
+  int* rowkey = nullptr;
+  cudaEvent_t ev = prof_begin(c);
+  if (!a_img) {
+    unsigned char* ai = static_cast<unsigned char*>(ws_get(c, "slice_a", (size_t)at * nstage * slice_a_bytes<L>()));
+    int* ean = static_cast<int*>(ws_get(c, "slice_ea", (size_t)at * kSliceM * sizeof(int)));
+    if (!ai || !ean) return PARO_ERR_CUDA;
+    rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)std::max(K, 1) * sizeof(int)));
+    if (!rowkey) return PARO_ERR_CUDA;
+    PARO_CU(c, cudaMemsetAsync(rowkey, 0, (size_t)K * sizeof(int), c->stream));
+    k_slice_rowkey<T><<<dim3(std::max(1, std::min((N + 1023) / 1024, 2048 / K)), K), 256, 0, c->stream>>>(N, X, ldx,
+                                                                                                     rowkey);
+    PARO_LAUNCH(c, "k_slice_rowkey");
+    k_slice_cols<T, L><<<at * kSliceM / 32, 256, 0, c->stream>>>(N, K, nstage, X, ldx, rowkey, ai, ean);
+    PARO_LAUNCH(c, "k_slice_cols");
+    a_img = ai;
+    ea = ean;
+  }
+  k_slice_w<L, T><<<bt * NC / 8, 256, 0, c->stream>>>(M, K, nstage, W, ldw, wt ? 1 : 0, s, rowkey, bi, eb);
+  PARO_LAUNCH(c, "k_slice_w");
+  prof_end(c, sizeof(T) == 8 ? "k_slice_cols<f64>" : "k_slice_cols<f32>", ev);
+  ev = prof_begin(c);
+  int st = slice_launch<L, 1, T>(c, dim3(bt, at), N, M, nstage, nstage, a_img, ea, 0, bi, eb, 0, Y, ldy, false, lower,
+                                 accum);
+  if (st) return st;
+  prof_end(c, sizeof(T) == 8 ? "k_slice_gemm_wx<f64>" : "k_slice_gemm_wx<f32>", ev);
+  return PARO_OK;
+}
+
+template <typename T>
+int gemm_wx_slice(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<T>* X,
+                  int ldx, cplx<T>* Y, int ldy, bool accum, bool lower) {
+  return slice_wx<T>(c, M, N, K, W, ldw, wt, s, X, ldx, nullptr, nullptr, Y, ldy, accum, lower);
+}
+
+// ---- the projectors as the fixed operand: their images change only with the atom positions ----
+template <typename T> static const cplx<T>* slice_beta(const Basis& b);
+template <> const double2* slice_beta<double>(const Basis& b) { return b.d_beta; }
+template <> const float2* slice_beta<float>(const Basis& b) { return b.d_beta32; }
+
+template <typename T>
+static int slice_beta_images(Ctx* c, int ik) {
+  constexpr int L = SliceL<T>::value, q = sizeof(T) == 8 ? 1 : 0;
+  Basis& B = c->bases[ik];
+  SliceImages& im = B.beta_slices[q];
+  if (im.cn) return PARO_OK;
+  const int np = c->nproj, npw = B.npw;
+  const int ma = round_up(np, kSliceM), na = round_up(npw, kSliceM);
+  const int scn = (npw + kSliceK - 1) / kSliceK, swx = (np + kSliceK - 1) / kSliceK;
+  const size_t bcn = (size_t)(ma / kSliceM) * scn * slice_a_bytes<L>();
+  const size_t bwx = (size_t)(na / kSliceM) * swx * slice_a_bytes<L>();
+  unsigned char* p = nullptr;  // [cn image | wx image | cn scales | wx scales]
+  PARO_CU(c, cudaMalloc(&p, bcn + bwx + (size_t)(ma + na) * sizeof(int)));
+  im.cn = p;
+  im.wx = p + bcn;
+  im.ecn = reinterpret_cast<int*>(p + bcn + bwx);
+  im.ewx = im.ecn + ma;
+  k_slice_rows<T, L><<<ma / 8, 256, 0, c->stream>>>(np, ma, 0, npw, scn * kSliceK, scn, slice_beta<T>(B), npw, 0, im.cn,
+                                                    nullptr, im.ecn, ma);
+  PARO_LAUNCH(c, "k_slice_rows");
+  k_slice_cols<T, L><<<na / 32, 256, 0, c->stream>>>(npw, np, swx, slice_beta<T>(B), npw, nullptr, im.wx,
+                                                        im.ewx);
+  PARO_LAUNCH(c, "k_slice_cols");
+  return PARO_OK;
+}
+
+template <typename T>
+int kb_project_slice(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P) {
+  int st = slice_beta_images<T>(c, ik);
+  if (st) return st;
+  const Basis& B = c->bases[ik];
+  const SliceImages& im = B.beta_slices[sizeof(T) == 8 ? 1 : 0];
+  return slice_cn<T>(c, c->nproj, nb, B.npw, nullptr, 0, im.cn, im.ecn, psi, B.npw, P, nb, false);
+}
+
+template <typename T>
+int kb_update_slice(Ctx* c, int ik, int nb, const double2* P, cplx<T>* hpsi) {
+  int st = slice_beta_images<T>(c, ik);
+  if (st) return st;
+  const Basis& B = c->bases[ik];
+  const SliceImages& im = B.beta_slices[sizeof(T) == 8 ? 1 : 0];
+  return slice_wx<T>(c, nb, B.npw, c->nproj, P, nb, false, c->d_dvec, nullptr, 0, im.wx, im.ewx, hpsi, B.npw, true,
+                     false);
+}
+
+template int gemm_cn_slice<double>(Ctx*, int, int, int, const double2*, int, const double2*, int, double2*, int, bool);
+template int gemm_wx_slice<double>(Ctx*, int, int, int, const double2*, int, bool, const double*, const double2*, int,
+                                   double2*, int, bool, bool);
+template int kb_project_slice<double>(Ctx*, int, int, const double2*, double2*);
+template int kb_project_slice<float>(Ctx*, int, int, const float2*, double2*);
+template int kb_update_slice<double>(Ctx*, int, int, const double2*, double2*);
+template int kb_update_slice<float>(Ctx*, int, int, const double2*, float2*);
+
+}  // namespace paro

@@ -12,6 +12,13 @@
 
 namespace paro {
 
+// Digit images of the projectors for the sliced products (k_slice.cu), one allocation at cn: rows along k for
+// the projections, columns for the update, and the scales of both.
+struct SliceImages {
+  unsigned char *cn = nullptr, *wx = nullptr;
+  int *ecn = nullptr, *ewx = nullptr;
+};
+
 // Plane-wave basis of one k-point (Eq. e3) with the z-column ("stick") structure the FFT passes use.
 struct Basis {
   int hx_recur = 0;  // ParO iterations of this k-point since H of its Rayleigh-Ritz basis was applied directly
@@ -43,6 +50,7 @@ struct Basis {
   float4* d_beta_img_cn = nullptr;
   float4* d_beta_img_wx = nullptr;
   int img_cn_nstage = 0, img_wx_nstage = 0;
+  SliceImages beta_slices[2];     // FP32, FP64; formed on first use, dropped when the projectors change
   double* d_prec_base = nullptr;  // |k+G|^2/2 (copy used by the preconditioner)
   // orbitals
   double2* d_psi = nullptr;       // n_bands x npw, orthonormal
@@ -150,6 +158,8 @@ struct Ctx {
   // FP32 products may run on the tensor cores (3xTF32): inside the inexact inner solves and the adjoint,
   // not in the Rayleigh-Ritz step, the rotations or the energy, which fix the self-consistent result
   bool tc_scope = false;
+  // the FP64 iteration's own arithmetic (PlainF64)
+  bool plain64 = false;
   struct CholShape {  // launch shape of the cluster Cholesky for order n on device dev
     int n = -1, dev = -1, kind = 0, cls = 0, thr = 0;
     size_t smem = 0;
@@ -197,6 +207,17 @@ struct TcScope {
   bool old;
   explicit TcScope(Ctx* ctx) : c(ctx), old(ctx->tc_scope) { ctx->tc_scope = true; }
   ~TcScope() { c->tc_scope = old; }
+};
+// FP64 contexts inside the ParO iteration: products and transforms on the FP64 pipe (k_gemm_cn, k_gemm_wx, the
+// register FFT), operation by operation as they always were. The signs of the orbitals come out of inverse
+// iteration, where the last bit of a Ritz value decides them, so any other rounding, however much smaller,
+// turns about half of the orbitals of a stored state around. Calls that do not decide orbitals (H psi, source
+// problems, orthonormalisation, adjoint, density, energy) take the digit slices.
+struct PlainF64 {
+  Ctx* c;
+  bool old;
+  explicit PlainF64(Ctx* ctx) : c(ctx), old(ctx->plain64) { ctx->plain64 = ctx->prec == PARO_FP64; }
+  ~PlainF64() { c->plain64 = old; }
 };
 // Scoped phase tag: names recorded inside become "tag:name".
 struct ProfTag {
@@ -255,6 +276,21 @@ int beta_images(Ctx* c, int ik);  // forms the two images of k-point ik if they 
 int gemm_cn_tc_beta(Ctx* c, int ik, int nb, const float2* x, double2* P, int* err);
 // y_b += sum_p beta_p D_p P[p][b] (y: nb rows, FP32, ld = N_pw)
 int gemm_wx_tc_beta(Ctx* c, int ik, int nb, const double2* P, const double* dvec, float2* y, int* err);
+// whether FP64 products take the digit slices
+inline bool slices_on(const Ctx* c) { return tc_enabled() && !c->plain64; }
+// ---- FP64-accurate products on the bf16 tensor cores by digit slices (k_slice.cu) ----
+// gemm_cn / gemm_wx (beta = 0, or 1 when accum) of FP64 operands
+template <typename T>
+int gemm_cn_slice(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, const cplx<T>* B, int ldb, double2* C,
+                  int ldc, bool herm);
+template <typename T>
+int gemm_wx_slice(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<T>* X,
+                  int ldx, cplx<T>* Y, int ldy, bool accum, bool lower);
+// P = beta^H psi (nproj x nb) and hpsi += beta (D o P) from the projectors' images
+template <typename T>
+int kb_project_slice(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P);
+template <typename T>
+int kb_update_slice(Ctx* c, int ik, int nb, const double2* P, cplx<T>* hpsi);
 // pieces of k_tc.cu the projector products share
 void tc_cn_plan(int M, int N, int K, int* nz_out, int* kslice_out);
 int reduce_parts32(Ctx* c, int M, int N, int nz, const float2* part, double2* C, int ldc);
@@ -310,6 +346,9 @@ int convert(Ctx* c, size_t n, const cplx<TS>* src, cplx<TD>* dst);
 // ---- KB projectors (k_hpsi.cu) ----
 template <typename T>
 int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi);
+// the projections P[p][b] = <beta_p | psi_b> alone (nproj x nb)
+template <typename T>
+int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P);
 
 // Suspends the real-wavefunction mode for the scope (calls on general complex vectors, packed rows).
 struct GammaPackOff {
