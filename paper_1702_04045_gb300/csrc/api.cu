@@ -254,6 +254,8 @@ static int setup_bases(Ctx* c) {
   for (int ax = 0; ax < 3; ++ax) {
     if (c->d_tw64[ax]) cudaFree(c->d_tw64[ax]);
     if (c->d_tw32[ax]) cudaFree(c->d_tw32[ax]);
+    if (c->d_twfx[ax]) cudaFree(c->d_twfx[ax]);
+    c->d_twfx[ax] = nullptr;
     c->d_tw64[ax] = nullptr;
     c->d_tw32[ax] = nullptr;
   }
@@ -1163,6 +1165,7 @@ void paro_destroy(paro_ctx* ctx) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   for (Basis& b : c->bases) free_basis(b);
   void* ps[] = {c->d_tw64[0], c->d_tw64[1], c->d_tw64[2], c->d_tw32[0], c->d_tw32[1], c->d_tw32[2],
+                c->d_twfx[0], c->d_twfx[1], c->d_twfx[2],
                 c->d_vloc, c->d_dvec, c->d_dvec32, c->d_veff, c->d_vplane, c->d_vplane32,
                 c->d_rho_in, c->d_pulay_rho, c->d_pulay_res, c->d_pulay_gram, c->d_tc_err, c->d_occ_sqrt};
   for (void* p : ps)

@@ -174,6 +174,20 @@ template <> const float* kin_of<float>(const Basis& b) { return b.d_kin32; }
 
 #include "hpsi_passes_reg.cuh"
 
+// the passes with lines in registers where a form covers the grid (*used): FP32 on 32, 36, 48, 72, 128 and the
+// plain FP64 iteration by hpsi_passes_reg.cuh, FP64 elsewhere by hpsi_passes_tile.cuh
+template <typename T>
+static int passes_fast(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, cplx<T>* hpsi, double shift,
+                       const int* active, bool* used, const T* vplane = nullptr, bool acc = false) {
+  *used = false;
+  if (sizeof(T) == 4 || c->plain64) {
+    const int st = passes_reg_dispatch<T>(c, B, nb, psi, S, hpsi, shift, active, used, vplane, acc);
+    if (st || *used || sizeof(T) == 8) return st;
+  }
+  if constexpr (sizeof(T) == 8) return passes_tile<T>(c, B, nb, psi, S, hpsi, shift, active, vplane, acc, used);
+  return PARO_OK;
+}
+
 template <typename T>
 int apply_h(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi, double shift, const int* active) {
   if (!c->have_veff) return fail(c, PARO_ERR_STATE, "no effective potential set");
@@ -186,7 +200,7 @@ int apply_h(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi, double sh
   cplx<T>* S = static_cast<cplx<T>*>(ws_get(c, sizeof(T) == 8 ? "sticks64" : "sticks32", sbytes));
   if (!S) return PARO_ERR_CUDA;
   bool used = false;
-  if ((st = passes_reg_dispatch<T>(c, B, nb, psi, S, hpsi, shift, active, &used))) return st;
+  if ((st = passes_fast<T>(c, B, nb, psi, S, hpsi, shift, active, &used))) return st;
   if (used) {
     if (!c->have_kb) return PARO_OK;
     cudaEvent_t ev = prof_begin(c);
@@ -238,7 +252,7 @@ int apply_dv(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi, const T*
   const size_t sbytes = (size_t)nb * c->N[2] * B.ncol * sizeof(cplx<T>);
   cplx<T>* S = static_cast<cplx<T>*>(ws_get(c, sizeof(T) == 8 ? "sticks64" : "sticks32", sbytes));
   if (!S) return PARO_ERR_CUDA;
-  return passes_reg_dispatch<T>(c, B, nb, psi, S, hpsi, 0.0, nullptr, used, dvplane, true);
+  return passes_fast<T>(c, B, nb, psi, S, hpsi, 0.0, nullptr, used, dvplane, true);
 }
 template int apply_dv<double>(Ctx*, int, int, const double2*, double2*, const double*, bool*);
 template int apply_dv<float>(Ctx*, int, int, const float2*, float2*, const float*, bool*);
@@ -248,8 +262,11 @@ int sticks_inverse(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* S) {
   int st = configure<T>(c);
   if (st) return st;
   bool used = false;
-  if ((st = sticks_inverse_reg<T>(c, ik, nb, psi, S, &used)) || used) return st;
   const Basis& B = c->bases[ik];
+  if ((sizeof(T) == 4 || c->plain64) && ((st = sticks_inverse_reg<T>(c, ik, nb, psi, S, &used)) || used)) return st;
+  if constexpr (sizeof(T) == 8) {
+    if (!c->plain64 && ((st = sticks_tile<T>(c, B, nb, psi, S, &used)) || used)) return st;
+  }
   const dim3 gz((B.ncol + kStickBatch - 1) / kStickBatch, nb);
   k_zpass_inv<T><<<gz, kZThreads, zpass_smem(c, sizeof(cplx<T>)), c->stream>>>(
       psi, B.npw, S, B.d_col_off, B.d_g_col, B.d_g_z, B.ncol, c->plan[2], tw_of<T>(c, 2), nullptr, kStickBatch);

@@ -4,6 +4,7 @@
 #include <cmath>
 #include <vector>
 
+#include "fft_tile.cuh"
 #include "paro_ctx.h"
 
 namespace paro {
@@ -15,13 +16,17 @@ __device__ __forceinline__ int signed_index(int j, int n) { return 2 * j < n ? j
 // ------------------------------------------------------------------------------------------------
 // twiddles exp(-2 pi i j / n)
 // ------------------------------------------------------------------------------------------------
-__global__ void k_twiddle(int n, double2* __restrict__ t64, float2* __restrict__ t32) {
+__global__ void k_twiddle(int n, double2* __restrict__ t64, float2* __restrict__ t32, fxw* __restrict__ tfx) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double s, c;
   sincospi(2.0 * (double)j / (double)n, &s, &c);
   t64[j] = make_double2(c, -s);
   t32[j] = make_float2((float)c, (float)-s);
+  if (tfx) {
+    const FxSplit r = fx_split((long long)(c * 4611686018427387904.0)), i = fx_split((long long)(-s * 4611686018427387904.0));
+    tfx[j] = fxw{r.h, r.l, i.h, i.l};
+  }
 }
 
 int build_twiddles(Ctx* c) {
@@ -29,7 +34,9 @@ int build_twiddles(Ctx* c) {
     const int n = c->N[ax];
     PARO_CU(c, cudaMalloc(&c->d_tw64[ax], n * sizeof(double2)));
     PARO_CU(c, cudaMalloc(&c->d_tw32[ax], n * sizeof(float2)));
-    k_twiddle<<<(n + 127) / 128, 128, 0, c->stream>>>(n, c->d_tw64[ax], c->d_tw32[ax]);
+    PARO_CU(c, cudaMalloc(&c->d_twfx[ax], n * sizeof(fxw)));
+    k_twiddle<<<(n + 127) / 128, 128, 0, c->stream>>>(n, c->d_tw64[ax], c->d_tw32[ax],
+                                                      static_cast<fxw*>(c->d_twfx[ax]));
     PARO_LAUNCH(c, "k_twiddle");
   }
   return PARO_OK;
@@ -644,7 +651,7 @@ static const double2* half_twiddles(Ctx* c) {
   float2* t32 = static_cast<float2*>(ws_get(c, "tw32_half", (size_t)M * sizeof(float2)));
   if (!t64 || !t32) return nullptr;
   if (!c->have_tw_half) {
-    k_twiddle<<<(M + 127) / 128, 128, 0, c->stream>>>(M, t64, t32);
+    k_twiddle<<<(M + 127) / 128, 128, 0, c->stream>>>(M, t64, t32, nullptr);
     if (cudaGetLastError() != cudaSuccess) return nullptr;
     c->have_tw_half = true;
   }
@@ -866,7 +873,13 @@ int density_bands(Ctx* c, int ik, int nbands, const cplx<T>* psi, double wfac, d
   if (st) return st;
   cudaEvent_t ev = prof_begin(c);
   bool used = false, f32part = false;
-  if ((st = density_planes_reg<T>(c, ik, S, nbands, ngrp, gsize, wfac, wsq, part, &used, &f32part))) return st;
+  if ((sizeof(T) == 4 || c->plain64) &&
+      (st = density_planes_reg<T>(c, ik, S, nbands, ngrp, gsize, wfac, wsq, part, &used, &f32part)))
+    return st;
+  f32part = f32part && used;
+  if constexpr (sizeof(T) == 8) {
+    if (!used && !c->plain64 && (st = density_tile<T>(c, B, S, nbands, ngrp, gsize, wfac, wsq, part, &used))) return st;
+  }
   if (!used) {
     if (smem > 227 * 1024) return fail(c, PARO_ERR_ARG, "density: plane too large for shared memory");
     PARO_CU(c, cudaFuncSetAttribute(k_plane_density<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
@@ -876,7 +889,7 @@ int density_bands(Ctx* c, int ik, int nbands, const cplx<T>* psi, double wfac, d
     PARO_LAUNCH(c, "k_plane_density");
   }
   prof_end(c, sizeof(T) == 8 ? "k_plane_density<f64>" : "k_plane_density<f32>", ev);
-  if (used && f32part)
+  if (f32part)
     k_density_reduce32<<<(c->ngrid + 255) / 256, 256, 0, c->stream>>>(N1, N2, N3, ngrp,
                                                                       reinterpret_cast<const float*>(part), wfac,
                                                                       rho_dev, accumulate);

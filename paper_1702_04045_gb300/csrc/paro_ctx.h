@@ -84,6 +84,7 @@ struct Ctx {
   FftPlan plan[3];
   double2* d_tw64[3] = {nullptr, nullptr, nullptr};
   float2* d_tw32[3] = {nullptr, nullptr, nullptr};
+  void* d_twfx[3] = {nullptr, nullptr, nullptr};  // the same in 62-bit fixed point (fxw, fft_tile.cuh)
   // pseudopotentials
   bool have_pp = false;
   double Z = 0, rc = 0, A = 0, a = 0;
@@ -212,7 +213,7 @@ struct TcScope {
 // register FFT), operation by operation as they always were. The signs of the orbitals come out of inverse
 // iteration, where the last bit of a Ritz value decides them, so any other rounding, however much smaller,
 // turns about half of the orbitals of a stored state around. Calls that do not decide orbitals (H psi, source
-// problems, orthonormalisation, adjoint, density, energy) take the digit slices.
+// problems, orthonormalisation, adjoint, density, energy) take the digit slices and the fixed-point FFT.
 struct PlainF64 {
   Ctx* c;
   bool old;
@@ -391,6 +392,21 @@ double ewald(const Ctx* c);
 int build_twiddles(Ctx* c);
 // radix plan (2, 3, 4, 8) of an FFT of length n (n = 2^a 3^b)
 FftPlan fft_plan(int n);
+// H psi passes, pass 1 alone and density planes with the line FFTs of fft_tile.cuh; *used = false on grids
+// they do not cover (k_tile_f64.cu)
+template <typename T>
+int passes_tile(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, cplx<T>* hpsi, double shift,
+                const int* active, const T* vplane, bool acc, bool* used);
+template <typename T>
+int sticks_tile(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, bool* used);
+template <typename T>
+int density_tile(Ctx* c, const Basis& B, const cplx<T>* S, int nbands, int ngrp, int gsize, double wfac,
+                 const double* wsq, double* part, bool* used);
+template <> int passes_tile<double>(Ctx*, const Basis&, int, const double2*, double2*, double2*, double, const int*,
+                                    const double*, bool, bool*);
+template <> int sticks_tile<double>(Ctx*, const Basis&, int, const double2*, double2*, bool*);
+template <> int density_tile<double>(Ctx*, const Basis&, const double2*, int, int, int, double, const double*, double*,
+                                     bool*);
 // pass 1 of H psi only (z-inverse FFT of the sticks), FP64, for the density
 template <typename T>
 int sticks_inverse(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* S);
