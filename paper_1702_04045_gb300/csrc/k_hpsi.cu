@@ -175,7 +175,8 @@ template <> const float* kin_of<float>(const Basis& b) { return b.d_kin32; }
 #include "hpsi_passes_reg.cuh"
 
 // the passes with lines in registers where a form covers the grid (*used): FP32 on 32, 36, 48, 72, 128 and the
-// plain FP64 iteration by hpsi_passes_reg.cuh, FP64 elsewhere by hpsi_passes_tile.cuh
+// plain FP64 iteration by hpsi_passes_reg.cuh, FP32 on the other grids up to 108 and FP64 elsewhere by
+// hpsi_passes_tile.cuh
 template <typename T>
 static int passes_fast(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, cplx<T>* hpsi, double shift,
                        const int* active, bool* used, const T* vplane = nullptr, bool acc = false) {
@@ -184,8 +185,7 @@ static int passes_fast(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<
     const int st = passes_reg_dispatch<T>(c, B, nb, psi, S, hpsi, shift, active, used, vplane, acc);
     if (st || *used || sizeof(T) == 8) return st;
   }
-  if constexpr (sizeof(T) == 8) return passes_tile<T>(c, B, nb, psi, S, hpsi, shift, active, vplane, acc, used);
-  return PARO_OK;
+  return passes_tile<T>(c, B, nb, psi, S, hpsi, shift, active, vplane, acc, used);
 }
 
 template <typename T>
@@ -264,9 +264,7 @@ int sticks_inverse(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* S) {
   bool used = false;
   const Basis& B = c->bases[ik];
   if ((sizeof(T) == 4 || c->plain64) && ((st = sticks_inverse_reg<T>(c, ik, nb, psi, S, &used)) || used)) return st;
-  if constexpr (sizeof(T) == 8) {
-    if (!c->plain64 && ((st = sticks_tile<T>(c, B, nb, psi, S, &used)) || used)) return st;
-  }
+  if (!(sizeof(T) == 8 && c->plain64) && ((st = sticks_tile<T>(c, B, nb, psi, S, &used)) || used)) return st;
   const dim3 gz((B.ncol + kStickBatch - 1) / kStickBatch, nb);
   k_zpass_inv<T><<<gz, kZThreads, zpass_smem(c, sizeof(cplx<T>)), c->stream>>>(
       psi, B.npw, S, B.d_col_off, B.d_g_col, B.d_g_z, B.ncol, c->plan[2], tw_of<T>(c, 2), nullptr, kStickBatch);

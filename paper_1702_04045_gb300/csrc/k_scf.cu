@@ -877,9 +877,9 @@ int density_bands(Ctx* c, int ik, int nbands, const cplx<T>* psi, double wfac, d
       (st = density_planes_reg<T>(c, ik, S, nbands, ngrp, gsize, wfac, wsq, part, &used, &f32part)))
     return st;
   f32part = f32part && used;
-  if constexpr (sizeof(T) == 8) {
-    if (!used && !c->plain64 && (st = density_tile<T>(c, B, S, nbands, ngrp, gsize, wfac, wsq, part, &used))) return st;
-  }
+  if (!used && !(sizeof(T) == 8 && c->plain64) &&
+      (st = density_tile<T>(c, B, S, nbands, ngrp, gsize, wfac, wsq, part, &used)))
+    return st;
   if (!used) {
     if (smem > 227 * 1024) return fail(c, PARO_ERR_ARG, "density: plane too large for shared memory");
     PARO_CU(c, cudaFuncSetAttribute(k_plane_density<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));

@@ -393,7 +393,7 @@ int build_twiddles(Ctx* c);
 // radix plan (2, 3, 4, 8) of an FFT of length n (n = 2^a 3^b)
 FftPlan fft_plan(int n);
 // H psi passes, pass 1 alone and density planes with the line FFTs of fft_tile.cuh; *used = false on grids
-// they do not cover (k_tile_f64.cu)
+// they do not cover (k_tile_f32.cu, k_tile_f64.cu)
 template <typename T>
 int passes_tile(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, cplx<T>* hpsi, double shift,
                 const int* active, const T* vplane, bool acc, bool* used);
@@ -402,9 +402,14 @@ int sticks_tile(Ctx* c, const Basis& B, int nb, const cplx<T>* psi, cplx<T>* S, 
 template <typename T>
 int density_tile(Ctx* c, const Basis& B, const cplx<T>* S, int nbands, int ngrp, int gsize, double wfac,
                  const double* wsq, double* part, bool* used);
+template <> int passes_tile<float>(Ctx*, const Basis&, int, const float2*, float2*, float2*, double, const int*,
+                                   const float*, bool, bool*);
 template <> int passes_tile<double>(Ctx*, const Basis&, int, const double2*, double2*, double2*, double, const int*,
                                     const double*, bool, bool*);
+template <> int sticks_tile<float>(Ctx*, const Basis&, int, const float2*, float2*, bool*);
 template <> int sticks_tile<double>(Ctx*, const Basis&, int, const double2*, double2*, bool*);
+template <> int density_tile<float>(Ctx*, const Basis&, const float2*, int, int, int, double, const double*, double*,
+                                    bool*);
 template <> int density_tile<double>(Ctx*, const Basis&, const double2*, int, int, int, double, const double*, double*,
                                      bool*);
 // pass 1 of H psi only (z-inverse FFT of the sticks), FP64, for the density
