@@ -40,6 +40,10 @@ static const int kMixMaxN = 160;  // largest n whose FP32 matrix fits one CTA's 
 // faster route)
 static const double kCouple = 1e-2;
 static const int kCoupleMaxCluster = 8;
+// longest cluster a warm start may leave: in the first hundred SCF iterations of the 64-atom cell the norm bound
+// joins most columns into one cluster, whose correction is then nil and whose Rayleigh-Ritz went to the FP64
+// solver (3.4 ms) or to long Jacobi sweeps (up to 0.9 ms); the FP32 solve takes about 1.1 ms
+static const int kWarmMaxCluster = 24;
 
 // ------------------------------------------------------------------------------------------------
 // Householder tridiagonalisation, one CTA, matrix (FP32) in shared memory. The same reflectors and outputs
@@ -271,7 +275,7 @@ __global__ void __launch_bounds__(1024) k_refine_lam(int n, const double2* __res
   __shared__ float red[32];
   __shared__ double s_lam[kMixMaxN];
   __shared__ int s_reach[kMixMaxN], s_cl[kMixMaxN], s_cst[kMixMaxN + 1];
-  __shared__ int s_wc[32], s_ncl, s_long;
+  __shared__ int s_wc[32], s_ncl, s_long, s_refuse;
   __shared__ double s_delta;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < n; i += blockDim.x) {
@@ -357,11 +361,16 @@ __global__ void __launch_bounds__(1024) k_refine_lam(int n, const double2* __res
     __syncthreads();
     if (!s_long) break;
   }
+  if (tid == 0) s_refuse = 0;
+  __syncthreads();
+  if (tid < s_ncl && s_cst[tid + 1] - s_cst[tid] > kWarmMaxCluster) s_refuse = 1;
+  __syncthreads();
   for (int i = tid; i < n; i += blockDim.x) cl[i] = s_cl[i];
   for (int i = tid; i <= s_ncl; i += blockDim.x) cst[i] = s_cst[i];
   if (tid == 0) {
     *ncl = s_ncl;
-    if (emax) *emax = 0.f;
+    // a warm start that would leave a long cluster to the FP64 Jacobi sweeps is refused by its correction
+    if (emax) *emax = s_refuse ? 1.f : 0.f;
   }
 }
 
