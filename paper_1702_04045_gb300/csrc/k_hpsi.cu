@@ -283,28 +283,22 @@ template <typename T> static const cplx<T>* beta_of(const Basis& b);
 template <> const double2* beta_of<double>(const Basis& b) { return b.d_beta; }
 template <> const float2* beta_of<float>(const Basis& b) { return b.d_beta32; }
 
-// P[p][b] = <beta_p | psi_b> (nproj x nb). FP64: digit slices on the tensor cores (k_slice.cu). FP32 outside
-// the inexact inner solves: sums carried in a two-sum pair, because a long FP32 accumulation biases
-// |<beta|psi>|^2 (and with it the Rayleigh-Ritz H and the energy) at the 1e-6 level.
-template <typename T>
-int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P) {
-  const Basis& B = c->bases[ik];
-  if constexpr (sizeof(T) == 8) {
-    if (slices_on(c)) return kb_project_slice<double>(c, ik, nb, psi, P);
-  }
-  const bool carry = sizeof(T) == 4 && !c->tc_scope;
-  return gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, carry);
+// FP32 products of nproj x nb x npw multiply-adds from which the digit slices are faster than the CUDA cores
+// (launch latency of their five kernels against three): V_nl on 256 projectors and 23847 plane waves takes
+// 172 us instead of 195 for 64 rows and 221 instead of 409 for 144, 147 instead of 160 for 32; on 32 projectors and
+// 2721 plane waves they lose up to 288 rows (85 us against 49).
+static const double kSlice32Work = 1.5e8;
+static bool kb_slices(const Ctx* c, int ik, int nb, bool f64) {
+  return slices_on(c) && (f64 || (double)c->nproj * nb * c->bases[ik].npw >= kSlice32Work);
 }
-template int kb_project<double>(Ctx*, int, int, const double2*, double2*);
-template int kb_project<float>(Ctx*, int, int, const float2*, double2*);
 
-// H psi += beta (D o (beta^H psi))
+// P[p][b] = <beta_p | psi_b> (nproj x nb). FP64, and FP32 of some size outside the inexact inner solves: digit
+// slices on the tensor cores (k_slice.cu). FP32 inside the inner solves and the adjoint: 3xTF32 on the tensor
+// cores from the projectors' presplit image. Else FP32 sums carried in a two-sum pair, because a long FP32
+// accumulation biases |<beta|psi>|^2 (and with it the Rayleigh-Ritz H and the energy) at the 1e-6 level.
 template <typename T>
-int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
+int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P, int plan_nb) {
   const Basis& B = c->bases[ik];
-  double2* P = static_cast<double2*>(ws_get(c, "kb_proj", (size_t)c->nproj * nb * sizeof(double2)));
-  if (!P) return PARO_ERR_CUDA;
-  // inside the inexact inner solves: the tensor-core products fed by the projectors' presplit images
   if constexpr (sizeof(T) == 4) {
     if (c->tc_scope && tc_enabled()) {
       int* err = tc_err_flag(c);
@@ -312,19 +306,38 @@ int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
       int st = beta_images(c, ik);
       if (st) return st;
       cudaEvent_t ev = prof_begin(c);
-      if ((st = gemm_cn_tc_beta(c, ik, nb, reinterpret_cast<const float2*>(psi), P, err))) return st;
+      if ((st = gemm_cn_tc_beta(c, ik, nb, reinterpret_cast<const float2*>(psi), P, err, plan_nb))) return st;
       prof_end(c, "k_gemm_cn_tcb", ev);
-      ev = prof_begin(c);
+      return PARO_OK;
+    }
+  }
+  if (kb_slices(c, ik, nb, sizeof(T) == 8)) return kb_project_slice<T>(c, ik, nb, psi, P);
+  const bool carry = sizeof(T) == 4 && !c->tc_scope;
+  return gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, carry);
+}
+template int kb_project<double>(Ctx*, int, int, const double2*, double2*, int);
+template int kb_project<float>(Ctx*, int, int, const float2*, double2*, int);
+
+// H psi += beta (D o (beta^H psi))
+template <typename T>
+int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
+  const Basis& B = c->bases[ik];
+  double2* P = static_cast<double2*>(ws_get(c, "kb_proj", (size_t)c->nproj * nb * sizeof(double2)));
+  if (!P) return PARO_ERR_CUDA;
+  int st = kb_project<T>(c, ik, nb, psi, P);
+  if (st) return st;
+  // inside the inexact inner solves: the tensor-core product fed by the projectors' presplit image
+  if constexpr (sizeof(T) == 4) {
+    if (c->tc_scope && tc_enabled()) {
+      int* err = tc_err_flag(c);
+      if (!err) return PARO_ERR_CUDA;
+      cudaEvent_t ev = prof_begin(c);
       if ((st = gemm_wx_tc_beta(c, ik, nb, P, c->d_dvec, reinterpret_cast<float2*>(hpsi), err))) return st;
       prof_end(c, "k_gemm_wx_tcb", ev);
       return PARO_OK;
     }
   }
-  int st = kb_project<T>(c, ik, nb, psi, P);
-  if (st) return st;
-  if constexpr (sizeof(T) == 8) {
-    if (slices_on(c)) return kb_update_slice<double>(c, ik, nb, P, hpsi);
-  }
+  if (kb_slices(c, ik, nb, sizeof(T) == 8)) return kb_update_slice<T>(c, ik, nb, P, hpsi);
   // W(k = p, m = b) = D_p P[p][b]
   return gemm_wx<T, T>(c, nb, B.npw, c->nproj, P, nb, false, c->d_dvec, beta_of<T>(B), B.npw, hpsi, B.npw, 1.0);
 }

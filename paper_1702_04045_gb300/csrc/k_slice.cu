@@ -3,17 +3,17 @@
 // 2012; the tensor-core form of Mukunoki, Ozaki, Ogita, Imamura, ISC 2020): the FP64 pipe of this chip does
 // 1.25 TFLOP/s, its bf16 tensor cores about 2 PFLOP/s.
 //
-// Every operand row is brought to a common exponent (|x| < 2^e), rounded to an integer of 8 L - 1 bits and
-// sign and written in L balanced base-256 digits, d_i in [-128, 128], which bf16 holds exactly:
-//   x = 2^(e + 1) sum_i d_i 256^-i.
+// Every operand row is brought to a common exponent (|x| < 2^e), rounded to an integer of 8 L - 2 bits and
+// sign and written in L balanced base-256 digits, d_i in [-128, 127], which bf16 holds exactly:
+//   x = 2^(e + 2) sum_i d_i 256^-i.
 // A product of rows is sum over (i, j) of 256^-(i+j) (d_i . d'_j). The digit products are integers of at most
 // 2^14, and a chunk of K values is short enough that the sums of all (i, j) with one i + j = g stay below
 // 2^24, so the tensor core's FP32 accumulation of each group g is exact. After every chunk the groups are
 // read from tensor memory and added into 64-bit integers at their weights; floating point appears only in
 // the final conversion. Groups up to g = PMAX are kept:
-//   L = 7, PMAX = 9 (34 digit products): operands rounded to 2^-56 of the row's largest power of two, groups
-//     dropped below 2^-57: FP64 results, more accurate than FP64 sums of the same length;
-//   L = 4, PMAX = 5 (10 products): operands rounded to 2^-32, for FP32 operands outside the inner solves.
+//   L = 7, PMAX = 9 (34 digit products): operands rounded to 2^-55 of the row's largest power of two, groups
+//     dropped below that: FP64 results, more accurate than FP64 sums of the same length;
+//   L = 4, PMAX = 5 (10 products): operands rounded to 2^-31, for FP32 operands outside the inner solves.
 //
 // Measured on the 64-atom cell (N_pw = 23847): V_nl of 144 FP64 orbitals 17.7 -> 0.68 ms, Cholesky
 // orthonormalisation of 288 rows 31.8 -> 3.1 ms (2.1 ms of it the factorisation); the error against extended
@@ -37,14 +37,16 @@ static const int kSliceK = 16;            // complex K values per stage (one MMA
 static const int kSliceThreads = 320;     // producer warp, MMA warp, eight epilogue warps
 static const uint32_t kSlicePolls = 1u << 24;
 
-// NC: columns of an output tile (2 NC accumulator columns per group fill the 512 of tensor memory);
-// CH: stages per exact chunk: 2 (planes) * 16 CH * 2^14 * (most pairs in a group) < 2^24; NS: stage buffers
+// NC: columns of an output tile (2 NC accumulator columns per group, at most 512 in tensor memory): 32 for
+// L = 7, 64 or 48 for L = 4, whichever pads less;
+// CH: stages per exact chunk: 2 (planes) * 16 CH * 2^14 * (most pairs in a group) <= 2^24; NS: stage buffers
 template <int L> struct SliceCfg;
-template <> struct SliceCfg<7> { static constexpr int NC = 32, PMAX = 9, CH = 4, NS = 2; };
-template <> struct SliceCfg<4> { static constexpr int NC = 64, PMAX = 5, CH = 8, NS = 3; };
+template <> struct SliceCfg<7> { static constexpr int PMAX = 9, CH = 4, NS = 2; };
+template <> struct SliceCfg<4> { static constexpr int PMAX = 5, CH = 8, NS = 3; };
 
 template <int L> __host__ __device__ constexpr int slice_a_bytes() { return L * 2 * kSliceM * kSliceK * 2; }
-template <int L> __host__ __device__ constexpr int slice_b_bytes() { return L * 3 * SliceCfg<L>::NC * kSliceK * 2; }
+template <int L> __host__ __device__ constexpr int slice_b_bytes(int nc) { return L * 3 * nc * kSliceK * 2; }
+template <int L> static int slice_nc(int n) { return L == 7 ? 32 : (n + 47) / 48 * 48 < (n + 63) / 64 * 64 ? 48 : 64; }
 
 // ------------------------------------------------------------------------------------------------
 // digits
@@ -59,49 +61,60 @@ template <typename T> __device__ __forceinline__ int slice_exponent(int key, boo
   *bad = ex == (sizeof(T) == 8 ? 0x7ff : 0xff);
   return max(ex, 1) - (sizeof(T) == 8 ? 1022 : 126);
 }
-// round(x 2^(8 L - 1 - e)), halves away from zero
-template <int L> __device__ __forceinline__ long long slice_fixed(double x, int e) {
+// the integer of a value: round(x 2^(8 L - 2 - e)), halves away from zero; 30 bits fit 32-bit arithmetic
+template <int L> struct SliceInt { using t = long long; };
+template <> struct SliceInt<4> { using t = int; };
+template <int L> __device__ __forceinline__ typename SliceInt<L>::t slice_fixed(double x, int e) {
   const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
   unsigned long long u = ((unsigned long long)(hi & 0xfffff) << 32) | (unsigned)__double2loint(x);
   if (ex) u |= 1ull << 52;
-  const int s = max(ex, 1) - 1075 + 8 * L - 1 - e;
+  const int s = max(ex, 1) - 1075 + 8 * L - 2 - e;
   if (s >= 0) u <<= min(s, 63);
   else u = s < -55 ? 0ull : (u + (1ull << (-s - 1))) >> -s;
-  return hi < 0 ? -(long long)u : (long long)u;
+  const typename SliceInt<L>::t f = (typename SliceInt<L>::t)u;
+  return hi < 0 ? -f : f;
 }
-template <int L> __device__ __forceinline__ long long slice_fixed(float x, int e) {
+template <int L> __device__ __forceinline__ typename SliceInt<L>::t slice_fixed(float x, int e) {
   const int b = __float_as_int(x), ex = (b >> 23) & 0xff;
-  unsigned long long u = (unsigned)(b & 0x7fffff);
+  unsigned u = (unsigned)(b & 0x7fffff);
   if (ex) u |= 1u << 23;
-  const int s = max(ex, 1) - 150 + 8 * L - 1 - e;
-  if (s >= 0) u <<= min(s, 63);
-  else u = s < -26 ? 0ull : (u + (1ull << (-s - 1))) >> -s;
-  return b < 0 ? -(long long)u : (long long)u;
+  const int s = max(ex, 1) - 150 + 8 * L - 2 - e;
+  if (s >= 0) u <<= min(s, 31);
+  else u = s < -25 ? 0u : (u + (1u << (-s - 1))) >> -s;
+  return b < 0 ? -(int)u : (int)u;
 }
-// balanced digits of F, most significant first, as bf16 bits in the upper half of d[i]
-template <int L> __device__ __forceinline__ void slice_digits(long long F, uint32_t d[L]) {
-  long long carry = 0;
+// balanced digits of F, most significant first, as bf16 bits in the upper half of d[i]: with 128 added to
+// every low byte the bytes hold the digits + 128 (the top one as a signed byte), and a byte b under the
+// exponent of 2^23 is the float 2^23 + b
+__device__ __forceinline__ uint32_t slice_digit(uint32_t word, int byte) {
+  return __float_as_uint(__uint_as_float(__byte_perm(word, 0x4B000000u, 0x7540 | byte)) - 8388736.0f);
+}
+template <int L> __device__ __forceinline__ void slice_digits(typename SliceInt<L>::t F, uint32_t d[L]) {
+  if constexpr (L == 4) {
+    const uint32_t t = ((uint32_t)F + 0x00808080u) ^ 0x80000000u;
 #pragma unroll
-  for (int i = 0; i < L - 1; ++i) carry |= 128ll << (8 * i);
-  const long long t = F + carry;  // each low byte now holds its digit + 128
+    for (int i = 0; i < 4; ++i) d[i] = slice_digit(t, 3 - i);
+  } else {
+    static_assert(L == 7, "digit layouts");
+    const long long t = F + 0x0000808080808080ll;
+    const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32) ^ 0x00800000u;
 #pragma unroll
-  for (int i = 0; i < L; ++i) {
-    const int sh = 8 * (L - 1 - i);
-    const uint32_t v = i == 0 ? (uint32_t)(t >> sh) + 128u : (uint32_t)(t >> sh) & 255u;
-    d[i] = __float_as_uint(__uint_as_float(0x4B000000u | v) - 8388736.0f);  // v - 128, exact
+    for (int i = 0; i < 3; ++i) d[i] = slice_digit(hi, 2 - i);
+#pragma unroll
+    for (int i = 3; i < 7; ++i) d[i] = slice_digit(lo, 6 - i);
   }
 }
 __device__ __forceinline__ uint32_t slice_pack(uint32_t d0, uint32_t d1) { return __byte_perm(d0, d1, 0x7632); }
 
-// result scale of a row: 2^(e + 1 - 4 PMAX) (a result is the integer sum times the scales of its two rows)
-template <int L> __device__ __forceinline__ int slice_scale(int e) { return e + 1 - 4 * SliceCfg<L>::PMAX; }
+// result scale of a row: 2^(e + 2 - 4 PMAX) (a result is the integer sum times the scales of its two rows)
+template <int L> __device__ __forceinline__ int slice_scale(int e) { return e + 2 - 4 * SliceCfg<L>::PMAX; }
 static const int kSliceBad = 1 << 20;  // scale of a row with Inf or NaN: its results are NaN
 
 // eight consecutive k of one row (|v_j| < 2^e_j) -> its 16-byte core-matrix rows of every slice and plane
 template <int L, typename T>
 __device__ __forceinline__ void slice_store(const cplx<T>* v, const int* e, bool conj_a, unsigned char* a_dst,
-                                            unsigned char* b_dst) {
-  constexpr int NCB = SliceCfg<L>::NC * kSliceK * 2;
+                                            unsigned char* b_dst, int nc) {
+  const int NCB = nc * kSliceK * 2;
   uint32_t wr[L][4], wi[L][4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -142,64 +155,86 @@ __device__ __forceinline__ unsigned char* slice_a_at(unsigned char* img, int nst
   return img + ((size_t)(row / kSliceM) * nstage + (k8 >> 1)) * slice_a_bytes<L>() + slice_core(row % kSliceM, k8 & 1);
 }
 template <int L>
-__device__ __forceinline__ unsigned char* slice_b_at(unsigned char* img, int nstage, int row, int k8) {
-  constexpr int NC = SliceCfg<L>::NC;
-  return img + ((size_t)(row / NC) * nstage + (k8 >> 1)) * slice_b_bytes<L>() + slice_core(row % NC, k8 & 1);
+__device__ __forceinline__ unsigned char* slice_b_at(unsigned char* img, int nstage, int nc, int row, int k8) {
+  return img + ((size_t)(row / nc) * nstage + (k8 >> 1)) * slice_b_bytes<L>(nc) + slice_core(row % nc, k8 & 1);
 }
 
-// Rows along contiguous k (orbitals, projectors): 8 rows x one K slice per CTA. Exponents are those of the
-// slice (es[z][row], ld rows_pad). a_img, b_img: either may be null.
-template <typename T, int L>
-__global__ void __launch_bounds__(256) k_slice_rows(int rows, int rows_a, int rows_b, int K, int kslice, int nstage,
-                                                    const cplx<T>* __restrict__ x, int ld, int conj_a,
-                                                    unsigned char* __restrict__ a_img,
-                                                    unsigned char* __restrict__ b_img, int* __restrict__ es,
-                                                    int rows_pad) {
-  __shared__ int skey[8];
-  const int r = threadIdx.x & 7, row = blockIdx.x * 8 + r, z = blockIdx.y;
-  const int k0 = z * kslice, k1 = min(nstage * kSliceK, k0 + kslice);  // padded K: zeros past K
-  if (threadIdx.x < 8) skey[threadIdx.x] = 0;
-  __syncthreads();
-  const cplx<T>* xr = x + (size_t)min(row, rows - 1) * ld;
-  int key = 0;
-  if (row < rows)
-    for (int k = k0 + (threadIdx.x >> 3); k < min(k1, K); k += 32) {
-      const cplx<T> v = xr[k];
-      key = max(key, max(slice_key(v.x), slice_key(v.y)));
-    }
-  atomicMax(&skey[r], key);
-  __syncthreads();
-  bool bad;
-  const int e = slice_exponent<T>(skey[r], &bad);
-  if (threadIdx.x < 8) es[(size_t)z * rows_pad + row] = bad ? kSliceBad : slice_scale<L>(e);
-  for (int k8 = k0 / 8 + (threadIdx.x >> 3); k8 < k1 / 8; k8 += 32) {
-    cplx<T> v[8];
-    int ev[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      v[j] = row < rows && 8 * k8 + j < K ? xr[8 * k8 + j] : mk<T>(0, 0);
-      ev[j] = e;
-    }
-    slice_store<L, T>(v, ev, conj_a != 0, a_img && row < rows_a ? slice_a_at<L>(a_img, nstage, row, k8) : nullptr,
-                      b_img && row < rows_b ? slice_b_at<L>(b_img, nstage, row, k8) : nullptr);
-  }
-}
-
-// Largest finite key of every row of X[k][n] (rowkey cleared by the caller).
+// Largest key of every row (rowkey cleared by the caller); finite: of its finite values only.
 template <typename T>
 __global__ void __launch_bounds__(256) k_slice_rowkey(int N, const cplx<T>* __restrict__ x, int ld,
-                                                      int* __restrict__ rowkey) {
+                                                      int finite, int* __restrict__ rowkey) {
   const cplx<T>* xr = x + (size_t)blockIdx.y * ld;
   int key = 0;
   for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
     const cplx<T> v = xr[n];
     const int a = slice_key(v.x), b = slice_key(v.y);
-    if (slice_key_exp<T>(a) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, a);
-    if (slice_key_exp<T>(b) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, b);
+    if (!finite || slice_key_exp<T>(a) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, a);
+    if (!finite || slice_key_exp<T>(b) != (sizeof(T) == 8 ? 0x7ff : 0xff)) key = max(key, b);
   }
   key = __reduce_max_sync(0xffffffffu, key);
   if ((threadIdx.x & 31) == 0) atomicMax(&rowkey[blockIdx.y], key);
 }
+// Rows along contiguous k (orbitals, projectors): 8 rows x one K slice per CTA. Exponents are those of the
+// slice (es[z][row], ld rows_pad), or with rowkey those of the whole rows (es[row]). a_img, b_img: either may be null. The slice is staged in shared memory,
+// read coalesced (a thread's own eight values are 64 or 128 bytes apart from its neighbour's) and once when it
+// fits the stage's 32 KB, else in pieces after a first pass for the exponents.
+template <typename T> struct SliceStage { static constexpr int value = sizeof(T) == 8 ? 256 : 512; };
+template <typename T, int L>
+__global__ void __launch_bounds__(256) k_slice_rows(int rows, int rows_a, int rows_b, int K, int kslice, int nstage,
+                                                    const cplx<T>* __restrict__ x, int ld, int conj_a,
+                                                    unsigned char* __restrict__ a_img,
+                                                    unsigned char* __restrict__ b_img, int* __restrict__ es,
+                                                    int rows_pad, int stage, const int* __restrict__ rowkey, int nc) {
+  extern __shared__ __align__(16) unsigned char smem_dyn[];
+  cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_dyn);  // 8 x (stage + 1): columns of eight rows meet no bank twice
+  __shared__ int skey[8];
+  const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int k0 = z * kslice, k1 = min(nstage * kSliceK, k0 + kslice);  // padded K: zeros past K
+  const int lds = stage + 1;
+  const bool once = k1 - k0 <= stage;
+  if (once || !rowkey) {  // warp w: row w
+    const int row = blockIdx.x * 8 + warp;
+    const cplx<T>* xr = x + (size_t)min(row, rows - 1) * ld;
+    int key = 0;
+    for (int k = k0 + lane; k < k1; k += 32) {
+      const cplx<T> v = row < rows && k < K ? xr[k] : mk<T>(0, 0);
+      key = max(key, max(slice_key(v.x), slice_key(v.y)));
+      if (once) buf[warp * lds + k - k0] = v;
+    }
+    key = __reduce_max_sync(0xffffffffu, key);
+    if (rowkey) key = row < rows ? rowkey[row] : 0;
+    if (lane == 0) skey[warp] = key;
+  } else if (lane == 0) {
+    const int row = blockIdx.x * 8 + warp;
+    skey[warp] = row < rows ? rowkey[row] : 0;
+  }
+  __syncthreads();
+  const int r = threadIdx.x & 7, row = blockIdx.x * 8 + r;
+  bool bad;
+  const int e = slice_exponent<T>(skey[r], &bad);
+  if (threadIdx.x < 8 && (!rowkey || z == 0)) es[(size_t)z * rows_pad + row] = bad ? kSliceBad : slice_scale<L>(e);
+  int ev[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) ev[j] = e;
+  for (int p0 = k0; p0 < k1; p0 += stage) {
+    const int p1 = min(k1, p0 + stage);
+    if (!once) {
+      __syncthreads();
+      const int rw = blockIdx.x * 8 + warp;
+      const cplx<T>* xr = x + (size_t)min(rw, rows - 1) * ld;
+      for (int k = p0 + lane; k < p1; k += 32) buf[warp * lds + k - p0] = rw < rows && k < K ? xr[k] : mk<T>(0, 0);
+      __syncthreads();
+    }
+    for (int k8 = p0 / 8 + (threadIdx.x >> 3); k8 < p1 / 8; k8 += 32) {
+      cplx<T> v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = buf[r * lds + 8 * k8 - p0 + j];
+      slice_store<L, T>(v, ev, conj_a != 0, a_img && row < rows_a ? slice_a_at<L>(a_img, nstage, row, k8) : nullptr,
+                        b_img && row < rows_b ? slice_b_at<L>(b_img, nstage, nc, row, k8) : nullptr, nc);
+    }
+  }
+}
+
 // An update sums over the rows of X, whose sizes may differ widely (orbitals beside small corrections): the
 // digits are taken of X[k][n] 2^-c_k and W(k, m) 2^c_k with c_k the exponent of row k, so that every row
 // keeps its own accuracy. c_k = 0 without row keys (the projectors, all of one size).
@@ -244,7 +279,7 @@ __global__ void __launch_bounds__(256) k_slice_cols(int N, int K, int nstage, co
       v[j] = n < N && k < K ? x[(size_t)k * ld + n] : mk<T>(0, 0);
       ev[j] = e + (k < K ? slice_rowshift<T>(rowkey, k) : 0);
     }
-    slice_store<L, T>(v, ev, true, slice_a_at<L>(a_img, nstage, n, k8), nullptr);
+    slice_store<L, T>(v, ev, true, slice_a_at<L>(a_img, nstage, n, k8), nullptr, 0);
   }
 }
 
@@ -254,7 +289,7 @@ template <int L, typename TX>
 __global__ void __launch_bounds__(256) k_slice_w(int M, int K, int nstage, const double2* __restrict__ W, int ldw,
                                                  int wt, const double* __restrict__ s,
                                                  const int* __restrict__ rowkey, unsigned char* __restrict__ b_img,
-                                                 int* __restrict__ es) {
+                                                 int* __restrict__ es, int nc) {
   __shared__ int stop[8];
   const int r = threadIdx.x & 7, m = blockIdx.x * 8 + r;
   if (threadIdx.x < 8) stop[threadIdx.x] = -kSliceNonfinite;
@@ -280,7 +315,7 @@ __global__ void __launch_bounds__(256) k_slice_w(int M, int K, int nstage, const
       v[j] = at(k);
       ev[j] = e - (k < K ? slice_rowshift<TX>(rowkey, k) : 0);
     }
-    slice_store<L, double>(v, ev, false, nullptr, slice_b_at<L>(b_img, nstage, m, k8));
+    slice_store<L, double>(v, ev, false, nullptr, slice_b_at<L>(b_img, nstage, nc, m, k8), nc);
   }
 }
 
@@ -381,6 +416,12 @@ __device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* r) {
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld_x8_async(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 }  // namespace tc
 
@@ -390,33 +431,59 @@ template <int W> __device__ __forceinline__ void slice_acc(long long& acc, int v
 }
 
 // MODE 0: part[z][m][n] = C over K slice z (complex double; M x N), herm: tiles wholly left of the diagonal
-// are skipped. MODE 1: Y[n][m] (+)= C[m][n] (the update: A rows are the long axis of Y), OUT = double or float;
+// are left out. MODE 1: Y[n][m] (+)= C[m][n] (the update: A rows are the long axis of Y), OUT = double or float;
 // lower: B is lower triangular and the stages past a tile's last row are left out.
-template <int L, int MODE, typename OUT>
+// Persistent: a CTA takes the tiles blockIdx.x, + gridDim.x, .. (column tiles fastest, so that CTAs in flight
+// share the long operand's tile in L2). The roles run ahead of each other across tiles: while the eight
+// epilogue warps convert and store a tile from their registers, the next tile's operands and MMAs are under way.
+struct SliceTiles {
+  int nt, mt, nz;        // column tiles, row tiles, K slices
+  int nstage, kstages;   // stages in all, stages per K slice
+  int herm, lower;
+  int per_z;             // tiles of one K slice (Hermitian: those not wholly left of the diagonal)
+};
+template <int NC> struct SliceTile {
+  int nt, mt, z, st0, nst;
+  __device__ __forceinline__ SliceTile(const SliceTiles& g, int t) {
+    z = t / g.per_z;
+    int r = t - z * g.per_z;
+    if (g.herm) {  // row tile mt starts at the column tile of its first row
+      for (mt = 0;; ++mt) {
+        const int n0 = mt * kSliceM / NC;
+        if (r < g.nt - n0) {
+          nt = n0 + r;
+          break;
+        }
+        r -= g.nt - n0;
+      }
+    } else {
+      mt = r / g.nt;
+      nt = r - mt * g.nt;
+    }
+    st0 = z * g.kstages;
+    nst = max(0, min(g.kstages, g.nstage - st0));
+    if (g.lower) nst = min(nst, (nt * NC + NC + kSliceK - 1) / kSliceK);  // b_n,k = 0 for k > n
+  }
+};
+
+template <int L, int NC, int MODE, typename OUT>
 __global__ void __launch_bounds__(kSliceThreads, 1)
-    k_slice_gemm(int M, int N, int nstage_all, int kstages, const unsigned char* __restrict__ a_img,
-                 const int* __restrict__ ea, int ea_ld, const unsigned char* __restrict__ b_img,
-                 const int* __restrict__ eb, int eb_ld, cplx<OUT>* __restrict__ out, int ldo, int herm, int lower,
-                 int accum, int* __restrict__ err) {
+    k_slice_gemm(int M, int N, SliceTiles geo, const unsigned char* __restrict__ a_img, const int* __restrict__ ea,
+                 int ea_ld, const unsigned char* __restrict__ b_img, const int* __restrict__ eb, int eb_ld,
+                 cplx<OUT>* __restrict__ out, int ldo, int accum, int* __restrict__ err) {
   using Cfg = SliceCfg<L>;
-  constexpr int NC = Cfg::NC, PMAX = Cfg::PMAX, CH = Cfg::CH, NS = Cfg::NS, NG = PMAX - 1;
-  constexpr int AB = slice_a_bytes<L>(), BB = slice_b_bytes<L>(), BUF = AB + BB;
+  constexpr int PMAX = Cfg::PMAX, CH = Cfg::CH, NS = Cfg::NS, NG = PMAX - 1;
+  constexpr int AB = slice_a_bytes<L>(), BB = slice_b_bytes<L>(NC), BUF = AB + BB;
   constexpr int HC = NC / 2;                 // columns per epilogue thread
   constexpr int NSUM = NG > 4 ? 2 : 1;       // 64-bit sums per value (four groups each)
-  static_assert(2 * NC * NG <= 512 && HC % 16 == 0, "tensor memory columns");
+  static_assert(2 * NC * NG <= 512 && HC % 8 == 0, "tensor memory columns");
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   unsigned char* smem = tc_align1024(smem_dyn);
   __shared__ uint64_t full[NS], freeb[NS], gfull[NG], gfree[NG];
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail, s_last_commit, s_last_copy[NS];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  // MODE 1: column tiles fastest, so CTAs in flight share the long operand's tile in L2
-  const int nt = blockIdx.x, mt = blockIdx.y, z = blockIdx.z;
-  const int m0 = mt * kSliceM, n0 = nt * NC;
-  if (herm && n0 + NC - 1 < m0) return;
-  const int st0 = z * kstages;
-  int nst = max(0, min(kstages, nstage_all - st0));
-  if (lower) nst = min(nst, (n0 + NC + kSliceK - 1) / kSliceK);  // b_n,k = 0 for k > n
+  const int ntiles = geo.per_z * geo.nz;
   if (tid == 0) {
     for (int b = 0; b < NS; ++b) {
       tc::mbar_init(&full[b], 1);
@@ -440,101 +507,153 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
   tc::tc_fence_after();
   const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
   volatile int* vfail = &s_fail;
-  const int nchunk = (nst + CH - 1) / CH;
-  long long acc[NSUM][2][HC];
-#pragma unroll
-  for (int q = 0; q < NSUM; ++q)
-#pragma unroll
-    for (int j = 0; j < HC; ++j) acc[q][0][j] = acc[q][1][j] = 0;
+  // sg: stages so far (buffer sg % NS), cg: chunks so far (parity of the group barriers); every role counts alike
   if (tid == 0) {  // operand tiles: two bulk copies per stage
-    for (int s = 0; s < nst && !*vfail; ++s) {
-      const int b = s % NS;
-      if (s >= NS && !tc::mbar_wait(&freeb[b], (uint32_t)(s / NS - 1) & 1u, kSlicePolls)) {
-        *vfail = 1;
-        break;
+    int sg = 0;
+    for (int t = blockIdx.x; t < ntiles && !*vfail; t += gridDim.x) {
+      const SliceTile<NC> tl(geo, t);
+      for (int s = 0; s < tl.nst && !*vfail; ++s, ++sg) {
+        const int b = sg % NS;
+        if (sg >= NS && !tc::mbar_wait(&freeb[b], (uint32_t)(sg / NS - 1) & 1u, kSlicePolls)) {
+          *vfail = 1;
+          break;
+        }
+        tc::mbar_arrive_expect_tx(&full[b], (uint32_t)BUF);
+        tc::bulk_g2s(smem + b * BUF, a_img + ((size_t)tl.mt * geo.nstage + tl.st0 + s) * AB, (uint32_t)AB, &full[b]);
+        tc::bulk_g2s(smem + b * BUF + AB, b_img + ((size_t)tl.nt * geo.nstage + tl.st0 + s) * BB, (uint32_t)BB,
+                     &full[b]);
+        s_last_copy[b] = sg;
       }
-      tc::mbar_arrive_expect_tx(&full[b], (uint32_t)BUF);
-      tc::bulk_g2s(smem + b * BUF, a_img + ((size_t)mt * nstage_all + st0 + s) * AB, (uint32_t)AB, &full[b]);
-      tc::bulk_g2s(smem + b * BUF + AB, b_img + ((size_t)nt * nstage_all + st0 + s) * BB, (uint32_t)BB, &full[b]);
-      s_last_copy[b] = s;
     }
   } else if (warp == 1) {  // the MMAs: group by group, so that a chunk's first groups drain while its last are formed
     const uint32_t leader = tc::elect_one();
     constexpr uint32_t idesc = tc::idesc_bf16(128, 2 * NC);
-    for (int s = 0; s < nst; ++s) {
-      const int b = s % NS, ch = s / CH;
-      const bool first = s % CH == 0, last = s % CH == CH - 1 || s == nst - 1;
-      // votes keep the loop's control flow, and with it the descriptors, uniform over the warp
-      if (!__all_sync(0xffffffffu, !*vfail && tc::mbar_wait(&full[b], (uint32_t)(s / NS) & 1u, kSlicePolls))) {
-        *vfail = 1;
-        break;
-      }
-      tc::tc_fence_after();
-      // descriptors by their low words: the stage's base plus constant offsets (in 16 bytes); the issuing
-      // thread's instructions per MMA are what the tensor pipe would otherwise wait for
-      const uint32_t a0 = (tc::smem_addr(smem + b * BUF) >> 4) | (128u >> 4) << 16, b0 = a0 + (uint32_t)(AB >> 4);
-      bool okg = true;
-#pragma unroll
-      for (int g = 2; g <= PMAX; ++g) {
-        if (first && ch > 0 && okg) {
-          okg = __all_sync(0xffffffffu, tc::mbar_wait(&gfree[g - 2], (uint32_t)(ch - 1) & 1u, kSlicePolls));
-          tc::tc_fence_after();
-        }
-        if (okg) {
-          const uint32_t d = tm + (uint32_t)((g - 2) * 2 * NC);
-#pragma unroll
-          for (int i = g > L ? g - L : 1; i <= (g > L ? L : g - 1); ++i) {
-            const uint32_t ai = a0 + (uint32_t)((i - 1) * 2 * (kSliceM * kSliceK * 2) >> 4);
-            const uint32_t bj = b0 + (uint32_t)((g - i - 1) * 3 * (NC * kSliceK * 2) >> 4);
-            tc::mma_bf16(d, tc::desc_lo(ai), tc::desc_lo(bj), idesc, first && i == (g > L ? g - L : 1) ? 0u : 1u, leader);
-            tc::mma_bf16(d, tc::desc_lo(ai + (kSliceM * kSliceK * 2 >> 4)), tc::desc_lo(bj + (NC * kSliceK * 2 >> 4)),
-                         idesc, 1u, leader);
-          }
-          if (last && leader) tc::mma_commit(&gfull[g - 2]);
-        }
-      }
-      if (!okg) {
-        *vfail = 1;
-        break;
-      }
-      if (leader) {
-        tc::mma_commit(&freeb[b]);
-        s_last_commit = s;
-      }
-    }
-  } else if (warp >= 2) {  // the sums: TMEM lanes 32 (warp % 4) .., columns HC half .. of Re and of Im
-    const uint32_t base = tm + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(((warp - 2) >> 2) * HC);
-    bool okc = true;
-    for (int ch = 0; ch < nchunk && okc; ++ch) {
-#pragma unroll
-      for (int g = 0; g < NG; ++g) {
-        if (okc && (*vfail || !tc::mbar_wait(&gfull[g], (uint32_t)ch & 1u, kSlicePolls))) okc = false;
-        okc = __all_sync(0xffffffffu, okc);
-        if (!okc) continue;
+    int sg = 0, cg = 0;
+    bool okg = true;
+    for (int t = blockIdx.x; t < ntiles && okg; t += gridDim.x) {
+      const SliceTile<NC> tl(geo, t);
+      for (int s = 0; s < tl.nst && okg; ++s, ++sg) {
+        const int b = sg % NS, ch = cg + s / CH;
+        const bool first = s % CH == 0, last = s % CH == CH - 1 || s == tl.nst - 1;
+        // votes keep the loop's control flow, and with it the descriptors, uniform over the warp
+        okg = __all_sync(0xffffffffu, !*vfail && tc::mbar_wait(&full[b], (uint32_t)(sg / NS) & 1u, kSlicePolls));
+        if (!okg) break;
         tc::tc_fence_after();
+        // descriptors by their low words: the stage's base plus constant offsets (in 16 bytes); the issuing
+        // warp's instructions per MMA are what the tensor pipe would otherwise wait for
+        const uint32_t a0 = (tc::smem_addr(smem + b * BUF) >> 4) | (128u >> 4) << 16, b0 = a0 + (uint32_t)(AB >> 4);
 #pragma unroll
-        for (int c0 = 0; c0 < HC; c0 += 16) {
-          uint32_t re[16], im[16];
-          tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + c0), re);
-          tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + NC + c0), im);
-          tc::tmem_ld_wait();
-          if (c0 + 16 == HC) {
-            tc::tc_fence_before();
-            tc::mbar_arrive(&gfree[g]);
+        for (int g = 2; g <= PMAX; ++g) {
+          if (first && ch > 0 && okg) {
+            okg = __all_sync(0xffffffffu, tc::mbar_wait(&gfree[g - 2], (uint32_t)(ch - 1) & 1u, kSlicePolls));
+            tc::tc_fence_after();
           }
+          if (okg) {
+            const uint32_t d = tm + (uint32_t)((g - 2) * 2 * NC);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            // weight 256^(PMAX - g): four groups per 64-bit sum
-            constexpr int kW[4] = {1 << 24, 1 << 16, 1 << 8, 1};
-            const int ir = __float2int_rn(__uint_as_float(re[j])), ii = __float2int_rn(__uint_as_float(im[j]));
-            long long &ar = acc[NSUM == 2 ? g / 4 : 0][0][c0 + j], &ai = acc[NSUM == 2 ? g / 4 : 0][1][c0 + j];
-            if (g % 4 == 0) { slice_acc<kW[0]>(ar, ir); slice_acc<kW[0]>(ai, ii); }
-            if (g % 4 == 1) { slice_acc<kW[1]>(ar, ir); slice_acc<kW[1]>(ai, ii); }
-            if (g % 4 == 2) { slice_acc<kW[2]>(ar, ir); slice_acc<kW[2]>(ai, ii); }
-            if (g % 4 == 3) { slice_acc<kW[3]>(ar, ir); slice_acc<kW[3]>(ai, ii); }
+            for (int i = g > L ? g - L : 1; i <= (g > L ? L : g - 1); ++i) {
+              const uint32_t ai = a0 + (uint32_t)((i - 1) * 2 * (kSliceM * kSliceK * 2) >> 4);
+              const uint32_t bj = b0 + (uint32_t)((g - i - 1) * 3 * (NC * kSliceK * 2) >> 4);
+              tc::mma_bf16(d, tc::desc_lo(ai), tc::desc_lo(bj), idesc, first && i == (g > L ? g - L : 1) ? 0u : 1u,
+                           leader);
+              tc::mma_bf16(d, tc::desc_lo(ai + (kSliceM * kSliceK * 2 >> 4)),
+                           tc::desc_lo(bj + (NC * kSliceK * 2 >> 4)), idesc, 1u, leader);
+            }
+            if (last && leader) tc::mma_commit(&gfull[g - 2]);
+          }
+        }
+        if (!okg) break;
+        if (leader) {
+          tc::mma_commit(&freeb[b]);
+          s_last_commit = sg;
+        }
+      }
+      cg += (tl.nst + CH - 1) / CH;
+    }
+    if (!okg) *vfail = 1;
+  } else if (warp >= 2) {  // the sums: TMEM lanes 32 (warp % 4) .., columns HC half .. of Re and of Im
+    constexpr int PC = HC % 16 == 0 ? 16 : 8;  // columns per read
+    const uint32_t base = tm + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(((warp - 2) >> 2) * HC);
+    int cg = 0;
+    bool okc = true;
+    for (int t = blockIdx.x; t < ntiles && okc; t += gridDim.x) {
+      const SliceTile<NC> tl(geo, t);
+      const int nchunk = (tl.nst + CH - 1) / CH;
+      long long acc[NSUM][2][HC];
+#pragma unroll
+      for (int q = 0; q < NSUM; ++q)
+#pragma unroll
+        for (int j = 0; j < HC; ++j) acc[q][0][j] = acc[q][1][j] = 0;
+      for (int ch = 0; ch < nchunk && okc; ++ch, ++cg) {
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+          if (okc && (*vfail || !tc::mbar_wait(&gfull[g], (uint32_t)cg & 1u, kSlicePolls))) okc = false;
+          okc = __all_sync(0xffffffffu, okc);
+          if (!okc) continue;
+          tc::tc_fence_after();
+#pragma unroll
+          for (int c0 = 0; c0 < HC; c0 += PC) {
+            uint32_t re[PC], im[PC];
+            if constexpr (PC == 16) {
+              tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + c0), re);
+              tc::tmem_ld_x16(base + (uint32_t)(g * 2 * NC + NC + c0), im);
+            } else {
+              tc::tmem_ld_x8_async(base + (uint32_t)(g * 2 * NC + c0), re);
+              tc::tmem_ld_x8_async(base + (uint32_t)(g * 2 * NC + NC + c0), im);
+            }
+            tc::tmem_ld_wait();
+            if (c0 + PC == HC) {
+              tc::tc_fence_before();
+              tc::mbar_arrive(&gfree[g]);
+            }
+#pragma unroll
+            for (int j = 0; j < PC; ++j) {
+              // weight 256^(PMAX - g): four groups per 64-bit sum
+              constexpr int kW[4] = {1 << 24, 1 << 16, 1 << 8, 1};
+              const int ir = __float2int_rn(__uint_as_float(re[j])), ii = __float2int_rn(__uint_as_float(im[j]));
+              long long &ar = acc[NSUM == 2 ? g / 4 : 0][0][c0 + j], &ai = acc[NSUM == 2 ? g / 4 : 0][1][c0 + j];
+              if (g % 4 == 0) { slice_acc<kW[0]>(ar, ir); slice_acc<kW[0]>(ai, ii); }
+              if (g % 4 == 1) { slice_acc<kW[1]>(ar, ir); slice_acc<kW[1]>(ai, ii); }
+              if (g % 4 == 2) { slice_acc<kW[2]>(ar, ir); slice_acc<kW[2]>(ai, ii); }
+              if (g % 4 == 3) { slice_acc<kW[3]>(ar, ir); slice_acc<kW[3]>(ai, ii); }
+            }
           }
         }
       }
+      const int row = tl.mt * kSliceM + 32 * (warp & 3) + lane, n0 = tl.nt * NC + ((warp - 2) >> 2) * HC;
+      const int sa = row < M ? ea[(size_t)tl.z * ea_ld + row] : 0;
+      const int* ebz = eb + (size_t)tl.z * eb_ld;
+      constexpr int JB = sizeof(OUT) == 8 ? 4 : 8;  // loads in flight before their first store
+      if (okc && row < M)
+#pragma unroll
+      for (int j0 = 0; j0 < HC; j0 += JB) {
+        cplx<OUT> old[JB];
+        if constexpr (MODE == 1) {
+#pragma unroll
+          for (int j = 0; j < JB; ++j) {
+            const int n = n0 + j0 + j;
+            old[j] = accum && n < N ? out[(size_t)n * ldo + row] : mk<OUT>(0, 0);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < JB; ++j) {
+          const int n = n0 + j0 + j, i = j0 + j;
+          if (n >= N) continue;
+          const int sb = ebz[n];
+          cplx<OUT> v;
+          if (sa == kSliceBad || sb == kSliceBad) v = mk<OUT>(NAN, NAN);
+          else if constexpr (std::is_same<OUT, float>::value)
+            v = mk<OUT>(slice_to_float(acc[0][0][i], sa + sb), slice_to_float(acc[0][1][i], sa + sb));
+          else if constexpr (NSUM == 2)
+            v = mk<OUT>(slice_to_double(acc[0][0][i], acc[NSUM - 1][0][i], sa + sb),
+                        slice_to_double(acc[0][1][i], acc[NSUM - 1][1][i], sa + sb));
+          else
+            v = mk<OUT>(slice_to_double(0, acc[0][0][i], sa + sb), slice_to_double(0, acc[0][1][i], sa + sb));
+          if constexpr (MODE == 0) out[((size_t)tl.z * M + row) * N + n] = v;
+          else out[(size_t)n * ldo + row] = accum ? cadd(old[j], v) : v;
+        }
+      }
+      __syncwarp();
     }
     if (!okc) *vfail = 1;
   }
@@ -543,58 +662,17 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
   int ok = !*vfail;
   const int lc = s_last_commit;
   if (lc >= 0 && !tc::mbar_wait(&freeb[lc % NS], (uint32_t)(lc / NS) & 1u, kSlicePolls)) ok = 0;
-  if (lc != nst - 1) ok = 0;
   if (tid == 0)
     for (int b = 0; b < NS; ++b)
       if (s_last_copy[b] > lc) tc::mbar_wait(&full[b], (uint32_t)(s_last_copy[b] / NS) & 1u, kSlicePolls);
   ok = __syncthreads_and(ok);
-  if (warp >= 2 && ok) {
-    const int row = m0 + 32 * (warp & 3) + lane, c0 = n0 + ((warp - 2) >> 2) * HC;
-    if (row < M) {
-      const int sa = ea[(size_t)z * ea_ld + row];
-      const int* ebz = eb + (size_t)z * eb_ld;
-      if constexpr (MODE == 0) {
-        cplx<OUT>* o = out + ((size_t)z * M + row) * N;
-#pragma unroll
-        for (int j = 0; j < HC; ++j) {
-          const int n = c0 + j;
-          if (n >= N) continue;
-          const int sb = ebz[n];
-          cplx<OUT> v;
-          if (sa == kSliceBad || sb == kSliceBad) v = mk<OUT>(NAN, NAN);
-          else if constexpr (NSUM == 2)
-            v = mk<OUT>(slice_to_double(acc[0][0][j], acc[NSUM - 1][0][j], sa + sb),
-                        slice_to_double(acc[0][1][j], acc[NSUM - 1][1][j], sa + sb));
-          else
-            v = mk<OUT>(slice_to_double(0, acc[0][0][j], sa + sb), slice_to_double(0, acc[0][1][j], sa + sb));
-          o[n] = v;
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < HC; ++j) {
-          const int n = c0 + j;
-          if (n >= N) continue;
-          const int sb = ebz[n];
-          cplx<OUT>* y = out + (size_t)n * ldo + row;
-          cplx<OUT> v;
-          if (sa == kSliceBad || sb == kSliceBad) v = mk<OUT>(NAN, NAN);
-          else if constexpr (std::is_same<OUT, float>::value)
-            v = mk<OUT>(slice_to_float(acc[0][0][j], sa + sb), slice_to_float(acc[0][1][j], sa + sb));
-          else
-            v = mk<OUT>(slice_to_double(acc[0][0][j], acc[NSUM - 1][0][j], sa + sb),
-                        slice_to_double(acc[0][1][j], acc[NSUM - 1][1][j], sa + sb));
-          *y = accum ? cadd(*y, v) : v;
-        }
-      }
-    }
-  }
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc::tc_fence_after();
     tc::tmem_dealloc(tmem_base, 512u);
   }
-  if (!ok && tid == 0 && nst > 0) atomicExch(err, 1);
+  if (!ok && tid == 0) atomicExch(err, 1);
 }
 
 // C[m][n] = sum of the slices' partials; elements whose tile was skipped are the conjugate of their mirror
@@ -613,38 +691,71 @@ __global__ void k_slice_reduce(int M, int N, int nz, const double2* __restrict__
 // ------------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------------
+static const int kSliceSms = 152;  // one CTA per SM (its tensor memory is full)
 template <typename T> struct SliceL { static constexpr int value = sizeof(T) == 8 ? 7 : 4; };
 
-template <int L, int MODE, typename OUT>
-static int slice_launch(Ctx* c, dim3 grid, int M, int N, int nstage, int kstages, const unsigned char* a,
-                        const int* ea, int ea_ld, const unsigned char* b, const int* eb, int eb_ld, cplx<OUT>* out,
-                        int ldo, bool herm, bool lower, bool accum) {
+template <int L, int NC, int MODE, typename OUT>
+static int slice_launch_nc(Ctx* c, int M, int N, const SliceTiles& geo, const unsigned char* a, const int* ea, int ea_ld,
+                           const unsigned char* b, const int* eb, int eb_ld, cplx<OUT>* out, int ldo, bool accum) {
   int* err = tc_err_flag(c);
   if (!err) return PARO_ERR_CUDA;
-  const size_t sm = (size_t)SliceCfg<L>::NS * (slice_a_bytes<L>() + slice_b_bytes<L>()) + 1024;
+  const size_t sm = (size_t)SliceCfg<L>::NS * (slice_a_bytes<L>() + slice_b_bytes<L>(NC)) + 1024;
   static int attr_dev = -1;
   int dev = 0;
   PARO_CU(c, cudaGetDevice(&dev));
   if (attr_dev != dev) {
-    PARO_CU(c, cudaFuncSetAttribute(k_slice_gemm<L, MODE, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    PARO_CU(c, cudaFuncSetAttribute(k_slice_gemm<L, NC, MODE, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sm));
     attr_dev = dev;
   }
-  k_slice_gemm<L, MODE, OUT><<<grid, kSliceThreads, sm, c->stream>>>(M, N, nstage, kstages, a, ea, ea_ld, b, eb, eb_ld,
-                                                                     out, ldo, herm, lower, accum, err);
+  const int tiles = geo.per_z * geo.nz;
+  k_slice_gemm<L, NC, MODE, OUT><<<std::min(tiles, kSliceSms), kSliceThreads, sm, c->stream>>>(
+      M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum, err);
   PARO_LAUNCH(c, "k_slice_gemm");
   return PARO_OK;
+}
+template <int L, int MODE, typename OUT>
+static int slice_launch(Ctx* c, int nc, int M, int N, const SliceTiles& geo, const unsigned char* a, const int* ea,
+                        int ea_ld, const unsigned char* b, const int* eb, int eb_ld, cplx<OUT>* out, int ldo,
+                        bool accum) {
+  if constexpr (L == 7) {
+    return slice_launch_nc<7, 32, MODE, OUT>(c, M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum);
+  } else {
+    if (nc == 48) return slice_launch_nc<4, 48, MODE, OUT>(c, M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum);
+    return slice_launch_nc<4, 64, MODE, OUT>(c, M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum);
+  }
 }
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+template <typename T, int L>
+static int slice_rows(Ctx* c, int rows, int rows_a, int rows_b, int pad, int K, int kslice, int nz, int nstage,
+                      const cplx<T>* x, int ld, unsigned char* a_img, unsigned char* b_img, int* es,
+                      const int* rowkey = nullptr, int nc = 64) {
+  const int stage = std::min(kslice, SliceStage<T>::value);
+  k_slice_rows<T, L><<<dim3(pad / 8, nz), 256, (size_t)8 * (stage + 1) * sizeof(cplx<T>), c->stream>>>(
+      rows, rows_a, rows_b, K, kslice, nstage, x, ld, 0, a_img, b_img, es, pad, stage, rowkey, nc);
+  PARO_LAUNCH(c, "k_slice_rows");
+  return PARO_OK;
+}
+
+template <typename T>
+static int slice_rowkeys(Ctx* c, int rows, int n, const cplx<T>* x, int ld, bool finite, int* rowkey) {
+  PARO_CU(c, cudaMemsetAsync(rowkey, 0, (size_t)rows * sizeof(int), c->stream));
+  const int seg = std::max(1, std::min((n + 1023) / 1024, 2048 / rows));
+  k_slice_rowkey<T><<<dim3(seg, rows), 256, 0, c->stream>>>(n, x, ld, finite, rowkey);
+  PARO_LAUNCH(c, "k_slice_rowkey");
+  return PARO_OK;
+}
+
 // K slices of the long-K product: the count that minimises waves of 152 CTAs times (stages + the stages' worth
-// of a CTA's start and conversion, about 8)
+// of a CTA's start and a tile's conversion, about 4)
 static int slice_split_k(int tiles, int nstage) {
   int best_nz = 1;
   long long best = -1;
   for (int nz = 1; nz <= std::max(1, nstage / 4); ++nz) {
     const int ks = (nstage + nz - 1) / nz, z = (nstage + ks - 1) / ks;
-    const long long cost = ((long long)tiles * z + 151) / 152 * (ks + 8) * 64 + z;  // ties: fewer slices
+    const long long cost = ((long long)tiles * z + 151) / 152 * (ks + 4) * 64 + z;  // ties: fewer slices
     if (best < 0 || cost < best) {
       best = cost;
       best_nz = z;
@@ -657,7 +768,8 @@ static int slice_split_k(int tiles, int nstage) {
 template <typename T>
 static int slice_cn(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, const unsigned char* a_img, const int* ea,
                     const cplx<T>* B, int ldb, double2* C, int ldc, bool herm) {
-  constexpr int L = SliceL<T>::value, NC = SliceCfg<L>::NC;
+  constexpr int L = SliceL<T>::value;
+  const int NC = slice_nc<L>(N);
   const int mt = (M + kSliceM - 1) / kSliceM, nt = (N + NC - 1) / NC, nstage = (K + kSliceK - 1) / kSliceK;
   int tiles = mt * nt;
   if (herm)
@@ -668,7 +780,7 @@ static int slice_cn(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, cons
   const int ma = mt * kSliceM, nb = nt * NC;
   const bool same = !a_img && A == B && lda == ldb && M == N;
   const int pad = same ? std::max(ma, nb) : nb;
-  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)nt * nstage * slice_b_bytes<L>()));
+  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)nt * nstage * slice_b_bytes<L>(NC)));
   int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)nz * pad * sizeof(int)));
   double2* part = static_cast<double2*>(ws_get(c, "gemm_parts", (size_t)nz * M * N * sizeof(double2)));
   unsigned char* ai = nullptr;
@@ -680,18 +792,17 @@ static int slice_cn(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, cons
   }
   if (!bi || !eb || !part) return PARO_ERR_CUDA;
   cudaEvent_t ev = prof_begin(c);
-  if (!a_img && !same) {
-    k_slice_rows<T, L><<<dim3(ma / 8, nz), 256, 0, c->stream>>>(M, ma, 0, K, ks * kSliceK, nstage, A, lda, 0, ai,
-                                                                nullptr, ean, ma);
-    PARO_LAUNCH(c, "k_slice_rows");
-  }
-  k_slice_rows<T, L><<<dim3(pad / 8, nz), 256, 0, c->stream>>>(N, same ? ma : 0, nb, K, ks * kSliceK, nstage, B, ldb, 0,
-                                                               same ? ai : nullptr, bi, eb, pad);
-  PARO_LAUNCH(c, "k_slice_rows");
+  int st;
+  if (!a_img && !same && (st = slice_rows<T, L>(c, M, ma, 0, ma, K, ks * kSliceK, nz, nstage, A, lda, ai, nullptr, ean)))
+    return st;
+  if ((st = slice_rows<T, L>(c, N, same ? ma : 0, nb, pad, K, ks * kSliceK, nz, nstage, B, ldb, same ? ai : nullptr, bi, eb,
+                             nullptr, NC)))
+    return st;
   prof_end(c, sizeof(T) == 8 ? "k_slice_rows<f64>" : "k_slice_rows<f32>", ev);
   ev = prof_begin(c);
-  int st = slice_launch<L, 0, double>(c, dim3(nt, mt, nz), M, N, nstage, ks, a_img ? a_img : ai, a_img ? ea : ean,
-                                      a_img ? 0 : (same ? pad : ma), bi, eb, pad, part, 0, herm, false, false);
+  const SliceTiles geo{nt, mt, nz, nstage, ks, herm ? 1 : 0, 0, tiles};
+  st = slice_launch<L, 0, double>(c, NC, M, N, geo, a_img ? a_img : ai, a_img ? ea : ean,
+                                  a_img ? 0 : (same ? pad : ma), bi, eb, pad, part, 0, false);
   if (st) return st;
   prof_end(c, sizeof(T) == 8 ? "k_slice_gemm_cn<f64>" : "k_slice_gemm_cn<f32>", ev);
   k_slice_reduce<<<(M * N + 255) / 256, 256, 0, c->stream>>>(M, N, nz, part, C, ldc, herm, NC);
@@ -709,9 +820,10 @@ int gemm_cn_slice(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, const 
 template <typename T>
 static int slice_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<T>* X,
                     int ldx, const unsigned char* a_img, const int* ea, cplx<T>* Y, int ldy, bool accum, bool lower) {
-  constexpr int L = SliceL<T>::value, NC = SliceCfg<L>::NC;
+  constexpr int L = SliceL<T>::value;
+  const int NC = slice_nc<L>(M);
   const int at = (N + kSliceM - 1) / kSliceM, bt = (M + NC - 1) / NC, nstage = (K + kSliceK - 1) / kSliceK;
-  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)bt * nstage * slice_b_bytes<L>()));
+  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)bt * nstage * slice_b_bytes<L>(NC)));
   int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)bt * NC * sizeof(int)));
   if (!bi || !eb) return PARO_ERR_CUDA;
   int* rowkey = nullptr;
@@ -722,21 +834,18 @@ static int slice_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool
     if (!ai || !ean) return PARO_ERR_CUDA;
     rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)std::max(K, 1) * sizeof(int)));
     if (!rowkey) return PARO_ERR_CUDA;
-    PARO_CU(c, cudaMemsetAsync(rowkey, 0, (size_t)K * sizeof(int), c->stream));
-    k_slice_rowkey<T><<<dim3(std::max(1, std::min((N + 1023) / 1024, 2048 / K)), K), 256, 0, c->stream>>>(N, X, ldx,
-                                                                                                     rowkey);
-    PARO_LAUNCH(c, "k_slice_rowkey");
+    if (int st = slice_rowkeys<T>(c, K, N, X, ldx, true, rowkey)) return st;
     k_slice_cols<T, L><<<at * kSliceM / 32, 256, 0, c->stream>>>(N, K, nstage, X, ldx, rowkey, ai, ean);
     PARO_LAUNCH(c, "k_slice_cols");
     a_img = ai;
     ea = ean;
   }
-  k_slice_w<L, T><<<bt * NC / 8, 256, 0, c->stream>>>(M, K, nstage, W, ldw, wt ? 1 : 0, s, rowkey, bi, eb);
+  k_slice_w<L, T><<<bt * NC / 8, 256, 0, c->stream>>>(M, K, nstage, W, ldw, wt ? 1 : 0, s, rowkey, bi, eb, NC);
   PARO_LAUNCH(c, "k_slice_w");
   prof_end(c, sizeof(T) == 8 ? "k_slice_cols<f64>" : "k_slice_cols<f32>", ev);
   ev = prof_begin(c);
-  int st = slice_launch<L, 1, T>(c, dim3(bt, at), N, M, nstage, nstage, a_img, ea, 0, bi, eb, 0, Y, ldy, false, lower,
-                                 accum);
+  const SliceTiles geo{bt, at, 1, nstage, nstage, 0, lower ? 1 : 0, bt * at};
+  int st = slice_launch<L, 1, T>(c, NC, N, M, geo, a_img, ea, 0, bi, eb, 0, Y, ldy, accum);
   if (st) return st;
   prof_end(c, sizeof(T) == 8 ? "k_slice_gemm_wx<f64>" : "k_slice_gemm_wx<f32>", ev);
   return PARO_OK;
@@ -770,9 +879,15 @@ static int slice_beta_images(Ctx* c, int ik) {
   im.wx = p + bcn;
   im.ecn = reinterpret_cast<int*>(p + bcn + bwx);
   im.ewx = im.ecn + ma;
-  k_slice_rows<T, L><<<ma / 8, 256, 0, c->stream>>>(np, ma, 0, npw, scn * kSliceK, scn, slice_beta<T>(B), npw, 0, im.cn,
-                                                    nullptr, im.ecn, ma);
-  PARO_LAUNCH(c, "k_slice_rows");
+  int* rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)np * sizeof(int)));
+  if (!rowkey) return PARO_ERR_CUDA;
+  int st = slice_rowkeys<T>(c, np, npw, slice_beta<T>(B), npw, false, rowkey);
+  if (st) return st;
+  const int nzi = std::max(1, std::min((npw + 511) / 512, 1216 / (ma / 8)));
+  const int ksi = (scn + nzi - 1) / nzi;
+  if ((st = slice_rows<T, L>(c, np, ma, 0, ma, npw, ksi * kSliceK, (scn + ksi - 1) / ksi, scn, slice_beta<T>(B), npw,
+                             im.cn, nullptr, im.ecn, rowkey)))
+    return st;
   k_slice_cols<T, L><<<na / 32, 256, 0, c->stream>>>(npw, np, swx, slice_beta<T>(B), npw, nullptr, im.wx,
                                                         im.ewx);
   PARO_LAUNCH(c, "k_slice_cols");

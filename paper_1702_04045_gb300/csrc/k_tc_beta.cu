@@ -411,14 +411,14 @@ static size_t cnb_smem(int NT, int NR) {
   return (size_t)2 * (2 * kTileF4 * 16 + 4 * NT * kBCh * 16) + (size_t)NR * NT * kCnbRawPitch + 1024;
 }
 
-int gemm_cn_tc_beta(Ctx* c, int ik, int nb, const float2* x, double2* P, int* err) {
+int gemm_cn_tc_beta(Ctx* c, int ik, int nb, const float2* x, double2* P, int* err, int plan_nb) {
   const Basis& B = c->bases[ik];
   const int M = c->nproj, N = nb, K = B.npw;
   const int ntiles = (N + 255) / 256;
   const int NT = ((N + ntiles - 1) / ntiles + 15) / 16 * 16;
   const int mtiles = (M + kBM - 1) / kBM;
   int nz = 1, kslice = kBKC;
-  tc_cn_plan(M, N, K, &nz, &kslice);
+  tc_cn_plan(M, plan_nb > 0 ? plan_nb : N, K, &nz, &kslice);
   float2* part = static_cast<float2*>(ws_get(c, "tc_parts32", (size_t)nz * M * N * sizeof(float2)));
   if (!part) return PARO_ERR_CUDA;
   int nr = 4;

@@ -273,8 +273,9 @@ int* tc_err_flag(Ctx* c);
 int tc_flag_readback(Ctx* c, const int** h);
 // ---- tensor-core products with the projectors as the fixed operand (k_tc_beta.cu) ----
 int beta_images(Ctx* c, int ik);  // forms the two images of k-point ik if they are missing
-// P[p][b] = <beta_p | x_b> for nb rows x (FP32, ld = N_pw)
-int gemm_cn_tc_beta(Ctx* c, int ik, int nb, const float2* x, double2* P, int* err);
+// P[p][b] = <beta_p | x_b> for nb rows x (FP32, ld = N_pw); the K slices are those of plan_nb rows when given (the
+// tensor core's FP32 accumulation errs with the length of a slice, and fewer rows get shorter slices)
+int gemm_cn_tc_beta(Ctx* c, int ik, int nb, const float2* x, double2* P, int* err, int plan_nb = 0);
 // y_b += sum_p beta_p D_p P[p][b] (y: nb rows, FP32, ld = N_pw)
 int gemm_wx_tc_beta(Ctx* c, int ik, int nb, const double2* P, const double* dvec, float2* y, int* err);
 // whether FP64 products take the digit slices
@@ -347,9 +348,9 @@ int convert(Ctx* c, size_t n, const cplx<TS>* src, cplx<TD>* dst);
 // ---- KB projectors (k_hpsi.cu) ----
 template <typename T>
 int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi);
-// the projections P[p][b] = <beta_p | psi_b> alone (nproj x nb)
+// the projections P[p][b] = <beta_p | psi_b> alone (nproj x nb); plan_nb as in gemm_cn_tc_beta
 template <typename T>
-int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P);
+int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P, int plan_nb = 0);
 
 // Suspends the real-wavefunction mode for the scope (calls on general complex vectors, packed rows).
 struct GammaPackOff {
