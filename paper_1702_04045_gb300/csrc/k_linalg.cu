@@ -957,8 +957,9 @@ static size_t chol_blocked_smem(int n, int C) {
 static int chol_cluster_shape(Ctx* c, int n, Ctx::CholShape* out) {
   int dev = 0;
   PARO_CU(c, cudaGetDevice(&dev));
-  if (c->chol_shape.n == n && c->chol_shape.dev == dev) {
-    *out = c->chol_shape;
+  const auto known = c->chol_shapes.find(n);
+  if (known != c->chol_shapes.end() && known->second.dev == dev) {
+    *out = known->second;
     return PARO_OK;
   }
   const size_t cap = 220 * 1024;
@@ -1007,12 +1008,12 @@ static int chol_cluster_shape(Ctx* c, int n, Ctx::CholShape* out) {
         sh.cls = C;
         sh.thr = thr;
         sh.smem = sm;
-        c->chol_shape = *out = sh;
+        c->chol_shapes[n] = *out = sh;
         return PARO_OK;
       }
     }
   }
-  c->chol_shape = *out = sh;
+  c->chol_shapes[n] = *out = sh;
   return PARO_OK;
 }
 
@@ -1067,11 +1068,169 @@ __global__ void __launch_bounds__(1024) k_orth_first_order(int n, const double2*
                  : k == r ? make_double2(1.5 - 0.5 * v.x, 0.0)
                           : make_double2(__longlong_as_double(__double_as_longlong(v.x) ^ (long long)0x8000000000000000ULL),
                                          v.y);
+// C[i][j] = D[i][j] + sign sum_k a(i, k) b(k, j), complex FP64, for the small blocks of chol_split: a = A[i lda + k]
+// (conjugated with CA), b = B[j ldb + k] (TB) or B[k ldb + j] (conjugated with CB); D may be null. 8 x 16 outputs per
+// CTA with the K range in four parts, so a 144^3 product is 162 CTAs of FP64 work.
+template <bool CA, bool TB, bool CB>
+__global__ void __launch_bounds__(512) k_zblock(int M, int N, int K, const double2* __restrict__ A, int lda,
+                                                const double2* __restrict__ B, int ldb, const double2* __restrict__ D,
+                                                int ldd, double sign, double2* __restrict__ C, int ldc) {
+  __shared__ double2 As[4][8][17], Bs[4][16][17];
+  __shared__ double2 red[4][128];
+  const int q = threadIdx.x >> 7, t = threadIdx.x & 127, r = t >> 4, cc = t & 15;
+  const int i0 = blockIdx.y * 8, j0 = blockIdx.x * 16;
+  const int kp = ((K + 3) / 4 + 15) / 16 * 16, k0 = q * kp, k1 = min(K, k0 + kp);
+  double2 acc = make_double2(0.0, 0.0);
+  for (int s = 0; s < kp; s += 16) {
+    const int kb = k0 + s;
+    {
+      const int k = kb + cc;
+      As[q][r][cc] = i0 + r < M && k < k1 ? A[(size_t)(i0 + r) * lda + k] : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {  // B tile: 16 columns x 16 k
+      const int x = r + 8 * u;
+      double2 v = make_double2(0.0, 0.0);
+      if (TB) {
+        if (j0 + x < N && kb + cc < k1) v = B[(size_t)(j0 + x) * ldb + kb + cc];
+        Bs[q][x][cc] = v;
+      } else {
+        if (j0 + cc < N && kb + x < k1) v = B[(size_t)(kb + x) * ldb + j0 + cc];
+        Bs[q][cc][x] = v;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const double2 av = As[q][r][k], bv = Bs[q][cc][k];
+      acc = zfma(acc, CA ? cconj(av) : av, CB ? cconj(bv) : bv);
+    }
+    __syncthreads();
+  }
+  red[q][t] = acc;
+  __syncthreads();
+  if (q == 0 && i0 + r < M && j0 + cc < N) {
+    const double2 v = cadd(cadd(red[0][t], red[1][t]), cadd(red[2][t], red[3][t]));
+    const double2 d = D ? D[(size_t)(i0 + r) * ldd + j0 + cc] : make_double2(0.0, 0.0);
+    C[(size_t)(i0 + r) * ldc + j0 + cc] = make_double2(d.x + sign * v.x, d.y + sign * v.y);
+  }
+}
+
+// dst (n1 x n2, ld ldd) = src (ld lds), or zero when src is null
+__global__ void k_zcopy(int n1, int n2, const double2* __restrict__ src, int lds, double2* __restrict__ dst, int ldd) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n1 * n2) return;
+  const int r = i / n2, c = i - r * n2;
+  dst[(size_t)r * ldd + c] = src ? src[(size_t)r * lds + c] : make_double2(0.0, 0.0);
+}
+
+static int launch_chol_cluster(Ctx* c, const Ctx::CholShape& sh, int n, const double2* s, double2* g, int* flag,
+                               const int* skip) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = sh.cls;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(sh.cls);
+  cfg.blockDim = dim3(sh.thr);
+  cfg.dynamicSmemBytes = sh.smem;
+  cfg.stream = c->stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaEvent_t ev = prof_begin(c);
+  if (sh.kind == 1) PARO_CU(c, cudaLaunchKernelEx(&cfg, k_chol_blocked, n, s, g, flag, skip));
+  else PARO_CU(c, cudaLaunchKernelEx(&cfg, k_chol_cluster, n, s, g, flag, skip));
+  ++c->launches;
+  prof_end(c, "k_chol_cluster", ev);
+  return PARO_OK;
+}
+
+// Cholesky of orders whose blocked form does not fit one cluster's shared memory, by 2 x 2 blocks with a first
+// block of n1 columns (S11 = L11 L11^H by the blocked cluster kernel):
+//   L21 = S21 L11^{-H},  S22 - L21 L21^H = L22 L22^H (again by blocks when it does not fit),
+//   G = conj(L)^{-1}: G11, G22 from the factorisations, G21 = -G22 conj(L21) G11.
+// The products run on all SMs; the column-by-column cluster kernel took 2.1 ms for n = 288, the two blocked
+// factorisations and four products 0.7 ms. S (ld lds, its lower triangle) is overwritten in the Schur complement.
+static int chol_split(Ctx* c, int n, double2* S, int lds, double2* G, int ldg, double2* tmp, int piece, int* flags,
+                      int* nflag) {
+  const int pieces = (n + piece - 1) / piece;
+  const int n1 = std::min(n, ((n + pieces - 1) / pieces + 15) / 16 * 16), n2 = n - n1;
+  double2 *s1 = tmp, *g1 = tmp + (size_t)piece * piece;  // contiguous copies for the cluster kernel
+  auto grid = [](int m, int k) { return dim3((k + 15) / 16, (m + 7) / 8); };
+  auto copy = [&](int a, int b, const double2* src, int ls, double2* dst, int ld) {
+    k_zcopy<<<(a * b + 255) / 256, 256, 0, c->stream>>>(a, b, src, ls, dst, ld);
+  };
+  Ctx::CholShape sh;
+  int st = chol_cluster_shape(c, n1, &sh);
+  if (st) return st;
+  if (sh.kind == 0 || *nflag >= 64) return fail(c, PARO_ERR_CUDA, "Cholesky: cluster kernel not available");
+  copy(n1, n1, S, lds, s1, n1);
+  PARO_LAUNCH(c, "k_zcopy");
+  if ((st = launch_chol_cluster(c, sh, n1, s1, g1, flags + (*nflag)++, nullptr))) return st;
+  copy(n1, n1, g1, n1, G, ldg);
+  PARO_LAUNCH(c, "k_zcopy");
+  if (n2 == 0) return PARO_OK;
+  copy(n1, n2, nullptr, 0, G + n1, ldg);  // above the diagonal
+  PARO_LAUNCH(c, "k_zcopy");
+  double2 *L21 = tmp + 2 * (size_t)piece * piece, *T = L21 + (size_t)n2 * n1;
+  double2* S21 = S + (size_t)n1 * lds;
+  k_zblock<false, true, false><<<grid(n2, n1), 512, 0, c->stream>>>(n2, n1, n1, S21, lds, G, ldg, nullptr, 0, 1.0, L21, n1);
+  PARO_LAUNCH(c, "k_zblock");
+  double2* S22 = S21 + n1;
+  k_zblock<false, true, true><<<grid(n2, n2), 512, 0, c->stream>>>(n2, n2, n1, L21, n1, L21, n1, S22, lds, -1.0, S22, lds);
+  PARO_LAUNCH(c, "k_zblock");
+  k_zblock<true, false, false><<<grid(n2, n1), 512, 0, c->stream>>>(n2, n1, n1, L21, n1, G, ldg, nullptr, 0, 1.0, T, n1);
+  PARO_LAUNCH(c, "k_zblock");
+  double2* G22 = G + (size_t)n1 * ldg + n1;
+  if ((st = chol_split(c, n2, S22, lds, G22, ldg, T + (size_t)n2 * n1, piece, flags, nflag))) return st;
+  k_zblock<false, false, false><<<grid(n2, n1), 512, 0, c->stream>>>(n2, n1, n2, G22, ldg, T, n1, nullptr, 0, -1.0,
+                                                                     G + (size_t)n1 * ldg, ldg);
+  PARO_LAUNCH(c, "k_zblock");
+  return PARO_OK;
+}
+
+// largest order of the blocked cluster form on this device (0: none)
+static int chol_piece(Ctx* c, int* piece) {
+  *piece = 0;
+  for (int n = 192; n >= 96; n -= 16) {
+    Ctx::CholShape sh;
+    if (int st = chol_cluster_shape(c, n, &sh)) return st;
+    if (sh.kind == 1) {
+      *piece = n;
+      return PARO_OK;
+    }
+  }
+  return PARO_OK;
+}
+
   }
 }
 
 int chol_cluster_available(Ctx* c, int n, bool* avail) {
   Ctx::CholShape sh;
+    if (sh.kind != 1 && !defer && !skip && !c->plain64) {
+      int piece = 0, nflag = 0;
+      if ((st = chol_piece(c, &piece))) return st;
+      if (piece > 0 && n > piece) {
+        int* flags = static_cast<int*>(ws_get(c, "chol_split_flags", 64 * sizeof(int)));
+        // S, then per level the cluster kernel's blocks and L21, T (their sum stays below 2 n^2)
+        const size_t nn = (size_t)n * n, levels = (size_t)(n + piece - 1) / piece;
+        double2* W = static_cast<double2*>(
+            ws_get(c, "chol_split", (3 * nn + 2 * levels * piece * piece) * sizeof(double2)));
+        if (!flags || !W) return PARO_ERR_CUDA;
+        PARO_CU(c, cudaMemcpyAsync(W, s, nn * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
+        if ((st = chol_split(c, n, W, n, g, n, W + nn, piece, flags, &nflag))) return st;
+        int h[64];
+        PARO_CU(c, cudaMemcpyAsync(h, flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        PARO_CU(c, cudaStreamSynchronize(c->stream));
+        for (int i = 0; i < nflag; ++i)
+          if (h[i]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 in block " + std::to_string(i) + ", column " +
+                                                           std::to_string(h[i] - 1));
+        return PARO_OK;
+      }
+      if ((st = chol_cluster_shape(c, n, &sh))) return st;
+    }
   const int st = chol_cluster_shape(c, n, &sh);
   *avail = st == PARO_OK && sh.kind > 0;
   return st;
@@ -1095,23 +1254,7 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
     if (sh.kind > 0) {
       int* flags = static_cast<int*>(ws_get(c, "chol_flags", 8 * sizeof(int)));
       if (!flags) return PARO_ERR_CUDA;
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = sh.cls;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3(sh.cls);
-      cfg.blockDim = dim3(sh.thr);
-      cfg.dynamicSmemBytes = sh.smem;
-      cfg.stream = c->stream;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      cudaEvent_t ev = prof_begin(c);
-      if (sh.kind == 1) PARO_CU(c, cudaLaunchKernelEx(&cfg, k_chol_blocked, n, s, g, flags, skip));
-      else PARO_CU(c, cudaLaunchKernelEx(&cfg, k_chol_cluster, n, s, g, flags, skip));
-      ++c->launches;
-      prof_end(c, "k_chol_cluster", ev);
+      if ((st = launch_chol_cluster(c, sh, n, s, g, flags, skip))) return st;
       if (defer) {  // the flag comes back without waiting; chol_check() reads it
         const std::string nm = "chol_flag_" + std::to_string(c->chol_pending.size());
         if ((st = d2h_async(c, nm.c_str(), flags, sizeof(int), nullptr))) return st;

@@ -164,7 +164,8 @@ struct Ctx {
   struct CholShape {  // launch shape of the cluster Cholesky for order n on device dev
     int n = -1, dev = -1, kind = 0, cls = 0, thr = 0;
     size_t smem = 0;
-  } chol_shape;
+  };
+  std::map<int, CholShape> chol_shapes;  // by order
   std::vector<std::string> chol_pending;  // pinned flags of deferred Cholesky breakdown checks
   bool have_inv_g2 = false;  // the 1/|G|^2 table of the Hartree solve is in the "inv_g2" workspace
   bool have_tw_half = false;  // the N3/2-point FP64 twiddles of the Hartree energy are in "tw64_half"

@@ -60,3 +60,20 @@ def test_nonfinite_rows_stay_visible():
     assert torch.isfinite(torch.view_as_real(out[[0, 2]])).all()
     with pytest.raises(paro.ParoError):
         ctx.orthonormalize(x)
+
+
+# orders around the blocked cluster kernel's limit and above it: 2 x 2 blocks, then blocks of blocks
+@pytest.mark.parametrize("n", [175, 193, 208, 300, 401])
+def test_orthonormalisation_by_blocks(n):
+    ctx, _, _, _ = _ctx(ecut=8.0, kb=False)
+    x = inputs.start_vectors(n, ctx.npw(), n) + 0.3 * inputs.start_vectors(1, ctx.npw(), 1)
+    y = ctx.orthonormalize(torch.from_numpy(x).cuda()).cpu().numpy()
+    low = np.linalg.cholesky(np.conj(x) @ x.T)
+    ref = np.linalg.solve(np.conj(low), x)
+    # both factorisations err by n eps kappa(S) at most, kappa about 1 + 0.3^2 n here
+    tol = 4 * n * 2.0 ** -52 * (1 + 0.09 * n)
+    assert np.linalg.norm(y - ref) <= tol * np.linalg.norm(ref)
+    bad = x.copy()
+    bad[n - 2] = 0  # its pivot is zero exactly, in whichever block it falls
+    with pytest.raises(paro.ParoError):
+        ctx.orthonormalize(torch.from_numpy(bad).cuda())
