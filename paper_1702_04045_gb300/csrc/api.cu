@@ -1222,7 +1222,7 @@ int paro_set_local_pp(paro_ctx* ctx, double Z, double rc, double A, double a) {
   int st = build_vloc(c);
   if (st) return st;
   c->have_pp = true;
-  c->e_ewald = ewald(c);
+  if ((st = ewald(c))) return st;
   if ((st = set_veff_device(c, c->d_vloc))) return st;
   return PARO_OK;
 }
@@ -1263,7 +1263,7 @@ int paro_set_positions(paro_ctx* ctx, const double* pos) {
   c->pos.assign(pos, pos + 3 * c->nat);
   if (c->have_pp) {
     if ((st = build_vloc(c))) return st;
-    c->e_ewald = ewald(c);
+    if ((st = ewald(c))) return st;
   }
   if (c->have_kb && (st = build_beta(c))) return st;
   if (v) {

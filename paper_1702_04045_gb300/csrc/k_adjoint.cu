@@ -22,10 +22,16 @@ __global__ void k_polarize(int npw, double ngrid, const cplx<T>* __restrict__ ps
                            cplx<T>* __restrict__ v) {
   const int b = blockIdx.y;
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  // the band's two factors (square roots and a division in FP64) once per CTA
+  __shared__ double s_s, s_cf;
+  if (threadIdx.x == 0) {
+    const double a2 = np2[b], b2 = nw2[b];
+    s_s = (a2 > 0.0 && b2 > 0.0) ? sqrt(a2 / b2) : 1.0;
+    s_cf = 1.0 / sqrt(4.0 * s_s * ngrid);
+  }
+  __syncthreads();
   if (g >= npw) return;
-  const double a2 = np2[b], b2 = nw2[b];
-  const double s = (a2 > 0.0 && b2 > 0.0) ? sqrt(a2 / b2) : 1.0;
-  const double cf = 1.0 / sqrt(4.0 * s * ngrid);
+  const double s = s_s, cf = s_cf;
   const size_t o = (size_t)b * npw + g;
   const cplx<T> p = psi[o], q = w[o];
   const double px = (double)p.x, py = (double)p.y, qx = s * (double)q.x, qy = s * (double)q.y;
@@ -37,33 +43,49 @@ struct Rec3 {
   double m[9];
 };
 
-// Y[b][g] = (k + G_g)_a X[b][g]
+// Y[a nb + b][g] = (k + G_g)_a X[b][g] for the three directions; a thread takes one plane wave of 16 bands, its
+// q in FP64 once. The FP32 product is x q_hi + x q_lo with q split into two floats: the FP64 product's rounding.
+static const int kQBands = 16;
 template <typename T>
-__global__ void k_scale_q(int npw, const int* __restrict__ miller, Rec3 B, double ka, int al,
+__global__ void k_scale_q(int npw, int nb, const int* __restrict__ miller, Rec3 B, double kx, double ky, double kz,
                           const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Y) {
-  const int b = blockIdx.y;
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= npw) return;
-  const double q = ka + miller[3 * g] * B.m[al] + miller[3 * g + 1] * B.m[3 + al] + miller[3 * g + 2] * B.m[6 + al];
-  const size_t o = (size_t)b * npw + g;
-  const cplx<T> x = X[o];
-  Y[o] = mk<T>((T)(q * (double)x.x), (T)(q * (double)x.y));
+  const int n1 = miller[3 * g], n2 = miller[3 * g + 1], n3 = miller[3 * g + 2];
+  const double k[3] = {kx, ky, kz};
+  double q[3];
+#pragma unroll
+  for (int al = 0; al < 3; ++al) q[al] = k[al] + n1 * B.m[al] + n2 * B.m[3 + al] + n3 * B.m[6 + al];
+  const int b1 = min(nb, (int)(blockIdx.y + 1) * kQBands);
+  const size_t step = (size_t)nb * npw;
+  for (int b = blockIdx.y * kQBands; b < b1; ++b) {
+    const size_t o = (size_t)b * npw + g;
+    const cplx<T> x = X[o];
+#pragma unroll
+    for (int al = 0; al < 3; ++al) {
+      if constexpr (sizeof(T) == 4) {
+        const float qh = (float)q[al], ql = (float)(q[al] - (double)qh);
+        Y[al * step + o] = make_float2(fmaf(qh, x.x, ql * x.x), fmaf(qh, x.y, ql * x.y));
+      } else {
+        Y[al * step + o] = make_double2(q[al] * x.x, q[al] * x.y);
+      }
+    }
+  }
 }
 
 // gpos[I][a] += sum_{p in I} D_p sum_b Re[i (conj(A) P^a - conj(A^a) P)] = -sum D_p sum_b Im(...)
-// P, A, Pa[a], Aa[a]: nproj x nb complex (row p, ld nb). One CTA per atom.
-__global__ void __launch_bounds__(256) k_kb_force(int nb, const double2* __restrict__ P,
-                                                  const double2* __restrict__ A, const double2* __restrict__ Pa,
-                                                  const double2* __restrict__ Aa, size_t stride,
-                                                  const double* __restrict__ dvec, double* __restrict__ gpos) {
+// P, A: nproj x nb complex (row p); Q: nproj x 6 nb, columns [P^x P^y P^z A^x A^y A^z]. One CTA per atom.
+__global__ void __launch_bounds__(256) k_kb_force(int nb, const double2* __restrict__ P, const double2* __restrict__ A,
+                                                  const double2* __restrict__ Q, const double* __restrict__ dvec,
+                                                  double* __restrict__ gpos) {
   __shared__ double red[32];
   const int I = blockIdx.x;
   for (int al = 0; al < 3; ++al) {
     double acc = 0.0;
     for (int t = threadIdx.x; t < 4 * nb; t += blockDim.x) {
       const int p = 4 * I + t / nb, b = t % nb;
-      const size_t o = (size_t)p * nb + b;
-      const double2 a = A[o], pp = P[o], pa = Pa[al * stride + o], aa = Aa[al * stride + o];
+      const double2 a = A[(size_t)p * nb + b], pp = P[(size_t)p * nb + b];
+      const double2 pa = Q[(size_t)p * 6 * nb + al * nb + b], aa = Q[(size_t)p * 6 * nb + (3 + al) * nb + b];
       // Im(conj(a) pa - conj(aa) pp)
       const double im = (a.x * pa.y - a.y * pa.x) - (aa.x * pp.y - aa.y * pp.x);
       acc -= dvec[p] * im;
@@ -72,10 +94,6 @@ __global__ void __launch_bounds__(256) k_kb_force(int nb, const double2* __restr
     if (threadIdx.x == 0) gpos[3 * I + al] += acc;
   }
 }
-
-template <typename T> static const cplx<T>* projectors(const Basis& b);
-template <> const double2* projectors<double>(const Basis& b) { return b.d_beta; }
-template <> const float2* projectors<float>(const Basis& b) { return b.d_beta32; }
 
 template <typename T>
 static int hpsi_adjoint(Ctx* c, int ik, int nb, const cplx<T>* psi, const cplx<T>* w, cplx<T>* gpsi, double* gv,
@@ -115,23 +133,22 @@ static int hpsi_adjoint(Ctx* c, int ik, int nb, const cplx<T>* psi, const cplx<T
   const int np = c->nproj;
   const size_t mat = (size_t)np * nb;
   double2* M = static_cast<double2*>(ws_get(c, "adj_proj", 8 * mat * sizeof(double2)));
-  cplx<T>* Y = static_cast<cplx<T>*>(ws_get(c, f64 ? "adj_y64" : "adj_y32", (size_t)nb * npw * sizeof(cplx<T>)));
+  cplx<T>* Y = static_cast<cplx<T>*>(ws_get(c, f64 ? "adj_y64" : "adj_y32", (size_t)6 * nb * npw * sizeof(cplx<T>)));
   if (!M || !Y) return PARO_ERR_CUDA;
-  double2 *P = M, *A = M + mat, *Pa = M + 2 * mat, *Aa = M + 5 * mat;
-  const cplx<T>* beta = projectors<T>(B);
-  if ((st = gemm_cn<T, T, T>(c, np, nb, npw, beta, npw, psi, npw, P, nb, false, false))) return st;
-  if ((st = gemm_cn<T, T, T>(c, np, nb, npw, beta, npw, w, npw, A, nb, false, false))) return st;
+  double2 *P = M, *A = M + mat, *Q = M + 2 * mat;
   Rec3 R;
   for (int i = 0; i < 9; ++i) R.m[i] = c->bmat[i];
-  for (int al = 0; al < 3; ++al) {
-    k_scale_q<T><<<dim3((npw + 255) / 256, nb), 256, 0, c->stream>>>(npw, B.d_miller, R, B.kcart[al], al, psi, Y);
+  const dim3 gq((npw + 255) / 256, (nb + kQBands - 1) / kQBands);
+  for (int h = 0; h < 2; ++h) {
+    k_scale_q<T><<<gq, 256, 0, c->stream>>>(npw, nb, B.d_miller, R, B.kcart[0], B.kcart[1], B.kcart[2], h ? w : psi,
+                                            Y + (size_t)3 * h * nb * npw);
     PARO_LAUNCH(c, "k_scale_q");
-    if ((st = gemm_cn<T, T, T>(c, np, nb, npw, beta, npw, Y, npw, Pa + al * mat, nb, false, false))) return st;
-    k_scale_q<T><<<dim3((npw + 255) / 256, nb), 256, 0, c->stream>>>(npw, B.d_miller, R, B.kcart[al], al, w, Y);
-    PARO_LAUNCH(c, "k_scale_q");
-    if ((st = gemm_cn<T, T, T>(c, np, nb, npw, beta, npw, Y, npw, Aa + al * mat, nb, false, false))) return st;
   }
-  k_kb_force<<<c->nat, 256, 0, c->stream>>>(nb, P, A, Pa, Aa, mat, c->d_dvec, gpos);
+  // the projections of psi, w and of the six weighted blocks: three products with the projectors' images
+  if ((st = kb_project<T>(c, ik, nb, psi, P)) || (st = kb_project<T>(c, ik, nb, w, A)) ||
+      (st = kb_project<T>(c, ik, 6 * nb, Y, Q, nb)))
+    return st;
+  k_kb_force<<<c->nat, 256, 0, c->stream>>>(nb, P, A, Q, c->d_dvec, gpos);
   PARO_LAUNCH(c, "k_kb_force");
   return PARO_OK;
 }

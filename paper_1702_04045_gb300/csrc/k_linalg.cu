@@ -293,17 +293,6 @@ template <typename TA, typename TB, typename ACC>
 int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb, double2* C,
             int ldc, bool herm, bool carry) {
   if (M <= 0 || N <= 0) return PARO_OK;
-  if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4 && sizeof(ACC) == 4) {
-    if (!herm && !carry && K > 0 && c->tc_scope && tc_enabled()) {
-      int* err = tc_err_flag(c);
-      if (!err) return PARO_ERR_CUDA;
-      cudaEvent_t ev = prof_begin(c);
-      int st = gemm_cn_tc(c, M, N, K, A, lda, B, ldb, C, ldc, err);
-      if (st) return st;
-      prof_end(c, "k_gemm_cn_tc", ev);
-      return PARO_OK;
-    }
-  }
   if constexpr (sizeof(TA) == 8 && sizeof(TB) == 8) {
     // at every size the digit slices are faster than the FP64 pipe (Gram and V_nl of one 1189-coefficient row: 335 -> 85 us and 367 -> 70 us with the
     // steps around them; 144 rows of 23847: 8.8 -> 0.81 ms and 17.7 -> 0.68 ms)
@@ -560,15 +549,6 @@ int gemm_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, con
             int ldx, cplx<TY>* Y, int ldy, double beta, float2* wf, bool lower) {
   if (M <= 0 || N <= 0) return PARO_OK;
   if constexpr (sizeof(TX) == 4 && sizeof(TY) == 4) {
-    if (c->tc_scope && tc_enabled()) {
-      int* err = tc_err_flag(c);
-      if (!err) return PARO_ERR_CUDA;
-      cudaEvent_t ev = prof_begin(c);
-      int st = gemm_wx_tc(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta, err);
-      if (st) return st;
-      prof_end(c, "k_gemm_wx_tc", ev);
-      return PARO_OK;
-    }
     cudaEvent_t ev = prof_begin(c);
     int st = launch_wx32(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta, wf, lower);
     if (st) return st;
@@ -1068,6 +1048,26 @@ __global__ void __launch_bounds__(1024) k_orth_first_order(int n, const double2*
                  : k == r ? make_double2(1.5 - 0.5 * v.x, 0.0)
                           : make_double2(__longlong_as_double(__double_as_longlong(v.x) ^ (long long)0x8000000000000000ULL),
                                          v.y);
+  }
+}
+
+int chol_cluster_available(Ctx* c, int n, bool* avail) {
+  Ctx::CholShape sh;
+  const int st = chol_cluster_shape(c, n, &sh);
+  *avail = st == PARO_OK && sh.kind > 0;
+  return st;
+}
+
+int orth_first_order(Ctx* c, int n, const double2* s, double2* g, double tol, int** use_dev) {
+  int* use = static_cast<int*>(ws_get(c, "orth_first_use", sizeof(int)));
+  double* enorm = static_cast<double*>(ws_get(c, "orth_first_enorm", sizeof(double)));
+  if (!use || !enorm) return PARO_ERR_CUDA;
+  k_orth_first_order<<<16, 1024, 0, c->stream>>>(n, s, g, tol, use, enorm);
+  PARO_LAUNCH(c, "k_orth_first_order");
+  *use_dev = use;
+  return PARO_OK;
+}
+
 // C[i][j] = D[i][j] + sign sum_k a(i, k) b(k, j), complex FP64, for the small blocks of chol_split: a = A[i lda + k]
 // (conjugated with CA), b = B[j ldb + k] (TB) or B[k ldb + j] (conjugated with CB); D may be null. 8 x 16 outputs per
 // CTA with the K range in four parts, so a 144^3 product is 162 CTAs of FP64 work.
@@ -1204,11 +1204,11 @@ static int chol_piece(Ctx* c, int* piece) {
   return PARO_OK;
 }
 
-  }
-}
-
-int chol_cluster_available(Ctx* c, int n, bool* avail) {
-  Ctx::CholShape sh;
+int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int* skip) {
+  {
+    Ctx::CholShape sh;
+    int st;
+    if ((st = chol_cluster_shape(c, n, &sh))) return st;
     if (sh.kind != 1 && !defer && !skip && !c->plain64) {
       int piece = 0, nflag = 0;
       if ((st = chol_piece(c, &piece))) return st;
@@ -1231,26 +1231,6 @@ int chol_cluster_available(Ctx* c, int n, bool* avail) {
       }
       if ((st = chol_cluster_shape(c, n, &sh))) return st;
     }
-  const int st = chol_cluster_shape(c, n, &sh);
-  *avail = st == PARO_OK && sh.kind > 0;
-  return st;
-}
-
-int orth_first_order(Ctx* c, int n, const double2* s, double2* g, double tol, int** use_dev) {
-  int* use = static_cast<int*>(ws_get(c, "orth_first_use", sizeof(int)));
-  double* enorm = static_cast<double*>(ws_get(c, "orth_first_enorm", sizeof(double)));
-  if (!use || !enorm) return PARO_ERR_CUDA;
-  k_orth_first_order<<<16, 1024, 0, c->stream>>>(n, s, g, tol, use, enorm);
-  PARO_LAUNCH(c, "k_orth_first_order");
-  *use_dev = use;
-  return PARO_OK;
-}
-
-int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int* skip) {
-  {
-    Ctx::CholShape sh;
-    int st;
-    if ((st = chol_cluster_shape(c, n, &sh))) return st;
     if (sh.kind > 0) {
       int* flags = static_cast<int*>(ws_get(c, "chol_flags", 8 * sizeof(int)));
       if (!flags) return PARO_ERR_CUDA;

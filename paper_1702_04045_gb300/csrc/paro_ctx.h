@@ -106,7 +106,9 @@ struct Ctx {
   double vmean = 0, vmin = 0;
   std::vector<double> sigma_k;
   bool vstats_pending = false;
-  double e_ewald = 0;
+  // Ewald energy: its sums are read back behind an event, ewald_value() completes them
+  double e_ewald = 0, ewald_const = 0, ewald_real_scale = 0, ewald_rec_scale = 0;
+  bool ewald_pending = false;
   // SCF state
   double* d_rho_in = nullptr;
   bool have_rho = false;
@@ -260,12 +262,6 @@ int gemm_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, con
 template <typename TA, typename TB, typename ACC>
 int gemm_cn_scratch(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb,
                     double2* C, int ldc, double2* part, size_t part_elems);
-// Tensor-core (tcgen05, 3xTF32) C = conj(A) B^T for gemm_cn<float, float, float> (k_tc.cu); err: time-out flag.
-int gemm_cn_tc(Ctx* c, int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, double2* C,
-               int ldc, int* err);
-// Tensor-core gemm_wx<float, float> (k_tc.cu): Y = beta Y + sum_k s_k W(k, m) X[k].
-int gemm_wx_tc(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const float2* X,
-               int ldx, float2* Y, int ldy, double beta, int* err);
 // Tensor-core paths enabled (not when PARO_NO_TC is set in the environment), and their sticky error flag.
 bool tc_enabled();
 int* tc_err_flag(Ctx* c);
@@ -389,7 +385,8 @@ int energy_terms(Ctx* c, const double* rho_dev, double terms[7]);
 int pulay_mix(Ctx* c, const double* rho_out, int depth, double beta);
 template <typename T>
 int fft3d(Ctx* c, cplx<T>* data, bool inverse);  // in place, unnormalised, C order grid
-double ewald(const Ctx* c);
+int ewald(Ctx* c);
+int ewald_value(Ctx* c, double* e);
 
 int build_twiddles(Ctx* c);
 // radix plan (2, 3, 4, 8) of an FFT of length n (n = 2^a 3^b)
