@@ -247,8 +247,9 @@ int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* p
  *   of every problem must fit one CTA's shared memory (N1 x N2 complex elements of the working precision
  *   within 227 KB; otherwise PARO_ERR_ARG). The call times, on the batch's own problems, the unit shapes
  *   (32, 64 or 128 sticks per z-FFT unit; planes per unit for about 2048, 4096 or 8192 points), the launch
- *   forms (one cooperative launch with grid barriers between the phases, or one launch per phase) and the
- *   grids, and keeps the fastest (paro_batch_tuning). The batch refers to the contexts, which must
+ *   forms (one cooperative launch with grid barriers between the phases, or one launch per phase and
+ *   grid, with the line FFTs in registers on cubic grids of 27 to 72 points) and the grids, and keeps the
+ *   fastest (paro_batch_tuning). The batch refers to the contexts, which must
  *   outlive it.
  * paro_batch_apply_h -- H psi of every problem: psi[i], hpsi[i] device n_bands x npw arrays of dtype
  *   (the contexts' precision: PARO_C64 for FP64, PARO_C32 for mixed) of problem i. Enqueued on the
@@ -261,7 +262,8 @@ int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* p
  *   receives the largest occupied residual. Every context needs orbitals (paro_set_orbitals) first.
  *   Errors: PARO_ERR_BREAKDOWN (PCG or Cholesky), PARO_ERR_NOT_CONVERGED (Jacobi), PARO_ERR_TIMEOUT (a
  *   bounded grid-barrier wait gave up).
- * paro_batch_info -- problems, (problem, band) items, H psi launches per apply (1 or 3), its grid, and
+ * paro_batch_info -- problems, (problem, band) items, H psi launches per apply (1, or 3 for the form with
+ *   launches per phase), its grid, and
  *   kernels launched per captured step (0 before the first step).
  */
 typedef struct paro_batch paro_batch;

@@ -199,17 +199,20 @@ template <bool INV> struct TDft<18, INV> {
 };
 
 // ---- line shapes ----
+// Few values a lane keep the fixed-point kernels below 128 registers: 54 = 9 x 6 took 1.22 ms a plane pass of 144
+// orbitals where 18 x 3 (255 registers) took 3.03, 36 = 6 x 6 52 us (23 orbitals) where 12 x 3 took 71, 96 = 12 x 8
+// 3.3 ms (60 orbitals) where 16 x 6 took 3.7; 72 = 8 x 9 was no better than 12 x 6 (2.07 and 1.97 ms, 144 orbitals).
 template <int N> struct TileShape;
 template <> struct TileShape<27> { static constexpr int Q = 9, P = 3; };
 template <> struct TileShape<32> { static constexpr int Q = 8, P = 4; };
-template <> struct TileShape<36> { static constexpr int Q = 12, P = 3; };
+template <> struct TileShape<36> { static constexpr int Q = 6, P = 6; };
 template <> struct TileShape<48> { static constexpr int Q = 12, P = 4; };
-template <> struct TileShape<54> { static constexpr int Q = 18, P = 3; };
+template <> struct TileShape<54> { static constexpr int Q = 9, P = 6; };
 template <> struct TileShape<64> { static constexpr int Q = 8, P = 8; };
 template <> struct TileShape<72> { static constexpr int Q = 12, P = 6; };
 template <> struct TileShape<81> { static constexpr int Q = 9, P = 9; };
-template <> struct TileShape<96> { static constexpr int Q = 16, P = 6; };
-template <> struct TileShape<108> { static constexpr int Q = 18, P = 6; };
+template <> struct TileShape<96> { static constexpr int Q = 12, P = 8; };
+template <> struct TileShape<108> { static constexpr int Q = 12, P = 9; };
 
 template <int N> struct TileLine {
   static constexpr int Q = TileShape<N>::Q, P = TileShape<N>::P;

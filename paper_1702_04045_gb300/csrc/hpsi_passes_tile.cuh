@@ -8,10 +8,30 @@
 
 namespace paro {
 
-// warps of a plane CTA: one or two rounds of the N lines along x
+// warps of a plane CTA: one to three rounds of the N lines along x; twelve on the grids whose plane leaves room for
+// one CTA an SM
 template <int N> struct TileWarps {
   static constexpr int kRounds = (N + TileLine<N>::G - 1) / TileLine<N>::G;
-  static constexpr int value = kRounds <= 8 ? kRounds : kRounds <= 16 ? (kRounds + 1) / 2 : (kRounds + 2) / 3;
+  static constexpr int value = N >= 96 ? 12 : kRounds <= 8 ? kRounds : kRounds <= 16 ? (kRounds + 1) / 2 : (kRounds + 2) / 3;
+};
+// Resident plane CTAs the fixed-point kernels are compiled for (a register cap of 65536 / (CTAs x threads)), each
+// measured: uncapped, 72 points took 211 registers, eight warps an SM and 3.30 ms for 144 orbitals, with two CTAs
+// 1.97 ms; 64 points 1.43 -> 0.83 ms with three, 36 points 102 -> 49 us (23 orbitals), 32 points 38 -> 27 us (20 orbitals),
+// 81 points 2.12 -> 1.70 ms (60 orbitals).
+template <int N> struct TileCtas { static constexpr int value = 1; };
+template <> struct TileCtas<27> { static constexpr int value = 5; };
+template <> struct TileCtas<32> { static constexpr int value = 5; };
+template <> struct TileCtas<36> { static constexpr int value = 3; };
+template <> struct TileCtas<48> { static constexpr int value = 2; };
+template <> struct TileCtas<54> { static constexpr int value = 2; };
+template <> struct TileCtas<64> { static constexpr int value = 3; };
+template <> struct TileCtas<72> { static constexpr int value = 2; };
+template <> struct TileCtas<81> { static constexpr int value = 2; };
+template <typename NT, int N> struct TileMinBlocks {
+  // FP32: 32 warps an SM (64 registers): 81 points 462 -> 322 us (100 orbitals), 54 points 186 -> 151 us (144), a mesh of
+  // 27 problems on 32 points 181 -> 157 us; 24 and 40 warps were within a tenth of it
+  static constexpr int kF32 = 32 / TileWarps<N>::value;
+  static constexpr int value = NT::kFixed ? TileCtas<N>::value : kF32 < 1 ? 1 : kF32;
 };
 template <int N> struct TileStride { static constexpr int value = N | 1; };
 
@@ -28,28 +48,24 @@ template <int N> struct TileLane {
   }
 };
 
+// sticks c0 .. c0 + CB - 1 of one band: scatter, inverse transform along z, into the band's stick buffer Sb
 template <typename NT, int N>
-__global__ void __launch_bounds__(256) k_zinv_tile(const typename NT::S* __restrict__ psi, int ldpsi,
-                                                   typename NT::S* __restrict__ S, const int* __restrict__ col_off,
-                                                   const int* __restrict__ g_col, const int* __restrict__ g_z,
-                                                   int ncol, const typename NT::W* __restrict__ twz,
-                                                   const int* __restrict__ active, int CB) {
+__device__ __forceinline__ void zinv_sticks(unsigned char* smem_raw, const typename NT::S* __restrict__ pp,
+                                            typename NT::S* __restrict__ Sb, const int* __restrict__ col_off,
+                                            const int* __restrict__ g_col, const int* __restrict__ g_z, int ncol,
+                                            const typename NT::W* __restrict__ twz, int c0, int CB) {
   using L = TileLine<N>;
   using ST = typename NT::S;
   using C = typename NT::C;
   constexpr int LS = TileStride<N>::value;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tiles = reinterpret_cast<C*>(smem_raw);
   ST* line = reinterpret_cast<ST*>(tiles + (blockDim.x >> 5) * L::WTILE);
-  const int b = blockIdx.y;
-  if (active != nullptr && active[b] == 0) return;
-  const int c0 = blockIdx.x * CB, ncb = min(CB, ncol - c0);
+  const int ncb = min(CB, ncol - c0);
   ST zero;
   zero.x = zero.y = 0;
   for (int i = threadIdx.x; i < ncb * LS; i += blockDim.x) line[i] = zero;
   __syncthreads();
   const int g0 = col_off[c0], g1 = col_off[c0 + ncb];
-  const ST* pp = psi + (size_t)b * ldpsi;
   for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x) line[(g_col[g] - c0) * LS + g_z[g]] = pp[g];
   __syncthreads();
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -73,12 +89,24 @@ __global__ void __launch_bounds__(256) k_zinv_tile(const typename NT::S* __restr
       }
   }
   __syncthreads();
-  ST* Sb = S + (size_t)b * N * ncol;
   const int sh = 31 - __clz(CB);  // CB is a power of two
   for (int i = threadIdx.x; i < N << sh; i += blockDim.x) {
     const int z = i >> sh, cc = i & (CB - 1);
     if (cc < ncb) Sb[(size_t)z * ncol + c0 + cc] = line[cc * LS + z];
   }
+}
+
+template <typename NT, int N>
+__global__ void __launch_bounds__(256) k_zinv_tile(const typename NT::S* __restrict__ psi, int ldpsi,
+                                                   typename NT::S* __restrict__ S, const int* __restrict__ col_off,
+                                                   const int* __restrict__ g_col, const int* __restrict__ g_z,
+                                                   int ncol, const typename NT::W* __restrict__ twz,
+                                                   const int* __restrict__ active, int CB) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int b = blockIdx.y;
+  if (active != nullptr && active[b] == 0) return;
+  zinv_sticks<NT, N>(smem_raw, psi + (size_t)b * ldpsi, S + (size_t)b * N * ncol, col_off, g_col, g_z, ncol, twz,
+                     blockIdx.x * CB, CB);
 }
 
 // inverse along y of the plane's stick rows, from the stick buffer into the compact plane
@@ -125,13 +153,12 @@ __device__ __forceinline__ void tile_times_v(typename NT::C* v, const typename N
                                              int base, FxScale& sc) {
   using L = TileLine<N>;
   if constexpr (NT::kFixed) {
-    double vv[L::V];
+    // the potential is read twice, for its exponent and for the product, rather than held beside the line
     int key = 0;
 #pragma unroll
     for (int i = 0; i < L::V; ++i) {
       const int k = tile_index<N>(p, i);
-      vv[i] = ok && k >= 0 ? Vc[k * N] : 0.0;
-      key = max(key, __double2hiint(vv[i]) & 0x7fffffff);
+      if (ok && k >= 0) key = max(key, __double2hiint(Vc[k * N]) & 0x7fffffff);
     }
     key = tile_max<L::P>(key, base);
     const int ex = key >> 20, e = max(ex, 1) - 1022;
@@ -139,7 +166,8 @@ __device__ __forceinline__ void tile_times_v(typename NT::C* v, const typename N
     tile_normalise<NT, N, 61>(v, p, sc, base);
 #pragma unroll
     for (int i = 0; i < L::V; ++i) {
-      const FxSplit w = fx_cut(fx_from<62>(vv[i], e));
+      const int k = tile_index<N>(p, i);
+      const FxSplit w = fx_cut(ok && k >= 0 ? fx_from<62>(Vc[k * N], e) : 0);
       v[i] = fxc{fx_mul(fx_cut(v[i].x), w), fx_mul(fx_cut(v[i].y), w)};
     }
     sc.k += e;
@@ -153,27 +181,24 @@ __device__ __forceinline__ void tile_times_v(typename NT::C* v, const typename N
   }
 }
 
+// one plane of one band: sticks Sz in and out, V its potential plane
 template <typename NT, int N>
-__global__ void __launch_bounds__(32 * TileWarps<N>::value)
-    k_plane_tile(typename NT::S* __restrict__ S, int ncol, const int* __restrict__ stick_of,
-                 const int* __restrict__ xrow_c, int nxr, const typename NT::W* __restrict__ twx,
-                 const typename NT::W* __restrict__ twy, const typename NT::R* __restrict__ vplane,
-                 const int* __restrict__ active) {
+__device__ __forceinline__ void plane_sticks(unsigned char* smem_raw, typename NT::S* __restrict__ Sz,
+                                             const int* __restrict__ stick_of, const int* __restrict__ xrow_c, int nxr,
+                                             const typename NT::W* __restrict__ twx,
+                                             const typename NT::W* __restrict__ twy,
+                                             const typename NT::R* __restrict__ V) {
   using L = TileLine<N>;
   using ST = typename NT::S;
   using C = typename NT::C;
   constexpr int LS = TileStride<N>::value;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tiles = reinterpret_cast<C*>(smem_raw);
   ST* Pl = reinterpret_cast<ST*>(tiles + (blockDim.x >> 5) * L::WTILE);
   int* roff = reinterpret_cast<int*>(Pl + (size_t)nxr * LS);
-  const int z = blockIdx.x, b = blockIdx.y;
-  if (active != nullptr && active[b] == 0) return;
   for (int i = threadIdx.x; i < N; i += blockDim.x) {
     const int r = xrow_c[i];
     roff[i] = r >= 0 ? r * LS : -1;
   }
-  ST* Sz = S + ((size_t)b * N + z) * ncol;
   tile_rows_inv<NT, N>(Sz, stick_of, nxr, twy, tiles, Pl);
   __syncthreads();
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -181,7 +206,6 @@ __global__ void __launch_bounds__(32 * TileWarps<N>::value)
   C* tile = tiles + warp * L::WTILE + t.grp * L::TILE;
   ST zero;
   zero.x = zero.y = 0;
-  const typename NT::R* V = vplane + (size_t)z * N * N;
   for (int c0 = warp * L::G; c0 < N; c0 += nw * L::G) {  // along x: inverse, times V / N_grid, forward
     const int y = c0 + t.grp;
     const bool ok = t.ok && y < N;
@@ -244,27 +268,37 @@ __global__ void __launch_bounds__(32 * TileWarps<N>::value)
   }
 }
 
-// ACC: hpsi += the transformed potential term alone (no kinetic or shift term)
-template <typename NT, int N, bool ACC>
-__global__ void __launch_bounds__(256) k_zfwd_tile(const typename NT::S* __restrict__ S,
-                                                   const typename NT::S* __restrict__ psi, int ldpsi,
-                                                   typename NT::S* __restrict__ hpsi, int ldh,
-                                                   const typename NT::R* __restrict__ kin, typename NT::R shift,
-                                                   const int* __restrict__ col_off, const int* __restrict__ g_col,
-                                                   const int* __restrict__ g_z, int ncol,
-                                                   const typename NT::W* __restrict__ twz,
-                                                   const int* __restrict__ active, int CB) {
+template <typename NT, int N>
+__global__ void __launch_bounds__(32 * TileWarps<N>::value, TileMinBlocks<NT, N>::value)
+    k_plane_tile(typename NT::S* __restrict__ S, int ncol, const int* __restrict__ stick_of,
+                 const int* __restrict__ xrow_c, int nxr, const typename NT::W* __restrict__ twx,
+                 const typename NT::W* __restrict__ twy, const typename NT::R* __restrict__ vplane,
+                 const int* __restrict__ active) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int z = blockIdx.x, b = blockIdx.y;
+  if (active != nullptr && active[b] == 0) return;
+  plane_sticks<NT, N>(smem_raw, S + ((size_t)b * N + z) * ncol, stick_of, xrow_c, nxr, twx, twy,
+                      vplane + (size_t)z * N * N);
+}
+
+// sticks c0 .. of one band: forward transform along z, gather, kinetic term and shift; ACC: h += the transformed
+// potential term alone; KB: the projector term sum_j beta_j(G) dp_j as well (batches)
+template <typename NT, int N, bool ACC, bool KB>
+__device__ __forceinline__ void zfwd_sticks(unsigned char* smem_raw, const typename NT::S* __restrict__ Sb,
+                                            const typename NT::S* pp, typename NT::S* h,
+                                            const typename NT::R* __restrict__ kin, typename NT::R shift,
+                                            const int* __restrict__ col_off, const int* __restrict__ g_col,
+                                            const int* __restrict__ g_z, int ncol,
+                                            const typename NT::W* __restrict__ twz, int c0, int CB, int np = 0, int npw = 0,
+                                            const typename NT::S* __restrict__ beta = nullptr,
+                                            const typename NT::S* __restrict__ dp = nullptr) {
   using L = TileLine<N>;
   using ST = typename NT::S;
   using C = typename NT::C;
   constexpr int LS = TileStride<N>::value;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tiles = reinterpret_cast<C*>(smem_raw);
   ST* line = reinterpret_cast<ST*>(tiles + (blockDim.x >> 5) * L::WTILE);
-  const int b = blockIdx.y;
-  if (active != nullptr && active[b] == 0) return;
-  const int c0 = blockIdx.x * CB, ncb = min(CB, ncol - c0);
-  const ST* Sb = S + (size_t)b * N * ncol;
+  const int ncb = min(CB, ncol - c0);
   const int sh = 31 - __clz(CB);  // CB is a power of two
   for (int i = threadIdx.x; i < N << sh; i += blockDim.x) {
     const int z = i >> sh, cc = i & (CB - 1);
@@ -312,8 +346,6 @@ __global__ void __launch_bounds__(256) k_zfwd_tile(const typename NT::S* __restr
   }
   __syncthreads();
   const int g0 = col_off[c0], g1 = col_off[c0 + ncb];
-  const ST* pp = psi + (size_t)b * ldpsi;
-  ST* h = hpsi + (size_t)b * ldh;
   for (int g = g0 + threadIdx.x; g < g1; g += blockDim.x) {
     const ST v = line[(g_col[g] - c0) * LS + g_z[g]];
     if (ACC) {
@@ -324,9 +356,31 @@ __global__ void __launch_bounds__(256) k_zfwd_tile(const typename NT::S* __restr
       ST o;
       o.x = v.x + tk * cc.x;
       o.y = v.y + tk * cc.y;
+      if constexpr (KB)
+        for (int j = 0; j < np; ++j) {
+          const ST bv = beta[(size_t)j * npw + g], d = dp[j];
+          o.x += bv.x * d.x - bv.y * d.y;
+          o.y += bv.x * d.y + bv.y * d.x;
+        }
       h[g] = o;
     }
   }
+}
+
+template <typename NT, int N, bool ACC>
+__global__ void __launch_bounds__(256) k_zfwd_tile(const typename NT::S* __restrict__ S,
+                                                   const typename NT::S* __restrict__ psi, int ldpsi,
+                                                   typename NT::S* __restrict__ hpsi, int ldh,
+                                                   const typename NT::R* __restrict__ kin, typename NT::R shift,
+                                                   const int* __restrict__ col_off, const int* __restrict__ g_col,
+                                                   const int* __restrict__ g_z, int ncol,
+                                                   const typename NT::W* __restrict__ twz,
+                                                   const int* __restrict__ active, int CB) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int b = blockIdx.y;
+  if (active != nullptr && active[b] == 0) return;
+  zfwd_sticks<NT, N, ACC, false>(smem_raw, S + (size_t)b * N * ncol, psi + (size_t)b * ldpsi, hpsi + (size_t)b * ldh, kin,
+                                 shift, col_off, g_col, g_z, ncol, twz, blockIdx.x * CB, CB);
 }
 
 // Density planes: per (z-plane, band group) the inverse transforms of each band, |psi(r)|^2 summed in FP64

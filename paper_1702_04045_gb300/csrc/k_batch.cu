@@ -24,6 +24,7 @@
 #include <string>
 #include <vector>
 
+#include "batch_prob.cuh"
 #include "jacobi_small.cuh"
 #include "paro_ctx.h"
 
@@ -32,40 +33,6 @@ namespace paro {
 static const int kBMaxBands = 64;
 static const int kBChunk = 1024;  // plane waves per CTA in the batched vector kernels
 static const int kBSlice = 512;   // K slice of the batched Gram / H_sub products
-
-// Per problem (one k-point of one context), device-visible.
-struct ProbDev {
-  int npw, ncol, nxr, nb, N1, N2, N3, nproj;
-  long long off;   // first element of the problem's rows in the batch vectors
-  long long soff;  // first element of the problem's stick buffers (nb x N3 x ncol)
-  long long dpoff; // first element of the problem's scaled projections (nb x nproj)
-  int band0;       // first band of the problem in the flat band list
-  int pad;
-  FftPlan plan[3];
-  const int *col_x, *col_y, *col_off, *g_col, *g_z, *xrows;
-  const double* kin;
-  const float* kin32;
-  const double* vplane;
-  const float* vplane32;
-  const double2* tw64[3];
-  const float2* tw32[3];
-  const double2* beta;
-  const float2* beta32;
-  const double* dvec;
-};
-
-template <typename T> __device__ __forceinline__ const cplx<T>* pd_tw(const ProbDev& p, int a);
-template <> __device__ __forceinline__ const double2* pd_tw<double>(const ProbDev& p, int a) { return p.tw64[a]; }
-template <> __device__ __forceinline__ const float2* pd_tw<float>(const ProbDev& p, int a) { return p.tw32[a]; }
-template <typename T> __device__ __forceinline__ const T* pd_kin(const ProbDev& p);
-template <> __device__ __forceinline__ const double* pd_kin<double>(const ProbDev& p) { return p.kin; }
-template <> __device__ __forceinline__ const float* pd_kin<float>(const ProbDev& p) { return p.kin32; }
-template <typename T> __device__ __forceinline__ const T* pd_v(const ProbDev& p);
-template <> __device__ __forceinline__ const double* pd_v<double>(const ProbDev& p) { return p.vplane; }
-template <> __device__ __forceinline__ const float* pd_v<float>(const ProbDev& p) { return p.vplane32; }
-template <typename T> __device__ __forceinline__ const cplx<T>* pd_beta(const ProbDev& p);
-template <> __device__ __forceinline__ const double2* pd_beta<double>(const ProbDev& p) { return p.beta; }
-template <> __device__ __forceinline__ const float2* pd_beta<float>(const ProbDev& p) { return p.beta32; }
 
 // Work-unit shapes, chosen per batch by the autotuner: sg sticks per z-FFT unit, and z-planes per plane
 // unit enough that one unit's FFT stages cover about ppt points (at most 4 planes)
@@ -716,6 +683,11 @@ struct paro_batch {
   void *sbuf = nullptr, *dpbuf = nullptr;  // stick buffers and scaled projections of the H psi phases
   int2 *d_u1 = nullptr, *d_u2 = nullptr, *d_u3 = nullptr;
   int n1 = 0, n2 = 0, n3 = 0;
+  // the three-launch form: items on grids of the line-FFT passes by grid (k_tile_batch.cu), and the units left to
+  // the shared-memory passes (uncovered grids, and the projections of every item)
+  std::vector<BatchGroup> groups;
+  int2 *d_r1 = nullptr, *d_r2 = nullptr, *d_r3 = nullptr;
+  int r1 = 0, r2 = 0, r3 = 0;
   int sg = 64, ppt = 4096;         // work-unit shapes (autotuned)
   std::vector<int2> h_items;       // (problem, band) of every item, largest problems first
   std::vector<std::array<double, 5>> tuning;  // launches per apply, grid, sg, ppt, ms per apply
@@ -768,10 +740,11 @@ int berr(paro_batch* b, int code, const std::string& msg) {
 
 BandMap bandmap(const paro_batch* b) { return BandMap{b->d_bprob, b->d_brow, b->d_prob}; }
 
-// One H psi over every item: mode 0 = one cooperative launch of the three phases, mode 1 = three launches.
+// One H psi over every item: mode 0 = one cooperative launch of the three phases, mode 1 = a launch per phase
+// and grid. rows (mode 1, every item in a group and without projectors): the caller's own arrays.
 template <typename T>
 int launch_fused(paro_batch* b, cudaStream_t s, const cplx<T>* X, cplx<T>* Y, const int* active, int shifted,
-                 int mode, int grid) {
+                 int mode, int grid, const BatchRows<T>* rows = nullptr) {
   const HpsiLists L{b->d_u1, b->n1, b->d_u2, b->n2, b->d_u3, b->n3, b->sg, b->ppt};
   cplx<T>* S = static_cast<cplx<T>*>(b->sbuf);
   cplx<T>* DP = static_cast<cplx<T>*>(b->dpbuf);
@@ -792,15 +765,35 @@ int launch_fused(paro_batch* b, cudaStream_t s, const cplx<T>* X, cplx<T>* Y, co
     ++b->graph_kernels;
     return PARO_OK;
   }
-  k_hpsi_batch<T, 1><<<std::min(grid, b->n1), 256, b->smem, s>>>(b->d_prob, b->d_items, L, X, Y, S, DP, active,
-                                                                  b->sigma, shifted, b->d_bar, err);
-  BLAUNCH(b, "k_hpsi_batch<1>");
-  k_hpsi_batch<T, 2><<<std::min(grid, b->n2), 256, b->smem, s>>>(b->d_prob, b->d_items, L, X, Y, S, DP, active,
-                                                                  b->sigma, shifted, b->d_bar, err);
-  BLAUNCH(b, "k_hpsi_batch<2>");
-  k_hpsi_batch<T, 3><<<std::min(grid, b->n3), 256, b->smem, s>>>(b->d_prob, b->d_items, L, X, Y, S, DP, active,
-                                                                  b->sigma, shifted, b->d_bar, err);
-  BLAUNCH(b, "k_hpsi_batch<3>");
+  const HpsiLists R{b->d_r1, b->r1, b->d_r2, b->r2, b->d_r3, b->r3, b->sg, b->ppt};
+  BatchRows<T> own;
+  if (!rows) {
+    own.x = X;
+    own.y = Y;
+    own.direct = 0;
+    rows = &own;
+  }
+  for (int ph = 1; ph <= 3; ++ph) {
+    const int nr = ph == 1 ? b->r1 : ph == 2 ? b->r2 : b->r3;
+    if (nr > 0) {
+      const int gr = std::min(grid, nr);
+      if (ph == 1)
+        k_hpsi_batch<T, 1><<<gr, 256, b->smem, s>>>(b->d_prob, b->d_items, R, X, Y, S, DP, active, b->sigma, shifted,
+                                                    b->d_bar, err);
+      else if (ph == 2)
+        k_hpsi_batch<T, 2><<<gr, 256, b->smem, s>>>(b->d_prob, b->d_items, R, X, Y, S, DP, active, b->sigma, shifted,
+                                                    b->d_bar, err);
+      else
+        k_hpsi_batch<T, 3><<<gr, 256, b->smem, s>>>(b->d_prob, b->d_items, R, X, Y, S, DP, active, b->sigma, shifted,
+                                                    b->d_bar, err);
+      BLAUNCH(b, "k_hpsi_batch");
+    }
+    for (const BatchGroup& g : b->groups) {
+      if (int st = batch_tile_apply<T>(b->lead, s, g, b->d_prob, b->d_items, *rows, S, DP, active, b->sigma, shifted, ph))
+        return berr(b, st, "batch: " + b->lead->err);
+      ++b->graph_kernels;
+    }
+  }
   return PARO_OK;
 }
 
@@ -918,6 +911,63 @@ int enqueue_step(paro_batch* b, double tol, int maxit, bool carry_hx) {
   return PARO_OK;
 }
 
+// whether a problem's items go through the line-FFT passes (their grids index the items by blockIdx.y)
+bool line_covered(const paro_batch* b, const ProbDev& P) { return b->nitems <= 65535 && batch_tile_covers(P, b->f64); }
+
+// The passes can work on the caller's arrays themselves (54 device copies of a 27-problem mesh take longer than its
+// FFTs): every item in a line-FFT group, no projectors, every array aligned to its element, no input that
+// another problem's output overlaps (a problem's own output may be its input: a coefficient's two terms are read by
+// the thread that writes it).
+template <typename T>
+bool direct_ok(const paro_batch* b, const void* const* psi, void* const* hpsi) {
+  if (b->threads != 3 || b->groups.empty() || b->r1 > 0 || b->r2 > 0 || b->nprob > kBatchDirect) return false;
+  std::vector<std::pair<uintptr_t, uintptr_t>> in(b->nprob), out(b->nprob);
+  for (int i = 0; i < b->nprob; ++i) {
+    const uintptr_t n = (uintptr_t)b->hprob[i].nb * b->hprob[i].npw * sizeof(cplx<T>);
+    in[i] = {(uintptr_t)psi[i], (uintptr_t)psi[i] + n};
+    out[i] = {(uintptr_t)hpsi[i], (uintptr_t)hpsi[i] + n};
+    if (in[i].first % sizeof(cplx<T>) || out[i].first % sizeof(cplx<T>)) return false;
+  }
+  for (int i = 0; i < b->nprob; ++i)
+    for (int j = 0; j < b->nprob; ++j) {
+      if (i == j && in[i] == out[i]) continue;
+      if (in[i].first < out[j].second && out[j].first < in[i].second) return false;
+      if (i < j && out[i].first < out[j].second && out[j].first < out[i].second) return false;
+    }
+  return true;
+}
+
+template <typename T>
+int batch_apply(paro_batch* b, const void* const* psi, void* const* hpsi) {
+  cplx<T>*p = static_cast<cplx<T>*>(b->p), *ap = static_cast<cplx<T>*>(b->ap);
+  const int mode = b->threads == 1 ? 0 : 1;
+  int st;
+  if (direct_ok<T>(b, psi, hpsi)) {
+    BatchRows<T> rows;
+    rows.x = nullptr;
+    rows.y = nullptr;
+    rows.direct = 1;
+    for (int i = 0; i < b->nprob; ++i) {
+      rows.px[i] = static_cast<const cplx<T>*>(psi[i]);
+      rows.py[i] = static_cast<cplx<T>*>(hpsi[i]);
+    }
+    if ((st = launch_fused<T>(b, b->st, p, ap, nullptr, 0, mode, b->grid, &rows))) return st;
+    b->lead->launches += 3 * (long long)b->groups.size();
+    return PARO_OK;
+  }
+  for (int i = 0; i < b->nprob; ++i) {
+    const ProbDev& P = b->hprob[i];
+    BCU(b, cudaMemcpyAsync(p + P.off, psi[i], (size_t)P.nb * P.npw * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, b->st));
+  }
+  if ((st = launch_fused<T>(b, b->st, p, ap, nullptr, 0, mode, b->grid))) return st;
+  b->lead->launches += 1;
+  for (int i = 0; i < b->nprob; ++i) {
+    const ProbDev& P = b->hprob[i];
+    BCU(b, cudaMemcpyAsync(hpsi[i], ap + P.off, (size_t)P.nb * P.npw * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, b->st));
+  }
+  return PARO_OK;
+}
+
 // The three work lists for unit shapes (sg, ppt) on the device, and the shared memory they need (bytes).
 // Returns PARO_ERR_ARG (nothing changed) when a unit does not fit one CTA's shared memory.
 int build_lists(paro_batch* b, int sg, int ppt) {
@@ -925,7 +975,7 @@ int build_lists(paro_batch* b, int sg, int ppt) {
   size_t max_el = 0;
   for (const ProbDev& P : b->hprob) max_el = std::max(max_el, unit_elems(P, sg, ppt));
   if (max_el * es > 227 * 1024) return PARO_ERR_ARG;
-  std::vector<int2> u1, u2, u3;
+  std::vector<int2> u1, u2, u3, r1, r2, r3;
   for (int it = 0; it < (int)b->h_items.size(); ++it) {
     const ProbDev& P = b->hprob[b->h_items[it].x];
     const int ng = (P.ncol + sg - 1) / sg;
@@ -935,11 +985,18 @@ int build_lists(paro_batch* b, int sg, int ppt) {
       u3.push_back(make_int2(it, g));
     }
     for (int z = 0; z < P.N3; z += planes_per_unit(P.N1, P.N2, ppt)) u2.push_back(make_int2(it, z));
+    if (P.nproj > 0) r1.push_back(make_int2(it, -1));
+    if (line_covered(b, P)) continue;
+    for (int g = 0; g < ng; ++g) {
+      r1.push_back(make_int2(it, g));
+      r3.push_back(make_int2(it, g));
+    }
+    for (int z = 0; z < P.N3; z += planes_per_unit(P.N1, P.N2, ppt)) r2.push_back(make_int2(it, z));
   }
   BCU(b, cudaStreamSynchronize(b->st));
-  int2** dst[3] = {&b->d_u1, &b->d_u2, &b->d_u3};
-  const std::vector<int2>* src[3] = {&u1, &u2, &u3};
-  for (int i = 0; i < 3; ++i) {
+  int2** dst[6] = {&b->d_u1, &b->d_u2, &b->d_u3, &b->d_r1, &b->d_r2, &b->d_r3};
+  const std::vector<int2>* src[6] = {&u1, &u2, &u3, &r1, &r2, &r3};
+  for (int i = 0; i < 6; ++i) {
     if (*dst[i]) cudaFree(*dst[i]);
     *dst[i] = nullptr;
     BCU(b, cudaMalloc(dst[i], std::max<size_t>(src[i]->size(), 1) * sizeof(int2)));
@@ -948,6 +1005,9 @@ int build_lists(paro_batch* b, int sg, int ppt) {
   b->n1 = (int)u1.size();
   b->n2 = (int)u2.size();
   b->n3 = (int)u3.size();
+  b->r1 = (int)r1.size();
+  b->r2 = (int)r2.size();
+  b->r3 = (int)r3.size();
   b->sg = sg;
   b->ppt = ppt;
   b->smem = max_el * es;
@@ -1033,11 +1093,13 @@ void free_batch(paro_batch* b) {
   if (b->ev) cudaEventDestroy(b->ev);
   if (b->gst) cudaStreamDestroy(b->gst);
   void* bufs[] = {b->d_prob, b->d_items, b->d_bprob, b->d_brow, b->x, b->r, b->p, b->ap, b->rhs, b->y, b->hy, b->hx,
-                  b->sbuf, b->dpbuf, b->d_u1, b->d_u2, b->d_u3, b->d_bar,
+                  b->sbuf, b->dpbuf, b->d_u1, b->d_u2, b->d_u3, b->d_r1, b->d_r2, b->d_r3, b->d_bar,
                   b->psi64, b->hpsi64, b->prz, b->prr, b->rz, b->r0n, b->alpha, b->beta, b->active, b->still,
                   b->flags, b->part, b->S, b->G, b->eps, b->res, b->sigma, b->pshift};
   for (void* q : bufs)
     if (q) cudaFree(q);
+  for (BatchGroup& g : b->groups)
+    if (g.d_items) cudaFree(g.d_items);
   if (b->h_stage) cudaFreeHost(b->h_stage);
   if (b->h_flags) cudaFreeHost(b->h_flags);
   delete b;
@@ -1112,6 +1174,7 @@ int paro_batch_create(paro_batch** out, paro_ctx* const* ctxs, int n_ctx) {
         P.plan[a] = c.plan[a];
         P.tw64[a] = c.d_tw64[a];
         P.tw32[a] = c.d_tw32[a];
+        P.twfx[a] = static_cast<const fxw*>(c.d_twfx[a]);
       }
       P.col_x = B.d_col_x;
       P.col_y = B.d_col_y;
@@ -1119,6 +1182,8 @@ int paro_batch_create(paro_batch** out, paro_ctx* const* ctxs, int n_ctx) {
       P.g_col = B.d_g_col;
       P.g_z = B.d_g_z;
       P.xrows = B.d_xrows;
+      P.stick_of = B.d_stick_of;
+      P.xrow_c = B.d_xrow_c;
       P.kin = B.d_kin;
       P.kin32 = B.d_kin32;
       P.vplane = c.d_vplane;
@@ -1205,6 +1270,29 @@ int paro_batch_create(paro_batch** out, paro_ctx* const* ctxs, int n_ctx) {
   if (e == cudaSuccess) e = cudaMemcpy(b->d_bprob, bprob.data(), b->nbt * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(b->d_brow, brow.data(), b->nbt * sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(b->d_bar, 0, 4 * sizeof(unsigned));
+  // items by grid for the line-FFT passes
+  for (int pi : order) {
+    const ProbDev& P = b->hprob[pi];
+    if (!line_covered(b, P)) continue;
+    auto it = std::find_if(b->groups.begin(), b->groups.end(), [&](const BatchGroup& g) { return g.n == P.N1; });
+    if (it == b->groups.end()) {
+      b->groups.push_back(BatchGroup());
+      it = b->groups.end() - 1;
+      it->n = P.N1;
+    }
+    it->nitems += P.nb;
+    it->max_ncol = std::max(it->max_ncol, P.ncol);
+    it->max_nxr = std::max(it->max_nxr, P.nxr);
+  }
+  for (BatchGroup& g : b->groups) {
+    std::vector<int> gi;
+    for (int i = 0; i < b->nitems; ++i) {
+      const ProbDev& P = b->hprob[items[i].x];
+      if (P.N1 == g.n && line_covered(b, P)) gi.push_back(i);
+    }
+    if (e == cudaSuccess) e = cudaMalloc((void**)&g.d_items, gi.size() * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemcpy(g.d_items, gi.data(), gi.size() * sizeof(int), cudaMemcpyHostToDevice);
+  }
   if (e != cudaSuccess) return bail(PARO_ERR_CUDA, std::string("batch upload: ") + cudaGetErrorString(e));
   const int st = b->f64 ? autotune<double>(b) : autotune<float>(b);
   if (st) {
@@ -1219,26 +1307,9 @@ int paro_batch_apply_h(paro_batch* b, int dtype, const void* const* psi, void* c
   if (!b || !psi || !hpsi) return PARO_ERR_ARG;
   if ((dtype == PARO_C64) != b->f64 || (dtype != PARO_C64 && dtype != PARO_C32))
     return berr(b, PARO_ERR_ARG, "paro_batch_apply_h: dtype must match the contexts' precision");
-  const size_t es = b->f64 ? sizeof(double2) : sizeof(float2);
-  for (int i = 0; i < b->nprob; ++i) {
-    const ProbDev& P = b->hprob[i];
+  for (int i = 0; i < b->nprob; ++i)
     if (!psi[i] || !hpsi[i]) return berr(b, PARO_ERR_ARG, "paro_batch_apply_h: null pointer");
-    BCU(b, cudaMemcpyAsync(static_cast<char*>(b->p) + P.off * es, psi[i], (size_t)P.nb * P.npw * es,
-                           cudaMemcpyDeviceToDevice, b->st));
-  }
-  const int mode = b->threads == 1 ? 0 : 1;
-  int st = b->f64 ? launch_fused<double>(b, b->st, static_cast<const double2*>(b->p), static_cast<double2*>(b->ap),
-                                         nullptr, 0, mode, b->grid)
-                  : launch_fused<float>(b, b->st, static_cast<const float2*>(b->p), static_cast<float2*>(b->ap),
-                                        nullptr, 0, mode, b->grid);
-  if (st) return st;
-  b->lead->launches += 1;
-  for (int i = 0; i < b->nprob; ++i) {
-    const ProbDev& P = b->hprob[i];
-    BCU(b, cudaMemcpyAsync(hpsi[i], static_cast<char*>(b->ap) + P.off * es, (size_t)P.nb * P.npw * es,
-                           cudaMemcpyDeviceToDevice, b->st));
-  }
-  return PARO_OK;
+  return b->f64 ? batch_apply<double>(b, psi, hpsi) : batch_apply<float>(b, psi, hpsi);
 }
 
 int paro_batch_step(paro_batch* b, double rel_tol, int max_it, double* max_resid_out) {

@@ -58,3 +58,33 @@ def test_zero_and_nonfinite_rows(n):
     assert (out[0] == 0).all()
     assert torch.isnan(torch.view_as_real(out[1])).any()
     assert torch.isfinite(torch.view_as_real(out[2])).all()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_batch_on_the_callers_arrays(precision):
+    """paro_batch_apply_h reads and writes the caller's arrays where they allow it (their own outputs included) and
+    goes through its own buffers where outputs overlap other inputs: the same values either way."""
+    import ctypes
+    ctxs, rows = [], []
+    dt = torch.complex128 if precision == "fp64" else torch.complex64
+    for i, ecut in enumerate((20.2, 48.0, 20.2)):
+        ctx = paro.Context(np.eye(3) * L, np.array([[0.3 + 0.1 * i, 0.2, 0.1]]), ecut, 3, 2, precision)
+        ctx.set_local_pp(**inputs.LOCAL_PP)
+        ctxs.append(ctx)
+        rows.append(torch.from_numpy(inputs.start_vectors(3, ctx.npw(), 40 + i)).to(dt).cuda())
+    b = paro.Batch(ctxs)
+    want = [c.apply_h(x) for c, x in zip(ctxs, rows)]
+    tol = 1e-14 if precision == "fp64" else 1e-6
+
+    def call(src, dst):
+        p = (ctypes.c_void_p * 3)(*[t.data_ptr() for t in src])
+        q = (ctypes.c_void_p * 3)(*[t.data_ptr() for t in dst])
+        assert b.lib.paro_batch_apply_h(b.h, 0 if precision == "fp64" else 1, p, q) == 0
+        for w, t in zip(want, dst):
+            assert (torch.linalg.vector_norm(t - w) / torch.linalg.vector_norm(w)).item() < tol
+
+    call(rows, [torch.empty_like(x) for x in rows])
+    own = [x.clone() for x in rows]
+    call(own, own)  # in place
+    swapped = [x.clone() for x in rows]
+    call(swapped, [swapped[2], torch.empty_like(rows[1]), swapped[0]])  # outputs over other problems' inputs
