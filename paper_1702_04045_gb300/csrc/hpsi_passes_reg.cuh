@@ -6,13 +6,13 @@
 // Register-FFT versions of the three passes for cubic grids N^3 with N in {32, 36, 48, 72, 128}
 // (line FFTs of fft_reg.cuh: one group of P lanes per line, Q values per lane).
 // ------------------------------------------------------------------------------------------------
-// FP32 lines with Q > P keep step C in the lanes (line_inv_t / line_fwd_t). The z-passes and the density
+// Lines with Q > P keep step C in the lanes (line_inv_t / line_fwd_t). The z-passes and the density
 // pass exchange through the line's own storage in shared memory; the plane pass, whose column tiles
 // would meet two-way bank conflicts in both directions, gives each lane group of a warp its own tile
 // (kWarpTile elements per warp).
 template <typename T, int N> struct PlaneLines {
   static constexpr int Q = LineShape<N>::Q, P = LineShape<N>::P;
-  static constexpr bool kTile = sizeof(T) == 4 && Q > P;
+  static constexpr bool kTile = Q > P;
   static constexpr int kWarpTile = kTile ? (32 / P) * P * (P + 1) : 0;
 };
 
@@ -381,7 +381,8 @@ __global__ void __launch_bounds__(32 * NW) k_plane_density_reg(const cplx<T>* __
           const int cs = ok ? so[P * q + p] : -1;
           v[q] = cs >= 0 ? Sz[cs] : mk<T>(0, 0);
         }
-        if constexpr (LY::kTile) line_inv_tr<T, Q, P>(v, p, lty, tiles + warp * kWT + grp * P * (P + 1), 1, true);
+        if constexpr (LY::kTile && sizeof(T) == 8) line_inv_t<T, Q, P>(v, p, ty, tiles + warp * kWT + grp * P * (P + 1), 1, true);
+        else if constexpr (LY::kTile) line_inv_tr<T, Q, P>(v, p, lty, tiles + warp * kWT + grp * P * (P + 1), 1, true);
         else line_inv<T, Q, P>(v, p, ty);
         if (ok) {
           cplx<T>* row = Pl + r * LS;
@@ -405,7 +406,8 @@ __global__ void __launch_bounds__(32 * NW) k_plane_density_reg(const cplx<T>* __
           const int o = roff[P * q + p];
           v[q] = ok && o >= 0 ? Pl[o + y] : mk<T>(0, 0);
         }
-        if constexpr (LX::kTile) line_inv_tr<T, Q, P>(v, p, ltx, tiles + warp * kWT + grp * P * (P + 1), 1, true);
+        if constexpr (LX::kTile && sizeof(T) == 8) line_inv_t<T, Q, P>(v, p, tx, tiles + warp * kWT + grp * P * (P + 1), 1, true);
+        else if constexpr (LX::kTile) line_inv_tr<T, Q, P>(v, p, ltx, tiles + warp * kWT + grp * P * (P + 1), 1, true);
         else line_inv<T, Q, P>(v, p, tx);
         if (ok)
 #pragma unroll

@@ -88,3 +88,16 @@ def test_batch_on_the_callers_arrays(precision):
     call(own, own)  # in place
     swapped = [x.clone() for x in rows]
     call(swapped, [swapped[2], torch.empty_like(rows[1]), swapped[0]])  # outputs over other problems' inputs
+
+
+@pytest.mark.parametrize("n", [32, 36, 48, 72])
+def test_state_of_the_fp64_iteration(n):
+    """H psi as the FP64 iteration forms it (csrc/fft_reg.cuh, FP64 lines): the Ritz values and the vanishing
+    off-diagonal elements of H over the orbitals against the oracle's H."""
+    ctx, b, v = _setup(n, "fp64")
+    ctx.set_orbitals(inputs.start_vectors(3, b.npw, n) / (1.0 + b.kin))
+    psi = ctx.get_orbitals()
+    h = psi.conj() @ pw.apply_h(b, v, psi).T
+    norm = np.linalg.norm(b.kin * psi, axis=1).max() + np.abs(v).max()
+    # the bound of an H psi above, twice: H of the orthonormal rows, and the rows' own rounding and rotation
+    assert np.abs(h - np.diag(ctx.eigenvalues()[0])).max() <= 96 * 2.0 ** -53 * norm
