@@ -324,8 +324,22 @@ int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
   const Basis& B = c->bases[ik];
   double2* P = static_cast<double2*>(ws_get(c, "kb_proj", (size_t)c->nproj * nb * sizeof(double2)));
   if (!P) return PARO_ERR_CUDA;
-  int st = kb_project<T>(c, ik, nb, psi, P);
-  if (st) return st;
+  int st = PARO_OK;
+  // FP32 on the CUDA cores: the projections' reduction leaves D o P in FP32 for the update, three launches. The product is
+  // bound by launches and by how few CTAs share it: H psi of 23 bands on 32 projectors (8 atoms, 14 Ha) 63.6 -> 49.3 us with
+  // K slices of 64, the reduction's lanes, this conversion and update tiles of 32 rows.
+  if constexpr (sizeof(T) == 4) {
+    if (!(c->tc_scope && tc_enabled()) && !kb_slices(c, ik, nb, false)) {
+      float2* wf = static_cast<float2*>(ws_get(c, "wx32_w", (size_t)nb * c->nproj * sizeof(float2)));
+      if (!wf) return PARO_ERR_CUDA;
+      if ((st = gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, !c->tc_scope,
+                                 c->d_dvec, wf)))
+        return st;
+      return gemm_wx<T, T>(c, nb, B.npw, c->nproj, P, nb, false, c->d_dvec, beta_of<T>(B), B.npw, hpsi, B.npw, 1.0, wf,
+                           false, true);
+    }
+  }
+  if ((st = kb_project<T>(c, ik, nb, psi, P))) return st;
   // inside the inexact inner solves: the tensor-core product fed by the projectors' presplit image
   if constexpr (sizeof(T) == 4) {
     if (c->tc_scope && tc_enabled()) {

@@ -150,6 +150,35 @@ __global__ void k_reduce_parts(int M, int N, int nz, const double2* __restrict__
   C[(size_t)m * ldc + n] = mirror ? cconj(s) : s;
 }
 
+// The same sum with eight lanes an output (lane l the slices l, l + 8, ...; then three shuffle steps), for products of few
+// outputs and many slices, where one thread's chain of loads is the time. WF: the row-scaled FP32 copy wf[m N + n] =
+// s[m] C[m][n] as well, which the FP32 update product of the projectors reads (k_w_to_f32's result, without its launch).
+template <bool WF>
+__global__ void __launch_bounds__(256) k_reduce_lanes(int M, int N, int nz, const double2* __restrict__ part,
+                                                      double2* __restrict__ C, int ldc, int herm, int tile,
+                                                      const double* __restrict__ s, float2* __restrict__ wf) {
+  const int idx = (blockIdx.x * 256 + threadIdx.x) >> 3, l = threadIdx.x & 7;
+  const bool ok = idx < M * N;
+  const int m = ok ? idx / N : 0, n = ok ? idx - m * N : 0;
+  const bool mirror = herm && (m / tile) > (n / tile);
+  const size_t off = mirror ? (size_t)n * N + m : (size_t)m * N + n;
+  double2 t = make_double2(0.0, 0.0);
+  if (ok)
+    for (int z = l; z < nz; z += 8) t = cadd(t, part[(size_t)z * M * N + off]);
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, h);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, h);
+  }
+  if (!ok || l) return;
+  if (mirror) t = cconj(t);
+  C[(size_t)m * ldc + n] = t;
+  if (WF) {
+    const double2 w = cscale(t, s[m]);
+    wf[idx] = make_float2((float)w.x, (float)w.y);
+  }
+}
+
 // micro-tile R (tile 16 R) for an M x N product: the least padded work, weighted by the micro-tile's cost
 // per useful product (a thread's 2 R shared-memory loads feed 4 R^2 multiply-adds, so R = 2 spends about
 // half its issue slots on loads)
@@ -169,13 +198,13 @@ static int pick_r(int M, int N, bool herm) {
   return best;
 }
 
-// K slices: the count nz (at most one per 256 of K, at most max_slices) that minimises the modelled
+// K slices: the count nz (at most one per `grain` of K, at most max_slices) that minimises the modelled
 // makespan, ceil(tiles nz / 152) waves of CTAs sharing an SM times the steps (of `step` K values, the
 // kernel's stage) of one slice; ties go to fewer slices (less partial-sum traffic).
 static void split_k(int tiles, int K, size_t max_slices, int* nz_out, int* kslice_out, int resident = 1,
-                    int step = 16) {
+                    int step = 16, int grain = 256) {
   const int steps = (K + step - 1) / step;
-  int maxz = (K + 255) / 256;
+  int maxz = (K + grain - 1) / grain;
   if ((size_t)maxz > max_slices) maxz = (int)max_slices;
   if (maxz < 1) maxz = 1;
   const long long slots = 152LL * (resident < 1 ? 1 : resident);  // CTAs resident at once
@@ -291,7 +320,7 @@ int tc_flag_readback(Ctx* c, const int** h) {
 
 template <typename TA, typename TB, typename ACC>
 int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb, double2* C,
-            int ldc, bool herm, bool carry) {
+            int ldc, bool herm, bool carry, const double* wscale, float2* wf) {
   if (M <= 0 || N <= 0) return PARO_OK;
   if constexpr (sizeof(TA) == 8 && sizeof(TB) == 8) {
     // at every size the digit slices are faster than the FP64 pipe (Gram and V_nl of one 1189-coefficient row: 335 -> 85 us and 367 -> 70 us with the
@@ -302,7 +331,10 @@ int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<
   const int tiles_m = (M + tile - 1) / tile, tiles_n = (N + tile - 1) / tile;
   const int tiles = herm ? tiles_m * (tiles_m + 1) / 2 : tiles_m * tiles_n;
   int nz = 1, kslice = 16;
-  split_k(tiles, K, (size_t)1 << 20, &nz, &kslice, cn_resident<TA, TB, ACC>(r, carry), CnStepK<ACC>::value);
+  // FP32 products too small to give every SM a slice of 256: slices of 64 (two stages). FP64 keeps its sums.
+  const bool fine = sizeof(ACC) == 4 && (long long)tiles * ((K + 255) / 256) < 152;
+  split_k(tiles, K, (size_t)1 << 20, &nz, &kslice, cn_resident<TA, TB, ACC>(r, carry), CnStepK<ACC>::value,
+          fine ? 64 : 256);
   double2* part = static_cast<double2*>(ws_get(c, "gemm_parts", (size_t)nz * M * N * sizeof(double2)));
   if (!part) return PARO_ERR_CUDA;
   if (K == 0) {
@@ -314,8 +346,15 @@ int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<
     PARO_LAUNCH(c, "k_gemm_cn");
     prof_end(c, sizeof(ACC) == 8 ? "k_gemm_cn<f64>" : "k_gemm_cn<f32>", ev);
   }
-  k_reduce_parts<<<(M * N + 255) / 256, 256, 0, c->stream>>>(M, N, K == 0 ? 1 : nz, part, C, ldc, herm ? 1 : 0,
-                                                             tile);
+  if (wf)
+    k_reduce_lanes<true><<<(M * N + 31) / 32, 256, 0, c->stream>>>(M, N, K == 0 ? 1 : nz, part, C, ldc, herm ? 1 : 0,
+                                                                   tile, wscale, wf);
+  else if (fine)
+    k_reduce_lanes<false><<<(M * N + 31) / 32, 256, 0, c->stream>>>(M, N, K == 0 ? 1 : nz, part, C, ldc, herm ? 1 : 0,
+                                                                    tile, nullptr, nullptr);
+  else
+    k_reduce_parts<<<(M * N + 255) / 256, 256, 0, c->stream>>>(M, N, K == 0 ? 1 : nz, part, C, ldc, herm ? 1 : 0,
+                                                               tile);
   PARO_LAUNCH(c, "k_reduce_parts");
   return PARO_OK;
 }
@@ -506,12 +545,13 @@ __global__ void __launch_bounds__(256) k_gemm_wx32(int M, int N, int K, const fl
   }
 }
 
-// launch of k_gemm_wx32: RM = 9 (144-row blocks) unless M fits 64 rows; RN (32 or 64 columns) with the
+// launch of k_gemm_wx32: RM = 9 (144-row blocks) unless M fits 64 or 32 rows (RM = 4, 2); RN (32 or 64 columns) with the
 // smaller makespan in waves of 152 SMs x resident CTAs
 static int launch_wx32(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s,
-                       const float2* X, int ldx, float2* Y, int ldy, double beta, float2* Wf, bool lower) {
-  const bool big = M > 64;
-  const int tm = big ? 144 : 64;
+                       const float2* X, int ldx, float2* Y, int ldy, double beta, float2* Wf, bool lower,
+                       bool wf_ready) {
+  const bool big = M > 64, low = M <= 32;
+  const int tm = big ? 144 : low ? 32 : 64;
   const int mt = (M + tm - 1) / tm;
   const long long s2 = (long long)mt * ((N + 31) / 32), s4 = (long long)mt * ((N + 63) / 64);
   // resident CTAs per SM by register use: about 3 (RN = 2) and 2 (RN = 4) at RM = 9
@@ -521,11 +561,11 @@ static int launch_wx32(Ctx* c, int M, int N, int K, const double2* W, int ldw, b
   const float fb = (float)beta;
   if (!Wf) Wf = static_cast<float2*>(ws_get(c, "wx32_w", (size_t)M * K * sizeof(float2)));
   if (!Wf) return PARO_ERR_CUDA;
-  if (K > 0) {
+  if (K > 0 && !wf_ready) {
     k_w_to_f32<<<std::min((M * K + 255) / 256, 304), 256, 0, c->stream>>>(M, K, W, ldw, wt ? 1 : 0, s, Wf);
     PARO_LAUNCH(c, "k_w_to_f32");
   }
-  const int rm = big ? 9 : 4, rn = rn4 ? 4 : 2;
+  const int rm = big ? 9 : low ? 2 : 4, rn = rn4 ? 4 : 2;
   const size_t sm = (size_t)3 * 16 * 16 * (rm + rn) * sizeof(float2);  // three stages
   static int attr_dev = -1;  // dynamic shared memory above 48 KB, set per device
   int dev = 0;
@@ -533,7 +573,8 @@ static int launch_wx32(Ctx* c, int M, int N, int K, const double2* W, int ldw, b
   if (attr_dev != dev) {
     for (const void* f : {(const void*)k_gemm_wx32<9, 4>, (const void*)k_gemm_wx32<9, 4, true>,
                           (const void*)k_gemm_wx32<9, 2>, (const void*)k_gemm_wx32<9, 2, true>,
-                          (const void*)k_gemm_wx32<4, 4>, (const void*)k_gemm_wx32<4, 2>})
+                          (const void*)k_gemm_wx32<4, 4>, (const void*)k_gemm_wx32<4, 2>,
+                          (const void*)k_gemm_wx32<2, 4>, (const void*)k_gemm_wx32<2, 2>})
       PARO_CU(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
     attr_dev = dev;
   }
@@ -543,6 +584,9 @@ static int launch_wx32(Ctx* c, int M, int N, int K, const double2* W, int ldw, b
   } else if (big) {
     if (rn4) k_gemm_wx32<9, 4><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
     else k_gemm_wx32<9, 2><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
+  } else if (low) {
+    if (rn4) k_gemm_wx32<2, 4><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
+    else k_gemm_wx32<2, 2><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
   } else {
     if (rn4) k_gemm_wx32<4, 4><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
     else k_gemm_wx32<4, 2><<<grid, 256, sm, c->stream>>>(M, N, K, Wf, X, ldx, Y, ldy, fb);
@@ -553,11 +597,11 @@ static int launch_wx32(Ctx* c, int M, int N, int K, const double2* W, int ldw, b
 
 template <typename TX, typename TY>
 int gemm_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<TX>* X,
-            int ldx, cplx<TY>* Y, int ldy, double beta, float2* wf, bool lower) {
+            int ldx, cplx<TY>* Y, int ldy, double beta, float2* wf, bool lower, bool wf_ready) {
   if (M <= 0 || N <= 0) return PARO_OK;
   if constexpr (sizeof(TX) == 4 && sizeof(TY) == 4) {
     cudaEvent_t ev = prof_begin(c);
-    int st = launch_wx32(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta, wf, lower);
+    int st = launch_wx32(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta, wf, lower, wf_ready);
     if (st) return st;
     prof_end(c, "k_gemm_wx<f32>", ev);
     return PARO_OK;
@@ -1462,15 +1506,15 @@ int convert(Ctx* c, size_t n, const cplx<TS>* src, cplx<TD>* dst) {
 
 // instantiations
 template int gemm_cn<double, double, double>(Ctx*, int, int, int, const double2*, int, const double2*, int, double2*,
-                                             int, bool, bool);
+                                             int, bool, bool, const double*, float2*);
 template int gemm_cn<float, float, float>(Ctx*, int, int, int, const float2*, int, const float2*, int, double2*, int,
-                                          bool, bool);
+                                          bool, bool, const double*, float2*);
 template int gemm_wx<double, double>(Ctx*, int, int, int, const double2*, int, bool, const double*, const double2*,
-                                     int, double2*, int, double, float2*, bool);
+                                     int, double2*, int, double, float2*, bool, bool);
 template int gemm_wx<float, float>(Ctx*, int, int, int, const double2*, int, bool, const double*, const float2*, int,
-                                   float2*, int, double, float2*, bool);
+                                   float2*, int, double, float2*, bool, bool);
 template int gemm_wx<float, double>(Ctx*, int, int, int, const double2*, int, bool, const double*, const float2*,
-                                    int, double2*, int, double, float2*, bool);
+                                    int, double2*, int, double, float2*, bool, bool);
 template int band_norms<double>(Ctx*, int, int, const double2*, int, double*);
 template int band_norms<float>(Ctx*, int, int, const float2*, int, double*);
 template int convert<double, float>(Ctx*, size_t, const double2*, float2*);

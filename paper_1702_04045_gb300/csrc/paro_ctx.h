@@ -246,18 +246,19 @@ int check_fft_support(Ctx* c, int elem_bytes);
 // C[m][n] = sum_k conj(A[m][k]) B[n][k]; A: M x K (lda), B: N x K (ldb); C: M x N (ldc) complex double.
 // ACC = double: FP64 throughout. ACC = float: FP32 sums over each K slice, or with carry sums of 16
 // consecutive products in FP32 carried into FP64. K-slice partials are summed in double in a fixed order.
-// herm: A == B, only tiles with m-tile <= n-tile are computed, the rest mirrored.
+// herm: A == B, only tiles with m-tile <= n-tile are computed, the rest mirrored. wf (with wscale, device double[M],
+// and ldc = N): also wf[m N + n] = wscale[m] C[m][n] in FP32, the form gemm_wx reads with wf_ready.
 template <typename TA, typename TB, typename ACC>
 int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb,
-            double2* C, int ldc, bool herm, bool carry = false);
+            double2* C, int ldc, bool herm, bool carry = false, const double* wscale = nullptr, float2* wf = nullptr);
 // Y[m][n] = beta Y[m][n] + sum_k s_k W(k, m) X[k][n]; W: complex double, element (k, m) at W[k*ldw + m]
 // (or at W[m*ldw + k] when wt); s: device double[K] or nullptr (1); X: K x N (ldx) of TX;
 // Y: M x N (ldy) of TY; accumulation in TY. wf: device scratch of M K float2 for the FP32 form's converted
 // W (nullptr: a workspace of the context, allocated on first use). lower: W(k, m) = 0 for k > m (a
-// triangular factor), which lets the FP32 form skip the zero products.
+// triangular factor), whose zero products are skipped. wf_ready: wf holds s_k W(k, m) at wf[k M + m] already.
 template <typename TX, typename TY>
 int gemm_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, const double* s, const cplx<TX>* X,
-            int ldx, cplx<TY>* Y, int ldy, double beta, float2* wf = nullptr, bool lower = false);
+            int ldx, cplx<TY>* Y, int ldy, double beta, float2* wf = nullptr, bool lower = false, bool wf_ready = false);
 // gemm_cn with the K-slice partials in caller memory (part_elems complex doubles); allocates nothing.
 template <typename TA, typename TB, typename ACC>
 int gemm_cn_scratch(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb,
