@@ -4,7 +4,8 @@
 
 // ------------------------------------------------------------------------------------------------
 // Register-FFT versions of the three passes for cubic grids N^3 with N in {32, 36, 48, 72, 128}
-// (line FFTs of fft_reg.cuh: one group of P lanes per line, Q values per lane).
+// (line FFTs of fft_reg.cuh: one group of P lanes per line, Q values per lane): FP32, and FP64 inside the FP64
+// iteration, which keeps this arithmetic (PlainF64); other FP64 work takes hpsi_passes_tile.cuh.
 // ------------------------------------------------------------------------------------------------
 // Lines with Q > P keep step C in the lanes (line_inv_t / line_fwd_t). The z-passes and the density
 // pass exchange through the line's own storage in shared memory; the plane pass, whose column tiles

@@ -3,7 +3,8 @@
 // problem is an independent source problem, Algorithm 1 step 3, and the projection step 4 is local to
 // its problem).
 //
-//  * H psi: one persistent kernel per apply over flat work lists of every problem's orbitals, in three
+//  * H psi: problems on a grid with a line-FFT form (batch_tile_covers) run through k_tile_batch.cu, one launch per
+//    phase and grid; the others in one persistent kernel per apply over flat work lists of every problem's orbitals, in three
 //    phases: z-FFTs of stick groups (and the projections per orbital), one unit per (orbital, z-plane)
 //    for the 2D FFTs and V_eff(r), and z-FFTs back with the gather, kinetic and projector terms. The
 //    phases are separated by bounded grid barriers of a cooperative launch, or by kernel boundaries

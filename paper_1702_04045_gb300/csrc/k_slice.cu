@@ -15,8 +15,8 @@
 //     dropped below that: FP64 results, more accurate than FP64 sums of the same length;
 //   L = 4, PMAX = 5 (10 products): operands rounded to 2^-31, for FP32 operands outside the inner solves.
 //
-// Measured on the 64-atom cell (N_pw = 23847): V_nl of 144 FP64 orbitals 17.7 -> 0.68 ms, Cholesky
-// orthonormalisation of 288 rows 31.8 -> 3.1 ms (2.1 ms of it the factorisation); the error against extended
+// Measured on the 64-atom cell (N_pw = 23847): V_nl of 144 FP64 orbitals 17.7 -> 0.57 ms, Cholesky
+// orthonormalisation of 288 rows 31.8 -> 1.88 ms (0.8 ms of it the factorisation); the error against extended
 // precision is 3e-17 of the rows' norms where FP64 sums have 3e-15. A stage (16 K values) of a 128 x 32 tile takes
 // 1.8 us, 53 cycles per MMA of 64 columns against 48 for its operands' shared-memory traffic: the tensor
 // pipe's operand feed bounds it, the loads (79 KB a stage) and the sums are hidden.
