@@ -400,6 +400,7 @@ static int apply_h_noalloc(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* 
   if (!c->have_veff) return fail(c, PARO_ERR_STATE, "no effective potential set");
   int st = configure<T>(c);
   if (st) return st;
+  PlainF64 plain(c, true);  // the FP64 update product in place: the digit slices would grow workspaces
   const Basis& B = c->bases[ik];
   const int eb = (int)sizeof(cplx<T>);
   const size_t sticks = round256((size_t)nb * c->N[2] * B.ncol * eb);

@@ -217,10 +217,14 @@ struct TcScope {
 // iteration, where the last bit of a Ritz value decides them, so any other rounding, however much smaller,
 // turns about half of the orbitals of a stored state around. Calls that do not decide orbitals (H psi, source
 // problems, orthonormalisation, adjoint, density, energy) take the digit slices and the fixed-point FFT.
+// always: FP64 products on the FP64 pipe whatever the context's precision, for calls that may not allocate (the
+// digit slices work in workspaces of the context).
 struct PlainF64 {
   Ctx* c;
   bool old;
-  explicit PlainF64(Ctx* ctx) : c(ctx), old(ctx->plain64) { ctx->plain64 = ctx->prec == PARO_FP64; }
+  explicit PlainF64(Ctx* ctx, bool always = false) : c(ctx), old(ctx->plain64) {
+    ctx->plain64 = always || ctx->prec == PARO_FP64;
+  }
   ~PlainF64() { c->plain64 = old; }
 };
 // Scoped phase tag: names recorded inside become "tag:name".
