@@ -25,6 +25,7 @@
 // B tile NC rows three times (b_r; b_i; -b_r), so that a_r meets (b_r | b_i) and a_i meets (b_i | -b_r) as
 // one MMA of 2 NC columns each: Re and Im side by side in tensor memory.
 #include <algorithm>
+#include <cstdlib>
 #include <type_traits>
 
 #include "paro_ctx.h"
@@ -36,6 +37,15 @@ static const int kSliceM = 128;           // rows of the A tile (TMEM lanes)
 static const int kSliceK = 16;            // complex K values per stage (one MMA K step per plane)
 static const int kSliceThreads = 320;     // producer warp, MMA warp, eight epilogue warps
 static const uint32_t kSlicePolls = 1u << 24;
+// Polls after which a wait of the kernel's roles gives up: kSlicePolls, or PARO_SLICE_POLLS of the environment (0: at
+// once), which lets a test run the time-out path. The waits that drain the kernel keep kSlicePolls.
+static uint32_t slice_polls() {
+  static const uint32_t n = [] {
+    const char* e = std::getenv("PARO_SLICE_POLLS");
+    return e && e[0] ? (uint32_t)std::min<unsigned long>(std::strtoul(e, nullptr, 10), kSlicePolls) : kSlicePolls;
+  }();
+  return n;
+}
 
 // NC: columns of an output tile (2 NC accumulator columns per group, at most 512 in tensor memory): 32 for
 // L = 7, 64 or 48 for L = 4, whichever pads less;
@@ -470,7 +480,7 @@ template <int L, int NC, int MODE, typename OUT>
 __global__ void __launch_bounds__(kSliceThreads, 1)
     k_slice_gemm(int M, int N, SliceTiles geo, const unsigned char* __restrict__ a_img, const int* __restrict__ ea,
                  int ea_ld, const unsigned char* __restrict__ b_img, const int* __restrict__ eb, int eb_ld,
-                 cplx<OUT>* __restrict__ out, int ldo, int accum, int* __restrict__ err) {
+                 cplx<OUT>* __restrict__ out, int ldo, int accum, uint32_t polls, int* __restrict__ err) {
   using Cfg = SliceCfg<L>;
   constexpr int PMAX = Cfg::PMAX, CH = Cfg::CH, NS = Cfg::NS, NG = PMAX - 1;
   constexpr int AB = slice_a_bytes<L>(), BB = slice_b_bytes<L>(NC), BUF = AB + BB;
@@ -479,9 +489,9 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
   static_assert(2 * NC * NG <= 512 && HC % 8 == 0, "tensor memory columns");
   extern __shared__ __align__(128) unsigned char smem_dyn[];
   unsigned char* smem = tc_align1024(smem_dyn);
-  __shared__ uint64_t full[NS], freeb[NS], gfull[NG], gfree[NG];
+  __shared__ uint64_t full[NS], freeb[NS], gfull[NG], gfree[NG], done;
   __shared__ uint32_t tmem_base;
-  __shared__ int s_fail, s_last_commit, s_last_copy[NS];
+  __shared__ int s_fail, s_last_copy[NS];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int ntiles = geo.per_z * geo.nz;
   if (tid == 0) {
@@ -494,8 +504,8 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
       tc::mbar_init(&gfull[g], 1);
       tc::mbar_init(&gfree[g], kSliceThreads - 64);
     }
+    tc::mbar_init(&done, 1);
     s_fail = 0;
-    s_last_commit = -1;
     tc::fence_mbar_init();
   }
   if (warp == 1) {
@@ -514,7 +524,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
       const SliceTile<NC> tl(geo, t);
       for (int s = 0; s < tl.nst && !*vfail; ++s, ++sg) {
         const int b = sg % NS;
-        if (sg >= NS && !tc::mbar_wait(&freeb[b], (uint32_t)(sg / NS - 1) & 1u, kSlicePolls)) {
+        if (sg >= NS && !tc::mbar_wait(&freeb[b], (uint32_t)(sg / NS - 1) & 1u, polls)) {
           *vfail = 1;
           break;
         }
@@ -536,7 +546,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
         const int b = sg % NS, ch = cg + s / CH;
         const bool first = s % CH == 0, last = s % CH == CH - 1 || s == tl.nst - 1;
         // votes keep the loop's control flow, and with it the descriptors, uniform over the warp
-        okg = __all_sync(0xffffffffu, !*vfail && tc::mbar_wait(&full[b], (uint32_t)(sg / NS) & 1u, kSlicePolls));
+        okg = __all_sync(0xffffffffu, !*vfail && tc::mbar_wait(&full[b], (uint32_t)(sg / NS) & 1u, polls));
         if (!okg) break;
         tc::tc_fence_after();
         // descriptors by their low words: the stage's base plus constant offsets (in 16 bytes); the issuing
@@ -545,7 +555,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
 #pragma unroll
         for (int g = 2; g <= PMAX; ++g) {
           if (first && ch > 0 && okg) {
-            okg = __all_sync(0xffffffffu, tc::mbar_wait(&gfree[g - 2], (uint32_t)(ch - 1) & 1u, kSlicePolls));
+            okg = __all_sync(0xffffffffu, tc::mbar_wait(&gfree[g - 2], (uint32_t)(ch - 1) & 1u, polls));
             tc::tc_fence_after();
           }
           if (okg) {
@@ -563,13 +573,12 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
           }
         }
         if (!okg) break;
-        if (leader) {
-          tc::mma_commit(&freeb[b]);
-          s_last_commit = sg;
-        }
+        if (leader) tc::mma_commit(&freeb[b]);
       }
       cg += (tl.nst + CH - 1) / CH;
     }
+    // every MMA issued so far, those of a stage that was given up among them
+    if (leader) tc::mma_commit(&done);
     if (!okg) *vfail = 1;
   } else if (warp >= 2) {  // the sums: TMEM lanes 32 (warp % 4) .., columns HC half .. of Re and of Im
     constexpr int PC = HC % 16 == 0 ? 16 : 8;  // columns per read
@@ -587,7 +596,7 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
       for (int ch = 0; ch < nchunk && okc; ++ch, ++cg) {
 #pragma unroll
         for (int g = 0; g < NG; ++g) {
-          if (okc && (*vfail || !tc::mbar_wait(&gfull[g], (uint32_t)cg & 1u, kSlicePolls))) okc = false;
+          if (okc && (*vfail || !tc::mbar_wait(&gfull[g], (uint32_t)cg & 1u, polls))) okc = false;
           okc = __all_sync(0xffffffffu, okc);
           if (!okc) continue;
           tc::tc_fence_after();
@@ -658,13 +667,13 @@ __global__ void __launch_bounds__(kSliceThreads, 1)
     if (!okc) *vfail = 1;
   }
   __syncthreads();
-  // the last commit covers every MMA issued; copies of tiles that no MMA consumed land before exit
+  // every MMA has read its operands and written tensor memory, and every copy has landed, before the CTA gives
+  // either up (after a time-out too)
   int ok = !*vfail;
-  const int lc = s_last_commit;
-  if (lc >= 0 && !tc::mbar_wait(&freeb[lc % NS], (uint32_t)(lc / NS) & 1u, kSlicePolls)) ok = 0;
+  if (!tc::mbar_wait(&done, 0u, kSlicePolls)) ok = 0;
   if (tid == 0)
     for (int b = 0; b < NS; ++b)
-      if (s_last_copy[b] > lc) tc::mbar_wait(&full[b], (uint32_t)(s_last_copy[b] / NS) & 1u, kSlicePolls);
+      if (s_last_copy[b] >= 0 && !tc::mbar_wait(&full[b], (uint32_t)(s_last_copy[b] / NS) & 1u, kSlicePolls)) ok = 0;
   ok = __syncthreads_and(ok);
   tc::tc_fence_before();
   __syncthreads();
@@ -710,7 +719,7 @@ static int slice_launch_nc(Ctx* c, int M, int N, const SliceTiles& geo, const un
   }
   const int tiles = geo.per_z * geo.nz;
   k_slice_gemm<L, NC, MODE, OUT><<<std::min(tiles, kSliceSms), kSliceThreads, sm, c->stream>>>(
-      M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum, err);
+      M, N, geo, a, ea, ea_ld, b, eb, eb_ld, out, ldo, accum, slice_polls(), err);
   PARO_LAUNCH(c, "k_slice_gemm");
   return PARO_OK;
 }
