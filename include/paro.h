@@ -12,6 +12,11 @@
  *   - The caller owns every array argument; the library copies what it keeps. The library owns the
  *     context and all of its device buffers. Device pointers must stay valid for the duration of the
  *     call. All GPU work is enqueued on the context's stream; calls that return host data synchronise.
+ *   - The tensor-core kernels' waits are bounded. A call that waits for the GPU (paro_apply_vnl,
+ *     paro_solve_source, paro_orthonormalize, paro_energy, the ParO and SCF steps and every call that takes
+ *     Ritz pairs or residuals) returns PARO_ERR_TIMEOUT when such a wait gave up in it or in an
+ *     enqueue-only call before it on the context (paro_apply_h, paro_apply_h_adjoint), whose
+ *     output is then undefined. A time-out is reported once.
  *   - A context is not thread-safe; distinct contexts are independent.
  *   - There is no CPU fallback: every numerical step runs in this library's CUDA kernels.
  */
@@ -30,7 +35,7 @@ typedef enum {
   PARO_ERR_CUDA = -2,          /* a CUDA call failed; the message holds cudaGetErrorString */
   PARO_ERR_BREAKDOWN = -3,     /* PCG p^H A p <= 0 or NaN, or a Cholesky pivot <= 0 */
   PARO_ERR_NOT_CONVERGED = -4, /* SCF / ParO iteration limit reached; the last state is kept */
-  PARO_ERR_TIMEOUT = -5,       /* a bounded device-side wait (grid barrier) gave up */
+  PARO_ERR_TIMEOUT = -5,       /* a bounded device-side wait (grid barrier, tensor-core product) gave up */
   PARO_ERR_STATE = -6          /* call out of order (e.g. no potential or orbitals set yet) */
 } paro_status;
 
@@ -174,6 +179,8 @@ int paro_sigma(const paro_ctx* ctx, double* sigma);
  *   (H psi)(G) = |k+G|^2/2 c_G + [FFT(V_eff . IFFT(c))](G) / N_grid + sum_p beta_p(G) D_p <beta_p|c>.
  *   dtype  PARO_C64 (complex double) or PARO_C32 (complex float): the arithmetic of the whole apply.
  *   psi    device, nb x npw complex of dtype; hpsi device, same shape (must not alias psi).
+ * Enqueued on the context stream, no synchronisation: a tensor-core time-out in it is reported by the next
+ * call on the context that waits for the GPU.
  */
 int paro_apply_h(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, void* hpsi);
 
@@ -230,7 +237,8 @@ int paro_apply_h_noalloc(paro_ctx* ctx, int ik, int nb, int dtype, const void* p
  *   psi, w, g_psi: device nb x npw complex of dtype (row = band); g_v: device double[N1*N2*N3]
  *   (C order, overwritten); g_pos: device double[n_atoms*3] (overwritten). g_psi, g_v or g_pos may be
  *   NULL to skip that output. Work runs in the precision of dtype (FP32 FFTs and 3xTF32 tensor-core
- *   projections for PARO_C32), accumulated in FP64. Enqueued on the context stream, no synchronisation.
+ *   projections for PARO_C32), accumulated in FP64. Enqueued on the context stream, no synchronisation
+ *   (time-outs as in paro_apply_h).
  */
 int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, const void* w, void* g_psi,
                          double* g_v, double* g_pos);
@@ -287,7 +295,7 @@ void paro_batch_destroy(paro_batch* b);
  * preconditioner is diag(|k+G|^2/2 + mean V_eff - sigma)^{-1}. Each orbital stops once its residual
  * has dropped by rel_tol, or after max_it steps.
  *   eps host double[nb]; psi, x device nb x npw of dtype; iters_out host int[nb] or NULL.
- * Errors: PARO_ERR_BREAKDOWN if p^H A p <= 0 or is not finite for an active orbital.
+ * Errors: PARO_ERR_BREAKDOWN if p^H A p <= 0 or is not finite for an active orbital; PARO_ERR_TIMEOUT.
  */
 int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* eps, const void* psi, void* x,
                       double rel_tol, int max_it, int* iters_out);
@@ -301,7 +309,7 @@ int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* ep
  *          added into an FP32 two-sum pair); the factorisation and L^{-1} are FP64 for both.
  *   x, y   device n x npw complex of dtype (row = band); y may equal x (in place), else must not overlap.
  * Errors: PARO_ERR_ARG for a bad argument or n > npw; PARO_ERR_BREAKDOWN when a pivot of the
- * factorisation is not positive (rows linearly dependent to working precision).
+ * factorisation is not positive (rows linearly dependent to working precision); PARO_ERR_TIMEOUT.
  */
 int paro_orthonormalize(paro_ctx* ctx, int ik, int n, int dtype, const void* x, void* y);
 

@@ -472,7 +472,7 @@ static int project_readback(Ctx* c, int ik) {
   auto it = c->pinned.find("tc_err");
   if (it != c->pinned.end() && it->second.h) {
     if ((st = pinned_wait(c, "tc_err"))) return st;
-    if (*static_cast<const int*>(it->second.h)) return fail(c, PARO_ERR_TIMEOUT, "tensor-core product: mbarrier wait gave up");
+    if ((st = tc_report(c, *static_cast<const int*>(it->second.h)))) return st;
   }
   return PARO_OK;
 }
@@ -798,8 +798,11 @@ static int adopt_orbitals(Ctx* c, int ik) {
       return st;
   }
   b.res.resize(c->nb);
+  const int* htc = nullptr;
   PARO_CU(c, cudaMemcpyAsync(b.res.data(), res, c->nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  if ((st = tc_flag_readback(c, &htc))) return st;
   PARO_CU(c, cudaStreamSynchronize(c->stream));
+  if (htc && (st = tc_report(c, *htc))) return st;
   b.hx_recur = 0;
   b.have_psi = true;
   return PARO_OK;
@@ -1414,14 +1417,17 @@ int paro_apply_vnl(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, vo
   } else {
     st = kb_apply<float>(c, ik, nb, static_cast<const float2*>(psi), static_cast<float2*>(out));
   }
-  if (st) return st;
-  const int* htc = nullptr;
-  if ((st = tc_flag_readback(c, &htc))) return st;
-  if (htc) {
-    if ((st = pinned_wait(c, "tc_err"))) return st;
-    if (*htc) return fail(c, PARO_ERR_TIMEOUT, "tensor-core product: mbarrier wait gave up");
-  }
-  return PARO_OK;
+  return st ? st : tc_check(c);
+}
+
+// Status of a call that waits for the GPU: a tensor-core product that gave up leaves undefined sums, which the
+// factorisation or the solver may have met as a breakdown, so it is reported first.
+static int tc_status(Ctx* c, int st) {
+  if (st && st != PARO_ERR_BREAKDOWN) return st;
+  const std::string msg = c->err;
+  if (int s2 = tc_check(c)) return s2;
+  c->err = msg;
+  return st;
 }
 
 int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, const void* w, void* g_psi,
@@ -1447,8 +1453,8 @@ int paro_orthonormalize(paro_ctx* ctx, int ik, int n, int dtype, const void* x, 
   if (x != y && xb < yb + bytes && yb < xb + bytes) return fail(c, PARO_ERR_ARG, "paro_orthonormalize: x and y overlap");
   if (x != y) PARO_CU(c, cudaMemcpyAsync(y, x, bytes, cudaMemcpyDeviceToDevice, c->stream));
   GammaPackOff general(c);
-  return dtype == PARO_C64 ? orthonormalize<double>(c, ik, static_cast<double2*>(y), n)
-                           : orthonormalize<float>(c, ik, static_cast<float2*>(y), n);
+  return tc_status(c, dtype == PARO_C64 ? orthonormalize<double>(c, ik, static_cast<double2*>(y), n)
+                                        : orthonormalize<float>(c, ik, static_cast<float2*>(y), n));
 }
 
 int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* eps, const void* psi, void* x,
@@ -1467,20 +1473,28 @@ int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* ep
   std::vector<double> hf(nb);
   for (int i = 0; i < nb; ++i) hf[i] = eps[i] - c->sigma_k[ik];
   if ((st0 = h2d_async(c, "ss_f", f, hf.data(), nb * sizeof(double)))) return st0;
+  std::vector<int> its;  // pcg_run reads the tensor-core flag back with the step counts
+  if (!iters_out) {
+    its.resize(nb);
+    iters_out = its.data();
+  }
+  int st;
   if (dtype == PARO_C64) {
     double2* rhs = static_cast<double2*>(ws_get(c, "src_rhs64", (size_t)nb * npw * sizeof(double2)));
     if (!rhs) return PARO_ERR_CUDA;
-    int st = scale_rows<double>(c, nb, npw, static_cast<const double2*>(psi), f, rhs);
+    st = scale_rows<double>(c, nb, npw, static_cast<const double2*>(psi), f, rhs);
     if (st) return st;
     PARO_CU(c, cudaMemcpyAsync(x, psi, (size_t)nb * npw * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
-    return pcg_run<double>(c, ik, nb, rhs, static_cast<double2*>(x), false, rel_tol, max_it, iters_out);
+    st = pcg_run<double>(c, ik, nb, rhs, static_cast<double2*>(x), false, rel_tol, max_it, iters_out);
+    return st == PARO_ERR_BREAKDOWN ? tc_status(c, st) : st;
   }
   float2* rhs = static_cast<float2*>(ws_get(c, "src_rhs32", (size_t)nb * npw * sizeof(float2)));
   if (!rhs) return PARO_ERR_CUDA;
-  int st = scale_rows<float>(c, nb, npw, static_cast<const float2*>(psi), f, rhs);
+  st = scale_rows<float>(c, nb, npw, static_cast<const float2*>(psi), f, rhs);
   if (st) return st;
   PARO_CU(c, cudaMemcpyAsync(x, psi, (size_t)nb * npw * sizeof(float2), cudaMemcpyDeviceToDevice, c->stream));
-  return pcg_run<float>(c, ik, nb, rhs, static_cast<float2*>(x), false, rel_tol, max_it, iters_out);
+  st = pcg_run<float>(c, ik, nb, rhs, static_cast<float2*>(x), false, rel_tol, max_it, iters_out);
+  return st == PARO_ERR_BREAKDOWN ? tc_status(c, st) : st;
 }
 
 int paro_set_orbitals(paro_ctx* ctx, int ik, const void* psi, int on_device) {

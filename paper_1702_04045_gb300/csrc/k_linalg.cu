@@ -318,6 +318,20 @@ int tc_flag_readback(Ctx* c, const int** h) {
   return st;
 }
 
+int tc_report(Ctx* c, int flag) {
+  if (!flag) return PARO_OK;
+  PARO_CU(c, cudaMemsetAsync(c->d_tc_err, 0, sizeof(int), c->stream));
+  return fail(c, PARO_ERR_TIMEOUT, "tensor-core product: mbarrier wait gave up");
+}
+
+int tc_check(Ctx* c) {
+  const int* h = nullptr;
+  int st = tc_flag_readback(c, &h);
+  if (st || !h) return st;
+  if ((st = pinned_wait(c, "tc_err"))) return st;
+  return tc_report(c, *h);
+}
+
 template <typename TA, typename TB, typename ACC>
 int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<TB>* B, int ldb, double2* C,
             int ldc, bool herm, bool carry, const double* wscale, float2* wf) {

@@ -254,7 +254,8 @@ __global__ void k_shift_known(int npw, const cplx<T>* __restrict__ hx, const cpl
 
 // Solves (H - sigma_k) x_b = rhs_b for b < nb. On entry x holds the start vectors (ignored when
 // x0_zero), on exit the approximate solutions. Every orbital stops once ||r_b|| <= rel_tol ||r_b^0||
-// or after max_it steps; iters (host, may be null) receives the steps taken. hx0 (may be null): H x
+// or after max_it steps; iters (host, may be null) receives the steps taken, and with them the tensor-core flag of
+// the products is read back and reported. hx0 (may be null): H x
 // of the start vectors when the caller already has it (the orbitals' H psi from the last
 // Rayleigh-Ritz step), which saves the first H application. hx (may be null; needs hx0 or x0_zero):
 // receives H x of the solutions, carried along the iteration from the products the solver forms anyway.
@@ -341,8 +342,11 @@ int pcg_run(Ctx* c, int ik, int nb, const cplx<T>* rhs, cplx<T>* x, bool x0_zero
                                                          std::to_string(hflags[1] - 1));
   }
   if (iters) {
+    const int* htc = nullptr;
     PARO_CU(c, cudaMemcpyAsync(iters, its, nb * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    if ((st = tc_flag_readback(c, &htc))) return st;
     PARO_CU(c, cudaStreamSynchronize(c->stream));
+    if (htc) return tc_report(c, *htc);
   }
   return PARO_OK;
 }

@@ -1149,8 +1149,11 @@ int energy_terms(Ctx* c, const double* rho_dev, double terms[7]) {
   PARO_LAUNCH(c, "k_grid_energies");
   if ((st = hartree_g(c, rho_dev, z, ph, false))) return st;
   std::vector<double> h(ntot);
+  const int* htc = nullptr;  // the projections above may be tensor-core products
   PARO_CU(c, cudaMemcpyAsync(h.data(), part, ntot * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  if ((st = tc_flag_readback(c, &htc))) return st;
   PARO_CU(c, cudaStreamSynchronize(c->stream));
+  if (htc && (st = tc_report(c, *htc))) return st;
   for (int ik = 0; ik < c->nk; ++ik) {
     double sk = 0, sn = 0;
     for (int b = 0; b < nocc; ++b) {

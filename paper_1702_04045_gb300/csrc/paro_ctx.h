@@ -273,6 +273,10 @@ int* tc_err_flag(Ctx* c);
 // enqueues the read-back of the tensor-core error flag (set once a kernel gave up waiting) into pinned
 // memory; *h (null when no tensor-core kernel ran) is valid after pinned_wait(c, "tc_err")
 int tc_flag_readback(Ctx* c, const int** h);
+// PARO_ERR_TIMEOUT for a flag that was read back set, which clears it: a time-out is reported once
+int tc_report(Ctx* c, int flag);
+// both, for calls that wait for the GPU in any case: waits for what is enqueued and reports
+int tc_check(Ctx* c);
 // ---- tensor-core products with the projectors as the fixed operand (k_tc_beta.cu) ----
 int beta_images(Ctx* c, int ik);  // forms the two images of k-point ik if they are missing
 // P[p][b] = <beta_p | x_b> for nb rows x (FP32, ld = N_pw); the K slices are those of plan_nb rows when given (the
