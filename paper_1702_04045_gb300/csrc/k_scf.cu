@@ -327,8 +327,11 @@ int vloc_position_grad(Ctx* c, const double* gv, double* gpos) {
                                                                c->rc, c->A, c->a, c->omega, g);
   PARO_LAUNCH(c, "k_vloc_weight");
   const size_t smf = (size_t)32 * (c->N[2] | 1) * sizeof(double2);
-  if (smf > 227 * 1024) return fail(c, PARO_ERR_ARG, "position gradient: grid too long for shared memory");
-  PARO_CU(c, cudaFuncSetAttribute(k_vloc_force, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smf));
+  const size_t smf_max = 226 * 1024;  // beside the kernel's static shared memory; fft3d stops at N3 = 375 (192 KB here)
+  if (smf > smf_max) return fail(c, PARO_ERR_ARG, "position gradient: grid too long for shared memory");
+  // the most there is, not this grid's need: the limit is the kernel's, and another thread's context with a shorter
+  // grid would take it back between this call and the launch
+  PARO_CU(c, cudaFuncSetAttribute(k_vloc_force, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smf_max));
   k_vloc_force<<<dim3(nchunk, (c->nat + 7) / 8), 256, smf, c->stream>>>(c->N[0], c->N[1], c->N[2], B, c->nat, ph, g,
                                                                        part);
   PARO_LAUNCH(c, "k_vloc_force");
