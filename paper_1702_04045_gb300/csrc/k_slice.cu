@@ -872,22 +872,9 @@ template <> const double2* slice_beta<double>(const Basis& b) { return b.d_beta;
 template <> const float2* slice_beta<float>(const Basis& b) { return b.d_beta32; }
 
 template <typename T>
-static int slice_beta_images(Ctx* c, int ik) {
-  constexpr int L = SliceL<T>::value, q = sizeof(T) == 8 ? 1 : 0;
-  Basis& B = c->bases[ik];
-  SliceImages& im = B.beta_slices[q];
-  if (im.cn) return PARO_OK;
+static int slice_form_beta(Ctx* c, const Basis& B, const SliceImages& im, int ma, int na, int scn, int swx) {
+  constexpr int L = SliceL<T>::value;
   const int np = c->nproj, npw = B.npw;
-  const int ma = round_up(np, kSliceM), na = round_up(npw, kSliceM);
-  const int scn = (npw + kSliceK - 1) / kSliceK, swx = (np + kSliceK - 1) / kSliceK;
-  const size_t bcn = (size_t)(ma / kSliceM) * scn * slice_a_bytes<L>();
-  const size_t bwx = (size_t)(na / kSliceM) * swx * slice_a_bytes<L>();
-  unsigned char* p = nullptr;  // [cn image | wx image | cn scales | wx scales]
-  PARO_CU(c, cudaMalloc(&p, bcn + bwx + (size_t)(ma + na) * sizeof(int)));
-  im.cn = p;
-  im.wx = p + bcn;
-  im.ecn = reinterpret_cast<int*>(p + bcn + bwx);
-  im.ewx = im.ecn + ma;
   int* rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)np * sizeof(int)));
   if (!rowkey) return PARO_ERR_CUDA;
   int st = slice_rowkeys<T>(c, np, npw, slice_beta<T>(B), npw, false, rowkey);
@@ -900,6 +887,32 @@ static int slice_beta_images(Ctx* c, int ik) {
   k_slice_cols<T, L><<<na / 32, 256, 0, c->stream>>>(npw, np, swx, slice_beta<T>(B), npw, nullptr, im.wx,
                                                         im.ewx);
   PARO_LAUNCH(c, "k_slice_cols");
+  return PARO_OK;
+}
+
+template <typename T>
+static int slice_beta_images(Ctx* c, int ik) {
+  constexpr int L = SliceL<T>::value, q = sizeof(T) == 8 ? 1 : 0;
+  Basis& B = c->bases[ik];
+  if (B.beta_slices[q].cn) return PARO_OK;
+  const int np = c->nproj, npw = B.npw;
+  const int ma = round_up(np, kSliceM), na = round_up(npw, kSliceM);
+  const int scn = (npw + kSliceK - 1) / kSliceK, swx = (np + kSliceK - 1) / kSliceK;
+  const size_t bcn = (size_t)(ma / kSliceM) * scn * slice_a_bytes<L>();
+  const size_t bwx = (size_t)(na / kSliceM) * swx * slice_a_bytes<L>();
+  unsigned char* p = nullptr;  // [cn image | wx image | cn scales | wx scales]
+  PARO_CU(c, cudaMalloc(&p, bcn + bwx + (size_t)(ma + na) * sizeof(int)));
+  SliceImages im;
+  im.cn = p;
+  im.wx = p + bcn;
+  im.ecn = reinterpret_cast<int*>(p + bcn + bwx);
+  im.ewx = im.ecn + ma;
+  if (int st = slice_form_beta<T>(c, B, im, ma, na, scn, swx)) {
+    cudaStreamSynchronize(c->stream);
+    cudaFree(p);
+    return st;
+  }
+  B.beta_slices[q] = im;  // marks the images as formed
   return PARO_OK;
 }
 
