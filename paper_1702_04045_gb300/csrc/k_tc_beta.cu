@@ -73,14 +73,24 @@ int beta_images(Ctx* c, int ik) {
   B.img_wx_nstage = (c->nproj + kBKC - 1) / kBKC;
   const size_t ncn = (size_t)mtiles * B.img_cn_nstage * 2 * kTileF4;
   const size_t nwx = (size_t)ntiles * B.img_wx_nstage * 2 * kTileF4;
-  PARO_CU(c, cudaMalloc(&B.d_beta_img_cn, ncn * sizeof(float4)));
-  PARO_CU(c, cudaMalloc(&B.d_beta_img_wx, nwx * sizeof(float4)));
-  k_beta_img_cn<<<dim3(304, mtiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_cn_nstage, B.d_beta32,
-                                                          B.d_beta_img_cn);
-  PARO_LAUNCH(c, "k_beta_img_cn");
-  k_beta_img_wx<<<dim3(8, ntiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_wx_nstage, B.d_beta32,
-                                                        B.d_beta_img_wx);
-  PARO_LAUNCH(c, "k_beta_img_wx");
+  float4 *cn = nullptr, *wx = nullptr;
+  auto form = [&]() -> int {
+    PARO_CU(c, cudaMalloc(&cn, ncn * sizeof(float4)));
+    PARO_CU(c, cudaMalloc(&wx, nwx * sizeof(float4)));
+    k_beta_img_cn<<<dim3(304, mtiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_cn_nstage, B.d_beta32, cn);
+    PARO_LAUNCH(c, "k_beta_img_cn");
+    k_beta_img_wx<<<dim3(8, ntiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_wx_nstage, B.d_beta32, wx);
+    PARO_LAUNCH(c, "k_beta_img_wx");
+    return PARO_OK;
+  };
+  if (int st = form()) {
+    cudaStreamSynchronize(c->stream);
+    if (cn) cudaFree(cn);
+    if (wx) cudaFree(wx);
+    return st;
+  }
+  B.d_beta_img_cn = cn;  // set only now: they mark the images as formed
+  B.d_beta_img_wx = wx;
   return PARO_OK;
 }
 

@@ -1,4 +1,4 @@
-"""A failure while the projectors' digit images are formed leaves no half-formed images behind: the call that met it
+"""A failure while the projectors' images (digit images, and the TF32 images of the inner solves) are formed leaves no half-formed images behind: the call that met it
 reports it, and the next one, which finds nothing in its way, returns the right values. The failure is an error that
 another part of the process left pending in the CUDA runtime (an allocation refused), which the library's first check
 after a launch picks up."""
@@ -14,8 +14,10 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("precision,dtype,tol", [("fp64", torch.complex128, 1e-12), ("mixed", torch.complex64, 2e-6)])
-def test_products_after_a_failure_are_right(precision, dtype, tol):
+@pytest.mark.parametrize("precision,dtype,tol,form", [("fp64", torch.complex128, 1e-12, 0),
+                                                      ("mixed", torch.complex64, 2e-6, 0),
+                                                      ("mixed", torch.complex64, 3e-5, 1)])
+def test_products_after_a_failure_are_right(precision, dtype, tol, form):
     from paper_1702_04045_gb300 import paro
 
     def context():
@@ -23,7 +25,7 @@ def test_products_after_a_failure_are_right(precision, dtype, tol):
         return ctx, torch.from_numpy(inputs.start_vectors(144, ctx.npw(), 3)).to(dtype).cuda()
 
     ctx, x = context()
-    ref = ctx.apply_vnl(x).clone()
+    ref = ctx.apply_vnl(x, form).clone()
     ctx.close()
     ctx, x = context()
     out = torch.empty_like(x)
@@ -36,7 +38,7 @@ def test_products_after_a_failure_are_right(precision, dtype, tol):
 
     def call():
         return ctx.lib.paro_apply_vnl(ctx.h, 0, x.shape[0], paro.PARO_C64 if tol == 1e-12 else paro.PARO_C32,
-                                      ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()), 0)
+                                      ctypes.c_void_p(x.data_ptr()), ctypes.c_void_p(out.data_ptr()), form)
 
     assert rt.cudaMalloc(ctypes.byref(ptr), ctypes.c_size_t(1 << 60)) != 0
     first = call()
