@@ -22,6 +22,9 @@ Ctx* unwrap(paro_ctx* h) { return h ? &h->c : nullptr; }
 
 int fail(Ctx* c, int code, const std::string& msg) {
   if (c) c->err = msg;
+  // a refused allocation or launch is reported here, so it does not stay pending in the runtime for the next launch
+  // check, of another context or of the caller's own code (an error that lost the device stays)
+  if (code == PARO_ERR_CUDA) cudaGetLastError();
   return code;
 }
 

@@ -724,6 +724,7 @@ namespace {
 int berr(paro_batch* b, int code, const std::string& msg) {
   b->err = msg;
   if (b->lead) b->lead->err = msg;
+  if (code == PARO_ERR_CUDA) cudaGetLastError();  // as in fail()
   return code;
 }
 
@@ -1147,6 +1148,7 @@ int paro_batch_create(paro_batch** out, paro_ctx* const* ctxs, int n_ctx) {
   auto bail = [&](int code, const std::string& msg) {
     b->lead->err = msg;
     free_batch(b);
+    if (code == PARO_ERR_CUDA) cudaGetLastError();  // as in fail()
     return code;
   };
   size_t off = 0, max_el = 0, soff = 0, dpoff = 0;

@@ -303,8 +303,14 @@ bool tc_enabled() {
 
 int* tc_err_flag(Ctx* c) {
   if (!c->d_tc_err) {
-    if (cudaMalloc(&c->d_tc_err, sizeof(int)) != cudaSuccess) return nullptr;
-    if (cudaMemsetAsync(c->d_tc_err, 0, sizeof(int), c->stream) != cudaSuccess) return nullptr;
+    cudaError_t e = cudaMalloc(&c->d_tc_err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->d_tc_err, 0, sizeof(int), c->stream);
+    if (e != cudaSuccess) {
+      if (c->d_tc_err) cudaFree(c->d_tc_err);
+      c->d_tc_err = nullptr;
+      cuda_fail(c, e, "tensor-core error flag");
+      return nullptr;
+    }
   }
   return c->d_tc_err;
 }
