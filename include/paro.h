@@ -12,6 +12,11 @@
  *   - The caller owns every array argument; the library copies what it keeps. The library owns the
  *     context and all of its device buffers. Device pointers must stay valid for the duration of the
  *     call. All GPU work is enqueued on the context's stream; calls that return host data synchronise.
+ *   - Beside what a call cannot do without, contexts keep device memory that makes products faster: images of
+ *     the projectors (56 bytes an entry of their n_proj x npw table for PARO_C64, 32 for large PARO_C32
+ *     products, as long as the positions stay) and of the operands of FP64 products (up to 70 bytes a
+ *     coefficient). When an allocation is refused the call does without them, and what a context holds of
+ *     them is given back before one of its own allocations fails.
  *   - The tensor-core kernels' waits are bounded. A call that waits for the GPU (paro_apply_vnl,
  *     paro_solve_source, paro_orthonormalize, paro_energy, the ParO and SCF steps and every call that takes
  *     Ritz pairs or residuals) returns PARO_ERR_TIMEOUT when such a wait gave up in it or in an

@@ -32,21 +32,61 @@ int cuda_fail(Ctx* c, cudaError_t e, const char* where) {
   return fail(c, PARO_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
-void* ws_get(Ctx* c, const char* name, size_t bytes) {
+void ws_drop(Ctx* c, const char* name) {
+  auto it = c->ws.find(name);
+  if (it == c->ws.end()) return;
+  cudaStreamSynchronize(c->stream);
+  cudaFree(it->second.first);
+  c->ws.erase(it);
+}
+
+static void* ws_alloc(Ctx* c, const char* name, size_t bytes, cudaError_t* e) {
+  *e = cudaSuccess;
   auto it = c->ws.find(name);
   if (it != c->ws.end() && it->second.second >= bytes) return it->second.first;
-  if (it != c->ws.end()) {
-    cudaStreamSynchronize(c->stream);
-    cudaFree(it->second.first);
-    c->ws.erase(it);
-  }
+  ws_drop(c, name);
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes > 0 ? bytes : 16);
-  if (e != cudaSuccess) {
-    cuda_fail(c, e, "workspace allocation");
+  *e = cudaMalloc(&p, bytes > 0 ? bytes : 16);
+  if (*e != cudaSuccess) {
+    cudaGetLastError();  // as in fail()
     return nullptr;
   }
   c->ws[name] = std::make_pair(p, bytes);
+  return p;
+}
+
+void* ws_try(Ctx* c, const char* name, size_t bytes) {
+  cudaError_t e;
+  return ws_alloc(c, name, bytes, &e);
+}
+
+bool drop_optional(Ctx* c) {
+  if (c->optional_in_use) return false;
+  bool any = false;
+  for (const char* name : {"slice_a", "slice_b", "adj_y32", "adj_y64"})
+    if (c->ws.count(name)) {
+      ws_drop(c, name);
+      any = true;
+    }
+  for (Basis& b : c->bases)
+    for (SliceImages& im : b.beta_slices)
+      if (im.cn) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(im.cn);
+        im = SliceImages();
+        any = true;
+      }
+  return any;
+}
+
+void* ws_get(Ctx* c, const char* name, size_t bytes) {
+  cudaError_t e;
+  void* p = ws_alloc(c, name, bytes, &e);
+  if (!p && e == cudaErrorMemoryAllocation && drop_optional(c)) p = ws_alloc(c, name, bytes, &e);
+  if (!p) {
+    c->ws_short = true;
+    cuda_fail(c, e, "workspace allocation");
+  }
   return p;
 }
 

@@ -43,26 +43,30 @@ struct Rec3 {
   double m[9];
 };
 
-// Y[a nb + b][g] = (k + G_g)_a X[b][g] for the three directions; a thread takes one plane wave of 16 bands, its
-// q in FP64 once. The FP32 product is x q_hi + x q_lo with q split into two floats: the FP64 product's rounding.
+// Y[a nb + b][g] = (k + G_g)_a X[b][g] for the three directions (NA = 3, a0 = 0) or for direction a0 alone (NA = 1); a
+// thread takes one plane wave of 16 bands, its q in FP64 once. The FP32 product is x q_hi + x q_lo with q split into
+// two floats: the FP64 product's rounding.
 static const int kQBands = 16;
-template <typename T>
-__global__ void k_scale_q(int npw, int nb, const int* __restrict__ miller, Rec3 B, double kx, double ky, double kz,
-                          const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Y) {
+template <typename T, int NA>
+__global__ void k_scale_q(int npw, int nb, int a0, const int* __restrict__ miller, Rec3 B, double kx, double ky,
+                          double kz, const cplx<T>* __restrict__ X, cplx<T>* __restrict__ Y) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= npw) return;
   const int n1 = miller[3 * g], n2 = miller[3 * g + 1], n3 = miller[3 * g + 2];
   const double k[3] = {kx, ky, kz};
-  double q[3];
+  double q[NA];
 #pragma unroll
-  for (int al = 0; al < 3; ++al) q[al] = k[al] + n1 * B.m[al] + n2 * B.m[3 + al] + n3 * B.m[6 + al];
+  for (int i = 0; i < NA; ++i) {
+    const int al = NA == 3 ? i : a0;
+    q[i] = k[al] + n1 * B.m[al] + n2 * B.m[3 + al] + n3 * B.m[6 + al];
+  }
   const int b1 = min(nb, (int)(blockIdx.y + 1) * kQBands);
   const size_t step = (size_t)nb * npw;
   for (int b = blockIdx.y * kQBands; b < b1; ++b) {
     const size_t o = (size_t)b * npw + g;
     const cplx<T> x = X[o];
 #pragma unroll
-    for (int al = 0; al < 3; ++al) {
+    for (int al = 0; al < NA; ++al) {
       if constexpr (sizeof(T) == 4) {
         const float qh = (float)q[al], ql = (float)(q[al] - (double)qh);
         Y[al * step + o] = make_float2(fmaf(qh, x.x, ql * x.x), fmaf(qh, x.y, ql * x.y));
@@ -74,10 +78,11 @@ __global__ void k_scale_q(int npw, int nb, const int* __restrict__ miller, Rec3 
 }
 
 // gpos[I][a] += sum_{p in I} D_p sum_b Re[i (conj(A) P^a - conj(A^a) P)] = -sum D_p sum_b Im(...)
-// P, A: nproj x nb complex (row p); Q: nproj x 6 nb, columns [P^x P^y P^z A^x A^y A^z]. One CTA per atom.
+// P, A: nproj x nb complex (row p); Q: [P^x P^y P^z A^x A^y A^z], each nproj x nb with rows rs and blocks bs apart. One
+// CTA per atom.
 __global__ void __launch_bounds__(256) k_kb_force(int nb, const double2* __restrict__ P, const double2* __restrict__ A,
-                                                  const double2* __restrict__ Q, const double* __restrict__ dvec,
-                                                  double* __restrict__ gpos) {
+                                                  const double2* __restrict__ Q, size_t rs, size_t bs,
+                                                  const double* __restrict__ dvec, double* __restrict__ gpos) {
   __shared__ double red[32];
   const int I = blockIdx.x;
   for (int al = 0; al < 3; ++al) {
@@ -85,7 +90,7 @@ __global__ void __launch_bounds__(256) k_kb_force(int nb, const double2* __restr
     for (int t = threadIdx.x; t < 4 * nb; t += blockDim.x) {
       const int p = 4 * I + t / nb, b = t % nb;
       const double2 a = A[(size_t)p * nb + b], pp = P[(size_t)p * nb + b];
-      const double2 pa = Q[(size_t)p * 6 * nb + al * nb + b], aa = Q[(size_t)p * 6 * nb + (3 + al) * nb + b];
+      const double2 pa = Q[p * rs + al * bs + b], aa = Q[p * rs + (3 + al) * bs + b];
       // Im(conj(a) pa - conj(aa) pp)
       const double im = (a.x * pa.y - a.y * pa.x) - (aa.x * pp.y - aa.y * pp.x);
       acc -= dvec[p] * im;
@@ -133,22 +138,51 @@ static int hpsi_adjoint(Ctx* c, int ik, int nb, const cplx<T>* psi, const cplx<T
   const int np = c->nproj;
   const size_t mat = (size_t)np * nb;
   double2* M = static_cast<double2*>(ws_get(c, "adj_proj", 8 * mat * sizeof(double2)));
-  cplx<T>* Y = static_cast<cplx<T>*>(ws_get(c, f64 ? "adj_y64" : "adj_y32", (size_t)6 * nb * npw * sizeof(cplx<T>)));
-  if (!M || !Y) return PARO_ERR_CUDA;
+  if (!M) return PARO_ERR_CUDA;
   double2 *P = M, *A = M + mat, *Q = M + 2 * mat;
   Rec3 R;
   for (int i = 0; i < 9; ++i) R.m[i] = c->bmat[i];
   const dim3 gq((npw + 255) / 256, (nb + kQBands - 1) / kQBands);
-  for (int h = 0; h < 2; ++h) {
-    k_scale_q<T><<<gq, 256, 0, c->stream>>>(npw, nb, B.d_miller, R, B.kcart[0], B.kcart[1], B.kcart[2], h ? w : psi,
-                                            Y + (size_t)3 * h * nb * npw);
-    PARO_LAUNCH(c, "k_scale_q");
-  }
+  const char* yname = f64 ? "adj_y64" : "adj_y32";
   // the projections of psi, w and of the six weighted blocks: three products with the projectors' images
-  if ((st = kb_project<T>(c, ik, nb, psi, P)) || (st = kb_project<T>(c, ik, nb, w, A)) ||
-      (st = kb_project<T>(c, ik, 6 * nb, Y, Q, nb)))
-    return st;
-  k_kb_force<<<c->nat, 256, 0, c->stream>>>(nb, P, A, Q, c->d_dvec, gpos);
+  if ((st = kb_project<T>(c, ik, nb, psi, P)) || (st = kb_project<T>(c, ik, nb, w, A))) return st;
+  auto together = [&]() -> int {
+    OptionalInUse use(c);
+    cplx<T>* Y = static_cast<cplx<T>*>(ws_try(c, yname, (size_t)6 * nb * npw * sizeof(cplx<T>)));
+    if (!Y) return kNoMemory;
+    for (int h = 0; h < 2; ++h) {
+      k_scale_q<T, 3><<<gq, 256, 0, c->stream>>>(npw, nb, 0, B.d_miller, R, B.kcart[0], B.kcart[1], B.kcart[2],
+                                                 h ? w : psi, Y + (size_t)3 * h * nb * npw);
+      PARO_LAUNCH(c, "k_scale_q");
+    }
+    c->ws_short = false;
+    const int s2 = kb_project<T>(c, ik, 6 * nb, Y, Q, nb);
+    return s2 == PARO_ERR_CUDA && c->ws_short ? kNoMemory : s2;
+  };
+  // one by one where memory for the six (and for the parts of their product) is short
+  auto singly = [&]() -> int {
+    ws_drop(c, yname);
+    cplx<T>* Y = static_cast<cplx<T>*>(ws_get(c, yname, (size_t)nb * npw * sizeof(cplx<T>)));
+    if (!Y) return PARO_ERR_CUDA;
+    OptionalInUse use(c);
+    for (int i = 0; i < 6; ++i) {
+      k_scale_q<T, 1><<<gq, 256, 0, c->stream>>>(npw, nb, i % 3, B.d_miller, R, B.kcart[0], B.kcart[1], B.kcart[2],
+                                                 i < 3 ? psi : w, Y);
+      PARO_LAUNCH(c, "k_scale_q");
+      if (int s2 = kb_project<T>(c, ik, nb, Y, Q + i * mat, nb)) return s2;
+    }
+    return PARO_OK;
+  };
+  size_t rs = (size_t)6 * nb, bs = nb;
+  st = together();
+  if (st == kNoMemory) {
+    rs = nb;
+    bs = mat;
+    c->err.clear();
+    st = singly();
+  }
+  if (st) return st;
+  k_kb_force<<<c->nat, 256, 0, c->stream>>>(nb, P, A, Q, rs, bs, c->d_dvec, gpos);
   PARO_LAUNCH(c, "k_kb_force");
   return PARO_OK;
 }

@@ -311,7 +311,10 @@ int kb_project(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P, int plan_
       return PARO_OK;
     }
   }
-  if (kb_slices(c, ik, nb, sizeof(T) == 8)) return kb_project_slice<T>(c, ik, nb, psi, P);
+  if (kb_slices(c, ik, nb, sizeof(T) == 8)) {
+    const int st = kb_project_slice<T>(c, ik, nb, psi, P);
+    if (st != kNoMemory) return st;
+  }
   const bool carry = sizeof(T) == 4 && !c->tc_scope;
   return gemm_cn<T, T, T>(c, c->nproj, nb, B.npw, beta_of<T>(B), B.npw, psi, B.npw, P, nb, false, carry);
 }
@@ -351,7 +354,10 @@ int kb_apply(Ctx* c, int ik, int nb, const cplx<T>* psi, cplx<T>* hpsi) {
       return PARO_OK;
     }
   }
-  if (kb_slices(c, ik, nb, sizeof(T) == 8)) return kb_update_slice<T>(c, ik, nb, P, hpsi);
+  if (kb_slices(c, ik, nb, sizeof(T) == 8)) {
+    st = kb_update_slice<T>(c, ik, nb, P, hpsi);
+    if (st != kNoMemory) return st;
+  }
   // W(k = p, m = b) = D_p P[p][b]
   return gemm_wx<T, T>(c, nb, B.npw, c->nproj, P, nb, false, c->d_dvec, beta_of<T>(B), B.npw, hpsi, B.npw, 1.0);
 }

@@ -345,7 +345,10 @@ int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<
   if constexpr (sizeof(TA) == 8 && sizeof(TB) == 8) {
     // at every size the digit slices are faster than the FP64 pipe (Gram and V_nl of one 1189-coefficient row: 335 -> 85 us and 367 -> 70 us with the
     // steps around them; 144 rows of 23847: 8.8 -> 0.81 ms and 17.7 -> 0.68 ms)
-    if (K > 0 && slices_on(c)) return gemm_cn_slice<double>(c, M, N, K, A, lda, B, ldb, C, ldc, herm);
+    if (K > 0 && slices_on(c)) {
+      const int st = gemm_cn_slice<double>(c, M, N, K, A, lda, B, ldb, C, ldc, herm);
+      if (st != kNoMemory) return st;
+    }
   }
   const int r = pick_r(M, N, herm), tile = 16 * r;
   const int tiles_m = (M + tile - 1) / tile, tiles_n = (N + tile - 1) / tile;
@@ -627,8 +630,10 @@ int gemm_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool wt, con
     return PARO_OK;
   }
   if constexpr (sizeof(TX) == 8 && sizeof(TY) == 8) {
-    if (K > 0 && slices_on(c) && (beta == 0.0 || beta == 1.0))
-      return gemm_wx_slice<double>(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta != 0.0, lower);
+    if (K > 0 && slices_on(c) && (beta == 0.0 || beta == 1.0)) {
+      const int st = gemm_wx_slice<double>(c, M, N, K, W, ldw, wt, s, X, ldx, Y, ldy, beta != 0.0, lower);
+      if (st != kNoMemory) return st;
+    }
   }
   cudaEvent_t ev = prof_begin(c);
   if ((M + 47) / 48 * 48 < (M + 31) / 32 * 32)
@@ -1288,21 +1293,22 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
       int piece = 0, nflag = 0;
       if ((st = chol_piece(c, &piece))) return st;
       if (piece > 0 && n > piece) {
-        int* flags = static_cast<int*>(ws_get(c, "chol_split_flags", 64 * sizeof(int)));
+        int* flags = static_cast<int*>(ws_try(c, "chol_split_flags", 64 * sizeof(int)));
         // S, then per level the cluster kernel's blocks and L21, T (their sum stays below 2 n^2)
         const size_t nn = (size_t)n * n, levels = (size_t)(n + piece - 1) / piece;
         double2* W = static_cast<double2*>(
-            ws_get(c, "chol_split", (3 * nn + 2 * levels * piece * piece) * sizeof(double2)));
-        if (!flags || !W) return PARO_ERR_CUDA;
-        PARO_CU(c, cudaMemcpyAsync(W, s, nn * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
-        if ((st = chol_split(c, n, W, n, g, n, W + nn, piece, flags, &nflag))) return st;
-        int h[64];
-        PARO_CU(c, cudaMemcpyAsync(h, flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        PARO_CU(c, cudaStreamSynchronize(c->stream));
-        for (int i = 0; i < nflag; ++i)
-          if (h[i]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 in block " + std::to_string(i) + ", column " +
-                                                           std::to_string(h[i] - 1));
-        return PARO_OK;
+            ws_try(c, "chol_split", (3 * nn + 2 * levels * piece * piece) * sizeof(double2)));
+        if (flags && W) {  // else the kernels below, which take two thirds of it or none
+          PARO_CU(c, cudaMemcpyAsync(W, s, nn * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
+          if ((st = chol_split(c, n, W, n, g, n, W + nn, piece, flags, &nflag))) return st;
+          int h[64];
+          PARO_CU(c, cudaMemcpyAsync(h, flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+          PARO_CU(c, cudaStreamSynchronize(c->stream));
+          for (int i = 0; i < nflag; ++i)
+            if (h[i]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 in block " + std::to_string(i) +
+                                                             ", column " + std::to_string(h[i] - 1));
+          return PARO_OK;
+        }
       }
       if ((st = chol_cluster_shape(c, n, &sh))) return st;
     }

@@ -789,17 +789,18 @@ static int slice_cn(Ctx* c, int M, int N, int K, const cplx<T>* A, int lda, cons
   const int ma = mt * kSliceM, nb = nt * NC;
   const bool same = !a_img && A == B && lda == ldb && M == N;
   const int pad = same ? std::max(ma, nb) : nb;
-  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)nt * nstage * slice_b_bytes<L>(NC)));
-  int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)nz * pad * sizeof(int)));
-  double2* part = static_cast<double2*>(ws_get(c, "gemm_parts", (size_t)nz * M * N * sizeof(double2)));
+  OptionalInUse use(c);
+  unsigned char* bi = static_cast<unsigned char*>(ws_try(c, "slice_b", (size_t)nt * nstage * slice_b_bytes<L>(NC)));
+  int* eb = static_cast<int*>(ws_try(c, "slice_eb", (size_t)nz * pad * sizeof(int)));
+  double2* part = static_cast<double2*>(ws_try(c, "gemm_parts", (size_t)nz * M * N * sizeof(double2)));
+  if (!bi || !eb || !part) return kNoMemory;
   unsigned char* ai = nullptr;
   int* ean = nullptr;
   if (!a_img) {
-    ai = static_cast<unsigned char*>(ws_get(c, "slice_a", (size_t)mt * nstage * slice_a_bytes<L>()));
-    ean = same ? eb : static_cast<int*>(ws_get(c, "slice_ea", (size_t)nz * ma * sizeof(int)));
-    if (!ai || !ean) return PARO_ERR_CUDA;
+    ai = static_cast<unsigned char*>(ws_try(c, "slice_a", (size_t)mt * nstage * slice_a_bytes<L>()));
+    ean = same ? eb : static_cast<int*>(ws_try(c, "slice_ea", (size_t)nz * ma * sizeof(int)));
+    if (!ai || !ean) return kNoMemory;
   }
-  if (!bi || !eb || !part) return PARO_ERR_CUDA;
   cudaEvent_t ev = prof_begin(c);
   int st;
   if (!a_img && !same && (st = slice_rows<T, L>(c, M, ma, 0, ma, K, ks * kSliceK, nz, nstage, A, lda, ai, nullptr, ean)))
@@ -832,17 +833,20 @@ static int slice_wx(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool
   constexpr int L = SliceL<T>::value;
   const int NC = slice_nc<L>(M);
   const int at = (N + kSliceM - 1) / kSliceM, bt = (M + NC - 1) / NC, nstage = (K + kSliceK - 1) / kSliceK;
-  unsigned char* bi = static_cast<unsigned char*>(ws_get(c, "slice_b", (size_t)bt * nstage * slice_b_bytes<L>(NC)));
-  int* eb = static_cast<int*>(ws_get(c, "slice_eb", (size_t)bt * NC * sizeof(int)));
-  if (!bi || !eb) return PARO_ERR_CUDA;
-  int* rowkey = nullptr;
+  OptionalInUse use(c);
+  unsigned char* bi = static_cast<unsigned char*>(ws_try(c, "slice_b", (size_t)bt * nstage * slice_b_bytes<L>(NC)));
+  int* eb = static_cast<int*>(ws_try(c, "slice_eb", (size_t)bt * NC * sizeof(int)));
+  if (!bi || !eb) return kNoMemory;
+  unsigned char* ai = nullptr;
+  int *ean = nullptr, *rowkey = nullptr;
+  if (!a_img) {
+    ai = static_cast<unsigned char*>(ws_try(c, "slice_a", (size_t)at * nstage * slice_a_bytes<L>()));
+    ean = static_cast<int*>(ws_try(c, "slice_ea", (size_t)at * kSliceM * sizeof(int)));
+    rowkey = static_cast<int*>(ws_try(c, "slice_rowkey", (size_t)std::max(K, 1) * sizeof(int)));
+    if (!ai || !ean || !rowkey) return kNoMemory;
+  }
   cudaEvent_t ev = prof_begin(c);
   if (!a_img) {
-    unsigned char* ai = static_cast<unsigned char*>(ws_get(c, "slice_a", (size_t)at * nstage * slice_a_bytes<L>()));
-    int* ean = static_cast<int*>(ws_get(c, "slice_ea", (size_t)at * kSliceM * sizeof(int)));
-    if (!ai || !ean) return PARO_ERR_CUDA;
-    rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)std::max(K, 1) * sizeof(int)));
-    if (!rowkey) return PARO_ERR_CUDA;
     if (int st = slice_rowkeys<T>(c, K, N, X, ldx, true, rowkey)) return st;
     k_slice_cols<T, L><<<at * kSliceM / 32, 256, 0, c->stream>>>(N, K, nstage, X, ldx, rowkey, ai, ean);
     PARO_LAUNCH(c, "k_slice_cols");
@@ -867,16 +871,16 @@ int gemm_wx_slice(Ctx* c, int M, int N, int K, const double2* W, int ldw, bool w
 }
 
 // ---- the projectors as the fixed operand: their images change only with the atom positions ----
+// 32 bytes an entry of the projectors' table in FP32, 56 in FP64 (512 atoms in FP32: 9 GB beside a table of 2.2).
 template <typename T> static const cplx<T>* slice_beta(const Basis& b);
 template <> const double2* slice_beta<double>(const Basis& b) { return b.d_beta; }
 template <> const float2* slice_beta<float>(const Basis& b) { return b.d_beta32; }
 
 template <typename T>
-static int slice_form_beta(Ctx* c, const Basis& B, const SliceImages& im, int ma, int na, int scn, int swx) {
+static int slice_form_beta(Ctx* c, const Basis& B, const SliceImages& im, int* rowkey, int ma, int na, int scn,
+                           int swx) {
   constexpr int L = SliceL<T>::value;
   const int np = c->nproj, npw = B.npw;
-  int* rowkey = static_cast<int*>(ws_get(c, "slice_rowkey", (size_t)np * sizeof(int)));
-  if (!rowkey) return PARO_ERR_CUDA;
   int st = slice_rowkeys<T>(c, np, npw, slice_beta<T>(B), npw, false, rowkey);
   if (st) return st;
   const int nzi = std::max(1, std::min((npw + 511) / 512, 1216 / (ma / 8)));
@@ -900,14 +904,18 @@ static int slice_beta_images(Ctx* c, int ik) {
   const int scn = (npw + kSliceK - 1) / kSliceK, swx = (np + kSliceK - 1) / kSliceK;
   const size_t bcn = (size_t)(ma / kSliceM) * scn * slice_a_bytes<L>();
   const size_t bwx = (size_t)(na / kSliceM) * swx * slice_a_bytes<L>();
+  int* rowkey = static_cast<int*>(ws_try(c, "slice_rowkey", (size_t)np * sizeof(int)));
   unsigned char* p = nullptr;  // [cn image | wx image | cn scales | wx scales]
-  PARO_CU(c, cudaMalloc(&p, bcn + bwx + (size_t)(ma + na) * sizeof(int)));
+  if (!rowkey || cudaMalloc(&p, bcn + bwx + (size_t)(ma + na) * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    return kNoMemory;
+  }
   SliceImages im;
   im.cn = p;
   im.wx = p + bcn;
   im.ecn = reinterpret_cast<int*>(p + bcn + bwx);
   im.ewx = im.ecn + ma;
-  if (int st = slice_form_beta<T>(c, B, im, ma, na, scn, swx)) {
+  if (int st = slice_form_beta<T>(c, B, im, rowkey, ma, na, scn, swx)) {
     cudaStreamSynchronize(c->stream);
     cudaFree(p);
     return st;
@@ -918,6 +926,7 @@ static int slice_beta_images(Ctx* c, int ik) {
 
 template <typename T>
 int kb_project_slice(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P) {
+  OptionalInUse use(c);
   int st = slice_beta_images<T>(c, ik);
   if (st) return st;
   const Basis& B = c->bases[ik];
@@ -927,6 +936,7 @@ int kb_project_slice(Ctx* c, int ik, int nb, const cplx<T>* psi, double2* P) {
 
 template <typename T>
 int kb_update_slice(Ctx* c, int ik, int nb, const double2* P, cplx<T>* hpsi) {
+  OptionalInUse use(c);
   int st = slice_beta_images<T>(c, ik);
   if (st) return st;
   const Basis& B = c->bases[ik];

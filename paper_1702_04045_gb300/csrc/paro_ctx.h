@@ -149,6 +149,8 @@ struct Ctx {
   const char* prof_tag = nullptr;  // phase prefix of recorded names ("pcg", "rr", ...)
   // workspaces by name
   std::map<std::string, std::pair<void*, size_t>> ws;
+  int optional_in_use = 0;  // OptionalInUse scopes
+  bool ws_short = false;    // a workspace could not be had (set by ws_get)
   // pinned host buffers by name for the small copies of every iteration, each with the event of its last
   // copy: a buffer is rewritten only after that copy has completed, so no copy waits for the stream
   struct Pinned {
@@ -180,6 +182,15 @@ int fp64_current(Ctx* c, Basis& b);
 int fail(Ctx* c, int code, const std::string& msg);
 int cuda_fail(Ctx* c, cudaError_t e, const char* where);
 void* ws_get(Ctx* c, const char* name, size_t bytes);  // nullptr on failure (err set)
+// the same for memory that a call can do without: nullptr on failure, with nothing reported
+void* ws_try(Ctx* c, const char* name, size_t bytes);
+void ws_drop(Ctx* c, const char* name);  // waits for the stream and frees the workspace, if there is one
+// Memory that calls do without when it is short: the digit images of the projectors and of products' operands, and
+// the blocks the adjoint projects together. What cannot have them returns kNoMemory, before any launch, and its
+// caller takes the plain form. ws_get gives them up (drop_optional) before it fails, but not inside an OptionalInUse
+// scope, whose pointers they are.
+static const int kNoMemory = 1;
+bool drop_optional(Ctx* c);
 // host -> device copy on the context's stream through the pinned buffer `name`; src may change as soon as
 // this returns, and the call does not wait for the stream (only, rarely, for the buffer's previous copy)
 int h2d_async(Ctx* c, const char* name, void* dst, const void* src, size_t bytes);
@@ -226,6 +237,11 @@ struct PlainF64 {
     ctx->plain64 = always || ctx->prec == PARO_FP64;
   }
   ~PlainF64() { c->plain64 = old; }
+};
+struct OptionalInUse {
+  Ctx* c;
+  explicit OptionalInUse(Ctx* ctx) : c(ctx) { ++c->optional_in_use; }
+  ~OptionalInUse() { --c->optional_in_use; }
 };
 // Scoped phase tag: names recorded inside become "tag:name".
 struct ProfTag {
