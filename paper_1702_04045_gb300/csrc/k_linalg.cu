@@ -1244,7 +1244,7 @@ static int chol_split(Ctx* c, int n, double2* S, int lds, double2* G, int ldg, d
   Ctx::CholShape sh;
   int st = chol_cluster_shape(c, n1, &sh);
   if (st) return st;
-  if (sh.kind == 0 || *nflag >= 64) return fail(c, PARO_ERR_CUDA, "Cholesky: cluster kernel not available");
+  if (sh.kind == 0) return fail(c, PARO_ERR_CUDA, "Cholesky: cluster kernel not available");
   copy(n1, n1, S, lds, s1, n1);
   PARO_LAUNCH(c, "k_zcopy");
   if ((st = launch_chol_cluster(c, sh, n1, s1, g1, flags + (*nflag)++, nullptr))) return st;
@@ -1293,16 +1293,17 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
       int piece = 0, nflag = 0;
       if ((st = chol_piece(c, &piece))) return st;
       if (piece > 0 && n > piece) {
-        int* flags = static_cast<int*>(ws_try(c, "chol_split_flags", 64 * sizeof(int)));
-        // S, then per level the cluster kernel's blocks and L21, T (their sum stays below 2 n^2)
+        // S, then per level the cluster kernel's blocks and L21, T (their sum stays below 2 n^2); a breakdown flag a
+        // level (a level leaves at most (levels - 1) / levels of its rows to the next, so there are no more of them)
         const size_t nn = (size_t)n * n, levels = (size_t)(n + piece - 1) / piece;
+        int* flags = static_cast<int*>(ws_try(c, "chol_split_flags", levels * sizeof(int)));
         double2* W = static_cast<double2*>(
             ws_try(c, "chol_split", (3 * nn + 2 * levels * piece * piece) * sizeof(double2)));
         if (flags && W) {  // else the kernels below, which take two thirds of it or none
           PARO_CU(c, cudaMemcpyAsync(W, s, nn * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
           if ((st = chol_split(c, n, W, n, g, n, W + nn, piece, flags, &nflag))) return st;
-          int h[64];
-          PARO_CU(c, cudaMemcpyAsync(h, flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+          std::vector<int> h(nflag);
+          PARO_CU(c, cudaMemcpyAsync(h.data(), flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
           PARO_CU(c, cudaStreamSynchronize(c->stream));
           for (int i = 0; i < nflag; ++i)
             if (h[i]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 in block " + std::to_string(i) +
