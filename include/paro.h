@@ -261,9 +261,10 @@ int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* p
  *   within 227 KB; otherwise PARO_ERR_ARG). The call times, on the batch's own problems, the unit shapes
  *   (32, 64 or 128 sticks per z-FFT unit; planes per unit for about 2048, 4096 or 8192 points), the launch
  *   forms (one cooperative launch with grid barriers between the phases, or one launch per phase and
- *   grid, with the line FFTs in registers on cubic grids of 27 to 72 points) and the grids, and keeps the
- *   fastest (paro_batch_tuning). The batch refers to the contexts, which must
- *   outlive it.
+ *   grid) and the grids, and keeps the fastest (paro_batch_tuning). With a cubic grid of 27, 32, 36, 48, 54,
+ *   64 or 72 points in the batch only the second form is timed: those grids have their line FFTs in
+ *   registers there, and the results may not depend on the search. The batch refers to the contexts, which
+ *   must outlive it.
  * paro_batch_apply_h -- H psi of every problem: psi[i], hpsi[i] device n_bands x npw arrays of dtype
  *   (the contexts' precision: PARO_C64 for FP64, PARO_C32 for mixed) of problem i. Enqueued on the
  *   contexts' stream.
@@ -276,8 +277,7 @@ int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* p
  *   Errors: PARO_ERR_BREAKDOWN (PCG or Cholesky), PARO_ERR_NOT_CONVERGED (Jacobi), PARO_ERR_TIMEOUT (a
  *   bounded grid-barrier wait gave up).
  * paro_batch_info -- problems, (problem, band) items, H psi launches per apply (1, or 3 for the form with
- *   launches per phase), its grid, and
- *   kernels launched per captured step (0 before the first step).
+ *   launches per phase), its grid, and kernels launched per captured step (0 before the first step).
  */
 typedef struct paro_batch paro_batch;
 int paro_batch_create(paro_batch** out, paro_ctx* const* ctxs, int n_ctx);

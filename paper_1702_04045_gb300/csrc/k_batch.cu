@@ -1032,7 +1032,15 @@ int autotune(paro_batch* b) {
   float best = 1e30f;
   int best_sg = 64, best_ppt = 4096;
   b->tuning.clear();
-  // unit shapes x launch form (one cooperative launch, or one launch per phase) x grid (CTAs per SM)
+  // Unit shapes x launch form (one cooperative launch, or one launch per phase) x grid (CTAs per SM). The cooperative
+  // form has the shared-memory FFTs only, whose rounding is not that of the line FFTs, so a batch with a grid of
+  // theirs keeps to a launch per phase: its results follow from its problems, not from this search's clock. (The other
+  // grids' operations are the same in both forms.) The line FFTs win at every size: 32 points, one orbital 38 us against
+  // 63 in FP64 and 21 against 30 in FP32, 80 orbitals 105 against 393 and 38 against 112. Without projectors or other
+  // grids nothing depends on the shapes and grids.
+  const bool lines_only = !b->groups.empty() &&
+                          std::all_of(b->hprob.begin(), b->hprob.end(),
+                                      [&](const ProbDev& P) { return P.nproj == 0 && line_covered(b, P); });
   for (int sg : {32, 64, 128})
     for (int ppt : {2048, 4096, 8192}) {
       if (build_lists(b, sg, ppt) != PARO_OK) continue;  // the unit does not fit shared memory
@@ -1043,13 +1051,14 @@ int autotune(paro_batch* b) {
         BCU(b, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
       }
       for (int mode : {0, 1}) {
+        if (mode == 0 && !b->groups.empty()) continue;
         int per_sm = 0;
         if (mode == 0)
           BCU(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hpsi_batch<T, 0>, 256, b->smem));
         else
           BCU(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hpsi_batch<T, 2>, 256, b->smem));
         for (int mult : {1, 2, 4, 8}) {  // mode 0: co-resident CTAs only
-          if (mult > per_sm) break;
+          if (mult > per_sm || (lines_only && mult > 1)) break;
           const int grid = mult * sms;
           int st;
           if ((st = launch_fused<T>(b, b->st, X, Y, nullptr, 0, mode, grid))) return st;
