@@ -1016,13 +1016,22 @@ int build_lists(paro_batch* b, int sg, int ppt) {
   return PARO_OK;
 }
 
+// All the dynamic shared memory a kernel can be given: the limit is the kernel's, and a limit at one batch's need would
+// be taken away from the batches that live beside it
+cudaError_t smem_all(const void* fn) {
+  cudaFuncAttributes at;
+  const cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)at.sharedSizeBytes);
+}
+
 template <typename T>
 int autotune(paro_batch* b) {
   int dev = 0, sms = 0;
   BCU(b, cudaGetDevice(&dev));
   BCU(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  BCU(b, cudaFuncSetAttribute(k_bjacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->small_smem));
-  BCU(b, cudaFuncSetAttribute(k_bchol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->small_smem));
+  BCU(b, smem_all((const void*)k_bjacobi));
+  BCU(b, smem_all((const void*)k_bchol));
   cplx<T>* X = static_cast<cplx<T>*>(b->p);
   cplx<T>* Y = static_cast<cplx<T>*>(b->ap);
   BCU(b, cudaMemsetAsync(X, 0, b->nelem * sizeof(cplx<T>), b->st));
@@ -1041,15 +1050,12 @@ int autotune(paro_batch* b) {
   const bool lines_only = !b->groups.empty() &&
                           std::all_of(b->hprob.begin(), b->hprob.end(),
                                       [&](const ProbDev& P) { return P.nproj == 0 && line_covered(b, P); });
+  for (const void* fn : {(const void*)k_hpsi_batch<T, 0>, (const void*)k_hpsi_batch<T, 1>,
+                         (const void*)k_hpsi_batch<T, 2>, (const void*)k_hpsi_batch<T, 3>})
+    BCU(b, smem_all(fn));
   for (int sg : {32, 64, 128})
     for (int ppt : {2048, 4096, 8192}) {
       if (build_lists(b, sg, ppt) != PARO_OK) continue;  // the unit does not fit shared memory
-      for (int ph = 0; ph < 4; ++ph) {
-        const void* fn = ph == 0 ? (const void*)k_hpsi_batch<T, 0>
-                         : ph == 1 ? (const void*)k_hpsi_batch<T, 1>
-                         : ph == 2 ? (const void*)k_hpsi_batch<T, 2> : (const void*)k_hpsi_batch<T, 3>;
-        BCU(b, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
-      }
       for (int mode : {0, 1}) {
         if (mode == 0 && !b->groups.empty()) continue;
         int per_sm = 0;
@@ -1085,12 +1091,6 @@ int autotune(paro_batch* b) {
   if (best >= 1e30f) return berr(b, PARO_ERR_ARG, "batch: H psi kernel cannot be resident");
   int st = build_lists(b, best_sg, best_ppt);
   if (st) return berr(b, st, "batch: work lists");
-  for (int ph = 0; ph < 4; ++ph) {
-    const void* fn = ph == 0 ? (const void*)k_hpsi_batch<T, 0>
-                     : ph == 1 ? (const void*)k_hpsi_batch<T, 1>
-                     : ph == 2 ? (const void*)k_hpsi_batch<T, 2> : (const void*)k_hpsi_batch<T, 3>;
-    BCU(b, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
-  }
   unsigned h[3] = {0, 0, 0};
   BCU(b, cudaMemcpy(h, b->d_bar, sizeof(h), cudaMemcpyDeviceToHost));
   if (h[2]) return berr(b, PARO_ERR_TIMEOUT, "batch: grid barrier wait gave up");
