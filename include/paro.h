@@ -21,7 +21,8 @@
  *     paro_solve_source, paro_orthonormalize, paro_energy, the ParO and SCF steps and every call that takes
  *     Ritz pairs or residuals) returns PARO_ERR_TIMEOUT when such a wait gave up in it or in an
  *     enqueue-only call before it on the context (paro_apply_h, paro_apply_h_adjoint), whose
- *     output is then undefined. A time-out is reported once.
+ *     output is then undefined. paro_orthonormalize waits for its factorisation; its last product is
+ *     enqueued like those. A time-out is reported once.
  *   - A context is not thread-safe; distinct contexts are independent.
  *   - There is no CPU fallback: every numerical step runs in this library's CUDA kernels.
  */

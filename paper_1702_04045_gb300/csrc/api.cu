@@ -1463,16 +1463,6 @@ int paro_apply_vnl(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, vo
   return st ? st : tc_check(c);
 }
 
-// Status of a call that waits for the GPU: a tensor-core product that gave up leaves undefined sums, which the
-// factorisation or the solver may have met as a breakdown, so it is reported first.
-static int tc_status(Ctx* c, int st) {
-  if (st && st != PARO_ERR_BREAKDOWN) return st;
-  const std::string msg = c->err;
-  if (int s2 = tc_check(c)) return s2;
-  c->err = msg;
-  return st;
-}
-
 int paro_apply_h_adjoint(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, const void* w, void* g_psi,
                          double* g_v, double* g_pos) {
   CTX_CHECK(ctx);
@@ -1496,8 +1486,8 @@ int paro_orthonormalize(paro_ctx* ctx, int ik, int n, int dtype, const void* x, 
   if (x != y && xb < yb + bytes && yb < xb + bytes) return fail(c, PARO_ERR_ARG, "paro_orthonormalize: x and y overlap");
   if (x != y) PARO_CU(c, cudaMemcpyAsync(y, x, bytes, cudaMemcpyDeviceToDevice, c->stream));
   GammaPackOff general(c);
-  return tc_status(c, dtype == PARO_C64 ? orthonormalize<double>(c, ik, static_cast<double2*>(y), n)
-                                        : orthonormalize<float>(c, ik, static_cast<float2*>(y), n));
+  return dtype == PARO_C64 ? orthonormalize<double>(c, ik, static_cast<double2*>(y), n)
+                           : orthonormalize<float>(c, ik, static_cast<float2*>(y), n);
 }
 
 int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* eps, const void* psi, void* x,
@@ -1516,11 +1506,6 @@ int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* ep
   std::vector<double> hf(nb);
   for (int i = 0; i < nb; ++i) hf[i] = eps[i] - c->sigma_k[ik];
   if ((st0 = h2d_async(c, "ss_f", f, hf.data(), nb * sizeof(double)))) return st0;
-  std::vector<int> its;  // pcg_run reads the tensor-core flag back with the step counts
-  if (!iters_out) {
-    its.resize(nb);
-    iters_out = its.data();
-  }
   int st;
   if (dtype == PARO_C64) {
     double2* rhs = static_cast<double2*>(ws_get(c, "src_rhs64", (size_t)nb * npw * sizeof(double2)));
@@ -1529,7 +1514,7 @@ int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* ep
     if (st) return st;
     PARO_CU(c, cudaMemcpyAsync(x, psi, (size_t)nb * npw * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
     st = pcg_run<double>(c, ik, nb, rhs, static_cast<double2*>(x), false, rel_tol, max_it, iters_out);
-    return st == PARO_ERR_BREAKDOWN ? tc_status(c, st) : st;
+    return st || max_it > 0 ? st : tc_check(c);
   }
   float2* rhs = static_cast<float2*>(ws_get(c, "src_rhs32", (size_t)nb * npw * sizeof(float2)));
   if (!rhs) return PARO_ERR_CUDA;
@@ -1537,7 +1522,7 @@ int paro_solve_source(paro_ctx* ctx, int ik, int nb, int dtype, const double* ep
   if (st) return st;
   PARO_CU(c, cudaMemcpyAsync(x, psi, (size_t)nb * npw * sizeof(float2), cudaMemcpyDeviceToDevice, c->stream));
   st = pcg_run<float>(c, ik, nb, rhs, static_cast<float2*>(x), false, rel_tol, max_it, iters_out);
-  return st == PARO_ERR_BREAKDOWN ? tc_status(c, st) : st;
+  return st || max_it > 0 ? st : tc_check(c);
 }
 
 int paro_set_orbitals(paro_ctx* ctx, int ik, const void* psi, int on_device) {

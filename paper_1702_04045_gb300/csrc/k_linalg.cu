@@ -1284,6 +1284,8 @@ static int chol_piece(Ctx* c, int* piece) {
   return PARO_OK;
 }
 
+// Without defer the breakdown flag is read back here, and with it the tensor-core flag of the Gram product, which is
+// reported first: undefined sums may have caused the breakdown.
 int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int* skip) {
   {
     Ctx::CholShape sh;
@@ -1299,12 +1301,15 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
         int* flags = static_cast<int*>(ws_try(c, "chol_split_flags", levels * sizeof(int)));
         double2* W = static_cast<double2*>(
             ws_try(c, "chol_split", (3 * nn + 2 * levels * piece * piece) * sizeof(double2)));
+        const int* htc = nullptr;
         if (flags && W) {  // else the kernels below, which take two thirds of it or none
           PARO_CU(c, cudaMemcpyAsync(W, s, nn * sizeof(double2), cudaMemcpyDeviceToDevice, c->stream));
           if ((st = chol_split(c, n, W, n, g, n, W + nn, piece, flags, &nflag))) return st;
           std::vector<int> h(nflag);
+          if ((st = tc_flag_readback(c, &htc))) return st;
           PARO_CU(c, cudaMemcpyAsync(h.data(), flags, nflag * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
           PARO_CU(c, cudaStreamSynchronize(c->stream));
+          if (htc && (st = tc_report(c, *htc))) return st;
           for (int i = 0; i < nflag; ++i)
             if (h[i]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 in block " + std::to_string(i) +
                                                              ", column " + std::to_string(h[i] - 1));
@@ -1324,8 +1329,11 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
         return PARO_OK;
       }
       int h = 0;
+      const int* htc = nullptr;
+      if (!c->plain64 && (st = tc_flag_readback(c, &htc))) return st;
       PARO_CU(c, cudaMemcpyAsync(&h, flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
       PARO_CU(c, cudaStreamSynchronize(c->stream));
+      if (htc && (st = tc_report(c, *htc))) return st;
       if (h) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 at column " + std::to_string(h - 1));
       return PARO_OK;
     }
@@ -1348,8 +1356,11 @@ int chol_inv(Ctx* c, int n, const double2* s, double2* g, bool defer, const int*
   ++c->launches;
   prof_end(c, "k_chol", ev);
   int h[2] = {0, 0};
+  const int* htc = nullptr;
+  if (!c->plain64 && (st = tc_flag_readback(c, &htc))) return st;
   PARO_CU(c, cudaMemcpyAsync(h, flags + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   PARO_CU(c, cudaStreamSynchronize(c->stream));
+  if (htc && (st = tc_report(c, *htc))) return st;
   if (h[0]) return fail(c, PARO_ERR_TIMEOUT, "Cholesky: grid barrier wait gave up");
   if (h[1]) return fail(c, PARO_ERR_BREAKDOWN, "Cholesky pivot <= 0 at column " + std::to_string(h[1] - 1));
   return PARO_OK;

@@ -181,9 +181,10 @@ __global__ void __launch_bounds__(kVT) k_pcg_update(int npw, int nchunk, cplx<T>
 __global__ void k_pcg_band_beta(int nb, int nchunk, const double* __restrict__ prr, const double* __restrict__ prz,
                                 const double* __restrict__ r0n, double tol, double* __restrict__ rz,
                                 int* __restrict__ active, int* __restrict__ its, double* __restrict__ beta,
-                                int* __restrict__ still_out, int* __restrict__ nactive) {
+                                int* __restrict__ still_out, int* __restrict__ nactive, const int* __restrict__ tc) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nb) return;
+  if (b == 0) nactive[2] = tc ? *tc : 0;  // the products' time-out flag, read back with the counts
   if (!active[b]) {
     still_out[b] = 0;
     beta[b] = 0.0;
@@ -254,8 +255,8 @@ __global__ void k_shift_known(int npw, const cplx<T>* __restrict__ hx, const cpl
 
 // Solves (H - sigma_k) x_b = rhs_b for b < nb. On entry x holds the start vectors (ignored when
 // x0_zero), on exit the approximate solutions. Every orbital stops once ||r_b|| <= rel_tol ||r_b^0||
-// or after max_it steps; iters (host, may be null) receives the steps taken, and with them the tensor-core flag of
-// the products is read back and reported. hx0 (may be null): H x
+// or after max_it steps; iters (host, may be null) receives the steps taken. A time-out of the
+// tensor-core products is reported after the step that met it. hx0 (may be null): H x
 // of the start vectors when the caller already has it (the orbitals' H psi from the last
 // Rayleigh-Ritz step), which saves the first H application. hx (may be null; needs hx0 or x0_zero):
 // receives H x of the solutions, carried along the iteration from the products the solver forms anyway.
@@ -284,7 +285,7 @@ int pcg_run(Ctx* c, int ik, int nb, const cplx<T>* rhs, cplx<T>* x, bool x0_zero
   int* ib = static_cast<int*>(ws_get(c, "pcg_int", (size_t)(nb * 3 + 4) * sizeof(int)));
   if (!r || !p || !ap || !prz || !prr || !band || !ib) return PARO_ERR_CUDA;
   double *rz = band, *r0n = band + nb, *alpha = band + 2 * nb, *beta = band + 3 * nb;
-  int *active = ib, *its = ib + nb, *still = ib + 2 * nb, *flags = ib + 3 * nb;  // flags: nactive, bad
+  int *active = ib, *its = ib + nb, *still = ib + 2 * nb, *flags = ib + 3 * nb;  // flags: nactive, bad, time-out
   const dim3 gv(nchunk, nb);
   const int tb = (nb + 127) / 128;
   PARO_CU(c, cudaMemsetAsync(flags, 0, 2 * sizeof(int), c->stream));
@@ -316,7 +317,7 @@ int pcg_run(Ctx* c, int ik, int nb, const cplx<T>* rhs, cplx<T>* x, bool x0_zero
   PARO_LAUNCH(c, "k_pcg_band_init");
   // the first step runs without reading the active count back: every orbital with a nonzero initial
   // residual is active, and the kernels pass over the others
-  int hflags[2] = {1, 0};
+  int hflags[3] = {1, 0, 0};
   for (int it = 0; it < max_it && hflags[0] > 0; ++it) {
     st = apply_h<T>(c, ik, nb, p, ap, sigma, active);
     if (st) return st;
@@ -330,23 +331,21 @@ int pcg_run(Ctx* c, int ik, int nb, const cplx<T>* rhs, cplx<T>* x, bool x0_zero
     PARO_LAUNCH(c, "k_pcg_update");
     PARO_CU(c, cudaMemsetAsync(flags, 0, sizeof(int), c->stream));
     k_pcg_band_beta<<<tb, 128, 0, c->stream>>>(nb, nchunk, prr, prz, r0n, rel_tol, rz, active, its, beta, still,
-                                               flags);
+                                               flags, c->d_tc_err);
     PARO_LAUNCH(c, "k_pcg_band_beta");
     k_pcg_pupdate<T><<<gv, kVT, 0, c->stream>>>(npw, p, r, kin_ptr<T>(B), pshift, beta, still);
     PARO_LAUNCH(c, "k_pcg_pupdate");
     prof_end(c, f64 ? "pcg_vector<f64>" : "pcg_vector<f32>", ev);
     PARO_CU(c, cudaMemcpyAsync(active, still, nb * sizeof(int), cudaMemcpyDeviceToDevice, c->stream));
-    PARO_CU(c, cudaMemcpyAsync(hflags, flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    PARO_CU(c, cudaMemcpyAsync(hflags, flags, 3 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     PARO_CU(c, cudaStreamSynchronize(c->stream));
+    if (hflags[2]) return tc_report(c, 1);  // before a breakdown that undefined products may have caused
     if (hflags[1]) return fail(c, PARO_ERR_BREAKDOWN, "PCG breakdown (p^H A p <= 0 or not finite) in orbital " +
                                                          std::to_string(hflags[1] - 1));
   }
   if (iters) {
-    const int* htc = nullptr;
     PARO_CU(c, cudaMemcpyAsync(iters, its, nb * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    if ((st = tc_flag_readback(c, &htc))) return st;
     PARO_CU(c, cudaStreamSynchronize(c->stream));
-    if (htc) return tc_report(c, *htc);
   }
   return PARO_OK;
 }

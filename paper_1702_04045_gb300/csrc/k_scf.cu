@@ -1089,9 +1089,10 @@ __global__ void k_nonlocal(int nproj, int nb, const double2* __restrict__ P, con
 // per block partials of sum V_loc rho and sum rho eps_xc(rho)
 template <typename R>
 __global__ void k_grid_energies(int n, const double* __restrict__ vloc, const double* __restrict__ rho,
-                                double* __restrict__ part) {
+                                double* __restrict__ part, const int* __restrict__ tc, double* __restrict__ tc_out) {
   __shared__ double red[32];
   double sl = 0.0, sx = 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *tc_out = tc ? *tc : 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double e;
     if constexpr (sizeof(R) == 8) {
@@ -1113,7 +1114,8 @@ __global__ void k_grid_energies(int n, const double* __restrict__ vloc, const do
 int energy_terms(Ctx* c, const double* rho_dev, double terms[7]) {
   for (int i = 0; i < 7; ++i) terms[i] = 0.0;
   // every partial sum lands in one buffer, read back with a single synchronisation:
-  // [kinetic: nk x nocc x kKch][nonlocal: nk x nocc][V_loc rho, rho eps_xc: 2 x 304][Hartree blocks]
+  // [kinetic: nk x nocc x kKch][nonlocal: nk x nocc][V_loc rho, rho eps_xc: 2 x 304][Hartree blocks][time-out flag of
+  // the projections, which may be tensor-core products]
   constexpr int kKch = 4;  // chunks of each row for the kinetic sums (enough CTAs to fill the GPU)
   if (c->occ.size() != (size_t)c->nk * c->nb) {
     const int st = update_occupations(c);
@@ -1121,7 +1123,7 @@ int energy_terms(Ctx* c, const double* rho_dev, double terms[7]) {
   }
   const int nocc = c->kT > 0 ? c->nocc_eff : c->nocc;  // bands with an occupation
   const int nblk = 304, nh = hartree_blocks(c), nkb = c->nk * nocc, nkk = nkb * kKch;
-  const size_t ntot = (size_t)nkk + nkb + 2 * nblk + nh;
+  const size_t ntot = (size_t)nkk + nkb + 2 * nblk + nh + 1;
   double* part = static_cast<double*>(ws_get(c, "energy_part", ntot * sizeof(double)));
   double2* z = static_cast<double2*>(ws_get(c, "grid_c0", (size_t)c->ngrid * sizeof(double2)));
   if (!part || !z) return PARO_ERR_CUDA;
@@ -1148,15 +1150,13 @@ int energy_terms(Ctx* c, const double* rho_dev, double terms[7]) {
   }
   // eps_xc per point in FP64 on both paths (an FP32 evaluation shifts E_xc of the 64-atom cell by ~1e-5 Ha;
   // one pass over the grid, a few tens of microseconds in FP64)
-  k_grid_energies<double><<<nblk, 256, 0, c->stream>>>(c->ngrid, c->d_vloc, rho_dev, pg);
+  k_grid_energies<double><<<nblk, 256, 0, c->stream>>>(c->ngrid, c->d_vloc, rho_dev, pg, c->d_tc_err, part + ntot - 1);
   PARO_LAUNCH(c, "k_grid_energies");
   if ((st = hartree_g(c, rho_dev, z, ph, false))) return st;
   std::vector<double> h(ntot);
-  const int* htc = nullptr;  // the projections above may be tensor-core products
   PARO_CU(c, cudaMemcpyAsync(h.data(), part, ntot * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  if ((st = tc_flag_readback(c, &htc))) return st;
   PARO_CU(c, cudaStreamSynchronize(c->stream));
-  if (htc && (st = tc_report(c, *htc))) return st;
+  if (h[ntot - 1] != 0.0) return tc_report(c, 1);
   for (int ik = 0; ik < c->nk; ++ik) {
     double sk = 0, sn = 0;
     for (int b = 0; b < nocc; ++b) {
