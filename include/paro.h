@@ -195,8 +195,10 @@ int paro_apply_h(paro_ctx* ctx, int ik, int nb, int dtype, const void* psi, void
  * Kleinman-Bylander form):  out_b(G) = sum_p beta_p(G) D_p <beta_p|psi_b>.
  *   dtype  PARO_C64 or PARO_C32, as paro_apply_h; psi, out device, nb x npw complex of dtype (out is
  *          overwritten and must not alias psi).
- *   form   PARO_VNL_ACCURATE: FP64 products (PARO_C64), or FP32 products whose sums are carried in a
- *          two-sum pair (PARO_C32) -- the form the Rayleigh-Ritz step and the energy use;
+ *   form   PARO_VNL_ACCURATE: FP64 products (PARO_C64), or FP32 rows with sums that do not lose accuracy with
+ *          their length (PARO_C32): exact sums of the operands rounded to 2^-31 of their rows' largest value
+ *          from n_proj nb npw = 1.5e8 on, FP32 products carried in a two-sum pair below -- the form the
+ *          Rayleigh-Ritz step and the energy use;
  *          PARO_VNL_TENSOR (PARO_C32 only): the form of the inexact inner solves, 3xTF32 on the tensor
  *          cores with the projectors' split formed once per position set (relative error about 1e-5).
  *   Errors: PARO_ERR_ARG (bad argument, PARO_VNL_TENSOR with PARO_C64), PARO_ERR_STATE (no projectors

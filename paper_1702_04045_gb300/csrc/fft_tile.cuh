@@ -13,8 +13,12 @@
 // instruction in 32 cycles of a quarter SM (1/64 of the FP32 rate), a 64-bit integer addition is two
 // instructions of the full-rate integer pipe and a product with a 62-bit constant about a dozen, so the
 // butterflies of FP64 lines run in integers: a line is brought to the exponent of its largest value with
-// the headroom of its growth (N sqrt 2), transformed exactly but for the rounding of the twiddle products
-// to the last bit (2^-56 of the line's largest value), and converted back to FP64 with its exponent.
+// the headroom of its growth (N sqrt 2), transformed, and converted back to FP64 with its exponent. The error is
+// that of an FP64 transform, relative to the line: values are multiples of 2^-(62 - GROW) of the power of two above
+// the line's largest (2^-56 up to 45 points, 2^-55 up to 90, 2^-54 above), so that elements far below it keep fewer
+// bits than FP64 would, sums are exact, products are rounded to that unit, and the constants are doubles scaled by
+// 2^62 (the twiddles to 2^-54; sqrt 3 / 2, 1 / sqrt 2 and t_root's series to 6.5 x 2^-56). Results below the normal
+// range of FP64 become zero.
 #pragma once
 
 #include "paro_common.cuh"
@@ -190,12 +194,6 @@ template <bool INV> struct TDft<9, INV> {
 };
 template <bool INV> struct TDft<12, INV> {
   template <typename C> static __device__ __forceinline__ void run(C* v) { t_dft_2f<4, 3, INV>(v); }
-};
-template <bool INV> struct TDft<16, INV> {
-  template <typename C> static __device__ __forceinline__ void run(C* v) { t_dft_2f<4, 4, INV>(v); }
-};
-template <bool INV> struct TDft<18, INV> {
-  template <typename C> static __device__ __forceinline__ void run(C* v) { t_dft_2f<2, 9, INV>(v); }
 };
 
 // ---- line shapes ----

@@ -42,7 +42,9 @@ static const double kCouple = 1e-2;
 static const int kCoupleMaxCluster = 8;
 // longest cluster a warm start may leave: in the first hundred SCF iterations of the 64-atom cell the norm bound
 // joins most columns into one cluster, whose correction is then nil and whose Rayleigh-Ritz went to the FP64
-// solver (3.4 ms) or to long Jacobi sweeps (up to 0.9 ms); the FP32 solve takes about 1.1 ms
+// solver (3.4 ms) or to long Jacobi sweeps (up to 0.9 ms); the FP32 solve takes about 1.1 ms. No other cell was
+// measured: 24 lies between the clusters of a converged cell (up to kCoupleMaxCluster joined columns and the levels'
+// own degeneracies) and those of most of the columns.
 static const int kWarmMaxCluster = 24;
 
 // ------------------------------------------------------------------------------------------------

@@ -343,8 +343,10 @@ int gemm_cn(Ctx* c, int M, int N, int K, const cplx<TA>* A, int lda, const cplx<
             int ldc, bool herm, bool carry, const double* wscale, float2* wf) {
   if (M <= 0 || N <= 0) return PARO_OK;
   if constexpr (sizeof(TA) == 8 && sizeof(TB) == 8) {
-    // at every size the digit slices are faster than the FP64 pipe (Gram and V_nl of one 1189-coefficient row: 335 -> 85 us and 367 -> 70 us with the
-    // steps around them; 144 rows of 23847: 8.8 -> 0.81 ms and 17.7 -> 0.68 ms)
+    // The digit slices are faster than this file's FP64 kernels from one row up: Gram and V_nl of one row of 1189
+    // coefficients 335 -> 85 us and 367 -> 70 us with the steps around them, of 144 rows of 23847 8.8 -> 0.81 ms and
+    // 17.7 -> 0.68 ms. (One row is a few CTAs here, whose K slices stay at 256 so that the FP64 iteration keeps its
+    // sums; FP64 kernels with finer slices for small products were not tried.)
     if (K > 0 && slices_on(c)) {
       const int st = gemm_cn_slice<double>(c, M, N, K, A, lda, B, ldb, C, ldc, herm);
       if (st != kNoMemory) return st;

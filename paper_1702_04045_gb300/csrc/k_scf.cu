@@ -1345,7 +1345,7 @@ int pulay_mix(Ctx* c, const double* rho_out, int depth, double beta) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Ewald energy of point ions Z in a neutralising background (host, FP64)
+// Ewald energy of point ions Z in a neutralising background (sums on the GPU in FP64, read back when asked for)
 // ------------------------------------------------------------------------------------------------
 static const int kEwaldBlocks = 608;
 struct EwaldCell {

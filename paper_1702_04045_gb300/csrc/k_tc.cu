@@ -6,9 +6,8 @@
 // (re0, im0, re1, im1, ...) is a real row of twice the length, so for C = conj(A) B^T
 //   Re C = A' . B'              (A', B' the interleaved rows)
 //   Im C = A'' . B',  A'' = (-im0, re0, -im1, re1, ...)
-// A'' is formed in registers while the tile is staged. Two accumulators per tile (Re in TMEM columns
-// 0.., Im in 256..), six MMAs per 8-wide K step.
-// This file holds the pieces that the products with the projectors as the fixed operand share (k_tc_beta.cu).
+// The products are those with the projectors as the fixed operand (k_tc_beta.cu). This file holds what they share: the
+// presplit of the small matrix, the K split and the reduction of its parts.
 #include <algorithm>
 
 #include "paro_ctx.h"

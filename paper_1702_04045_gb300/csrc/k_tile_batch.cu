@@ -106,6 +106,8 @@ template <typename NT, int... Ns> struct BatchGrids {
     return st;
   }
 };
+// Up to 72 points: batches are of small cells, and every grid more is three kernels of each type to compile; larger
+// grids keep the shared-memory passes of k_batch.cu, untimed against these.
 using Batch32 = BatchGrids<NumF32, 27, 32, 36, 48, 54, 64, 72>;
 using Batch64 = BatchGrids<NumF64, 27, 32, 36, 48, 54, 64, 72>;
 
