@@ -3,6 +3,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -129,6 +131,21 @@ int pinned_wait(Ctx* c, const char* name) {
   if (it == c->pinned.end() || !it->second.ev) return PARO_OK;
   PARO_CU(c, cudaEventSynchronize(it->second.ev));
   return PARO_OK;
+}
+
+cudaError_t smem_all(const void* fn) {
+  static std::mutex mu;
+  static std::set<std::pair<const void*, int>> done;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  if (done.count({fn, dev})) return cudaSuccess;
+  cudaFuncAttributes at;
+  if ((e = cudaFuncGetAttributes(&at, fn)) != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)at.sharedSizeBytes);
+  if (e == cudaSuccess) done.insert({fn, dev});
+  return e;
 }
 
 // ------------------------------------------------------------------------------------------------

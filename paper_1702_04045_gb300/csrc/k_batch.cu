@@ -1016,15 +1016,6 @@ int build_lists(paro_batch* b, int sg, int ppt) {
   return PARO_OK;
 }
 
-// All the dynamic shared memory a kernel can be given: the limit is the kernel's, and a limit at one batch's need would
-// be taken away from the batches that live beside it
-cudaError_t smem_all(const void* fn) {
-  cudaFuncAttributes at;
-  const cudaError_t e = cudaFuncGetAttributes(&at, fn);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)at.sharedSizeBytes);
-}
-
 template <typename T>
 int autotune(paro_batch* b) {
   int dev = 0, sms = 0;

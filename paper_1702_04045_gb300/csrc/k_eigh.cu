@@ -749,7 +749,7 @@ int invit(Ctx* c, int n, const R* d, const R* e, const R* w, R* Z, int* info) {
   int E = (int)std::min<size_t>(32, (200 * 1024) / per);
   if (E < 1) return fail(c, PARO_ERR_ARG, "inverse iteration: n too large");
   const size_t sm = per * E;
-  PARO_CU(c, cudaFuncSetAttribute(k_invit_solve<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  PARO_CU(c, smem_all((const void*)k_invit_solve<R>));
   R* fac = static_cast<R*>(ws_get(c, f64 ? "invit_fac64" : "invit_fac32", (size_t)4 * n * n * sizeof(R)));
   unsigned char* swg = static_cast<unsigned char*>(ws_get(c, "invit_sw", (size_t)n * n));
   if (!fac || !swg) return PARO_ERR_CUDA;
@@ -788,7 +788,7 @@ int eigh_fp32_pieces(Ctx* c, int n, const float* d, const float* e, float* w, co
     if (smw <= 200 * 1024 && n >= 2) {
       k_wy_t<float><<<nblk, 256, 0, c->stream>>>(n, U, tau, Tb);
       PARO_LAUNCH(c, "k_wy_t");
-      PARO_CU(c, cudaFuncSetAttribute(k_wy_apply<float, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
+      PARO_CU(c, smem_all((const void*)k_wy_apply<float, CG>));
       k_wy_apply<float, CG><<<(n + CG - 1) / CG, 256, smw, c->stream>>>(n, U, Tb, ph, Z, V);
       PARO_LAUNCH(c, "k_wy_apply");
       prof_end(c, "eigh32_backtransform", ev);
@@ -798,7 +798,7 @@ int eigh_fp32_pieces(Ctx* c, int n, const float* d, const float* e, float* w, co
   const int cpb = 4;
   const size_t sms = ((size_t)n * n + (size_t)n * cpb) * sizeof(float2) + (size_t)n * sizeof(float);
   if (sms <= 220 * 1024) {  // reflectors in shared memory
-    PARO_CU(c, cudaFuncSetAttribute(k_backtransform_s<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sms));
+    PARO_CU(c, smem_all((const void*)k_backtransform_s<float>));
     k_backtransform_s<float><<<(n + cpb - 1) / cpb, 32 * cpb, sms, c->stream>>>(n, U, tau, ph, Z, V);
     PARO_LAUNCH(c, "k_backtransform_s");
     prof_end(c, "eigh32_backtransform", ev);
@@ -806,7 +806,7 @@ int eigh_fp32_pieces(Ctx* c, int n, const float* d, const float* e, float* w, co
   }
   const int cpb2 = 2;
   const size_t sm4 = (size_t)n * cpb2 * sizeof(float2);
-  PARO_CU(c, cudaFuncSetAttribute(k_backtransform<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));
+  PARO_CU(c, smem_all((const void*)k_backtransform<float>));
   k_backtransform<float><<<(n + cpb2 - 1) / cpb2, 32 * cpb2, sm4, c->stream>>>(n, U, (size_t)n, 1, tau, ph, Z, V);
   PARO_LAUNCH(c, "k_backtransform");
   prof_end(c, "eigh32_backtransform", ev);
@@ -875,7 +875,7 @@ int eigh(Ctx* c, int n, const double2* a, double* w, double2* v) {
   ev = prof_begin(c);
   const int cpb = 2;
   const size_t sm4 = (size_t)n * cpb * sizeof(double2);
-  PARO_CU(c, cudaFuncSetAttribute(k_backtransform<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm4));
+  PARO_CU(c, smem_all((const void*)k_backtransform<double>));
   k_backtransform<double><<<(n + cpb - 1) / cpb, 32 * cpb, sm4, c->stream>>>(n, Uh, usj, usi, tau, ph, Z, v);
   PARO_LAUNCH(c, "k_backtransform");
   prof_end(c, "k_backtransform", ev);

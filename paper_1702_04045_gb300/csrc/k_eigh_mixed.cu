@@ -919,7 +919,7 @@ int eigh_mixed(Ctx* c, int n, const double2* a, double* w, double2* v, int refin
   // 1. FP32 solve
   cudaEvent_t ev = prof_begin(c);
   const size_t sm1 = ((size_t)n * (n + 1) + 2 * (size_t)n) * sizeof(float2);
-  PARO_CU(c, cudaFuncSetAttribute(k_tridiag_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+  PARO_CU(c, smem_all((const void*)k_tridiag_cta));
   k_tridiag_cta<<<1, 1024, sm1, c->stream>>>(n, Af, U32, d32, e32, ph32, tau32, ecx32);
   PARO_LAUNCH(c, "k_tridiag_cta");
   prof_end(c, "k_tridiag_cta", ev);
@@ -975,7 +975,7 @@ static int eigh_finish_tail(Ctx* c, int n, const double2* a, double2* X, const d
   const size_t nn = (size_t)n * n;
   cudaEvent_t ev = prof_begin(c);
   const size_t sm3 = (size_t)2 * 64 * 65 * sizeof(double2);
-  PARO_CU(c, cudaFuncSetAttribute(k_cluster_rr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
+  PARO_CU(c, smem_all((const void*)k_cluster_rr));
   k_cluster_rr<<<n, 256, sm3, c->stream>>>(n, S, cst, ncl, X, lam, info);
   PARO_LAUNCH(c, "k_cluster_rr");
   k_eig_sort<<<(n + 127) / 128, 128, 0, c->stream>>>(n, lam, X, w, v, perm);

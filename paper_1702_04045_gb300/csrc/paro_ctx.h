@@ -191,6 +191,9 @@ void ws_drop(Ctx* c, const char* name);  // waits for the stream and frees the w
 // scope, whose pointers they are.
 static const int kNoMemory = 1;
 bool drop_optional(Ctx* c);
+// All the dynamic shared memory a kernel can be given, set once per device: the limit is the kernel's, and a limit at one
+// call's need could be taken away by another context's call before the launch
+cudaError_t smem_all(const void* fn);
 // host -> device copy on the context's stream through the pinned buffer `name`; src may change as soon as
 // this returns, and the call does not wait for the stream (only, rarely, for the buffer's previous copy)
 int h2d_async(Ctx* c, const char* name, void* dst, const void* src, size_t bytes);
