@@ -211,7 +211,7 @@ static void sphere(const Ctx* c, const double kf[3], double ecut, std::vector<in
 
 template <typename T>
 static int upload(Ctx* c, T** d, const std::vector<T>& h) {
-  PARO_CU(c, cudaMalloc(d, std::max<size_t>(h.size(), 1) * sizeof(T)));
+  PARO_CU(c, dev_malloc(c, d, std::max<size_t>(h.size(), 1) * sizeof(T)));
   if (!h.empty()) PARO_CU(c, cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
   return PARO_OK;
 }
@@ -369,12 +369,12 @@ int fp64_current(Ctx* c, Basis& b) {
 
 static int alloc_orbitals(Ctx* c, Basis& b) {
   if (!b.d_psi) {
-    PARO_CU(c, cudaMalloc(&b.d_psi, (size_t)c->nb * b.npw * sizeof(double2)));
-    PARO_CU(c, cudaMalloc(&b.d_hpsi, (size_t)c->nb * b.npw * sizeof(double2)));
+    PARO_CU(c, dev_malloc(c, &b.d_psi, (size_t)c->nb * b.npw * sizeof(double2)));
+    PARO_CU(c, dev_malloc(c, &b.d_hpsi, (size_t)c->nb * b.npw * sizeof(double2)));
   }
   if (c->prec == PARO_MIXED && !b.d_psi32) {
-    PARO_CU(c, cudaMalloc(&b.d_psi32, (size_t)c->nb * b.npw * sizeof(float2)));
-    PARO_CU(c, cudaMalloc(&b.d_hpsi32, (size_t)c->nb * b.npw * sizeof(float2)));
+    PARO_CU(c, dev_malloc(c, &b.d_psi32, (size_t)c->nb * b.npw * sizeof(float2)));
+    PARO_CU(c, dev_malloc(c, &b.d_hpsi32, (size_t)c->nb * b.npw * sizeof(float2)));
   }
   return PARO_OK;
 }
@@ -749,7 +749,7 @@ int update_occupations(Ctx* c) {
     }
   c->mts = -ts;
   c->nocc_eff = std::max(neff, 1);
-  if (!c->d_occ_sqrt) PARO_CU(c, cudaMalloc(&c->d_occ_sqrt, (size_t)nk * nb * sizeof(double)));
+  if (!c->d_occ_sqrt) PARO_CU(c, dev_malloc(c, &c->d_occ_sqrt, (size_t)nk * nb * sizeof(double)));
   int st = h2d_async(c, "occ_sqrt", c->d_occ_sqrt, sq.data(), sq.size() * sizeof(double));
   if (st) return st;
   c->occ_key.swap(key);
@@ -1046,7 +1046,7 @@ static int set_ecut(Ctx* c, double ecut_new) {
   const bool carry_rest = !carry_rho && c->have_veff;
   double2* fold = nullptr;
   if (carry_rho || carry_rest) {
-    PARO_CU(c, cudaMalloc(&fold, (size_t)ngold * sizeof(double2)));
+    PARO_CU(c, dev_malloc(c, &fold, (size_t)ngold * sizeof(double2)));
     k_rest_complex<<<(ngold + 255) / 256, 256, 0, c->stream>>>(ngold, carry_rho ? c->d_rho_in : c->d_veff,
                                                               carry_rest && c->have_pp ? c->d_vloc : nullptr, fold);
     PARO_LAUNCH(c, "k_rest_complex");
@@ -1103,7 +1103,7 @@ static int set_ecut(Ctx* c, double ecut_new) {
     PARO_CU(c, cudaStreamSynchronize(c->stream));
     cudaFree(fold);
     if (carry_rho) {
-      PARO_CU(c, cudaMalloc(&c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
+      PARO_CU(c, dev_malloc(c, &c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
       PARO_CU(c, cudaMemcpyAsync(c->d_rho_in, fr, (size_t)c->ngrid * sizeof(double), cudaMemcpyDeviceToDevice,
                                  c->stream));
       if ((st = veff_from_density(c, c->d_rho_in, nullptr, nullptr))) return st;
@@ -1302,7 +1302,7 @@ int paro_set_kb(paro_ctx* ctx, double rc, const double* D) {
     dv[4 * I] = D[2 * I];
     dv[4 * I + 1] = dv[4 * I + 2] = dv[4 * I + 3] = D[2 * I + 1];
   }
-  if (!c->d_dvec) PARO_CU(c, cudaMalloc(&c->d_dvec, std::max(c->nproj, 1) * sizeof(double)));
+  if (!c->d_dvec) PARO_CU(c, dev_malloc(c, &c->d_dvec, std::max(c->nproj, 1) * sizeof(double)));
   PARO_CU(c, cudaMemcpy(c->d_dvec, dv.data(), c->nproj * sizeof(double), cudaMemcpyHostToDevice));
   c->have_kb = c->nproj > 0;
   return PARO_OK;
@@ -1389,7 +1389,7 @@ int paro_get_vloc(paro_ctx* ctx, double* v_r) {
 int paro_set_density(paro_ctx* ctx, const double* rho, int on_device) {
   CTX_CHECK(ctx);
   if (!rho) return PARO_ERR_ARG;
-  if (!c->d_rho_in) PARO_CU(c, cudaMalloc(&c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
+  if (!c->d_rho_in) PARO_CU(c, dev_malloc(c, &c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
   PARO_CU(c, cudaMemcpyAsync(c->d_rho_in, rho, (size_t)c->ngrid * sizeof(double),
                              on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
   int st = veff_from_density(c, c->d_rho_in, nullptr, nullptr);
@@ -1642,7 +1642,7 @@ int paro_scf_step(paro_ctx* ctx, const paro_scf_opts* o, double energy[7], doubl
     if (!c->bases[ik].have_psi) return fail(c, PARO_ERR_STATE, "orbitals not set");
   int st;
   if (!c->have_rho) {  // first iteration: uniform density, Ritz pairs of the start span under its potential
-    if (!c->d_rho_in) PARO_CU(c, cudaMalloc(&c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
+    if (!c->d_rho_in) PARO_CU(c, dev_malloc(c, &c->d_rho_in, (size_t)c->ngrid * sizeof(double)));
     k_fill<<<(c->ngrid + 255) / 256, 256, 0, c->stream>>>(c->ngrid, 2.0 * c->nocc / c->omega, c->d_rho_in);
     PARO_LAUNCH(c, "k_fill");
     if ((st = veff_from_density(c, c->d_rho_in, nullptr, nullptr))) return st;

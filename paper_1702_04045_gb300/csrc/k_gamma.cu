@@ -155,7 +155,7 @@ int gamma_build_table(Ctx* c, int ik) {
     if (it == where.end()) return fail(c, PARO_ERR_ARG, "real-wavefunction mode: the basis is not symmetric");
     mg[g] = it->second;
   }
-  if (!B.d_mg) PARO_CU(c, cudaMalloc(&B.d_mg, (size_t)B.npw * sizeof(int)));
+  if (!B.d_mg) PARO_CU(c, dev_malloc(c, &B.d_mg, (size_t)B.npw * sizeof(int)));
   PARO_CU(c, cudaMemcpyAsync(B.d_mg, mg.data(), mg.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   PARO_CU(c, cudaStreamSynchronize(c->stream));
   return PARO_OK;

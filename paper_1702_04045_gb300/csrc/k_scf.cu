@@ -32,9 +32,9 @@ __global__ void k_twiddle(int n, double2* __restrict__ t64, float2* __restrict__
 int build_twiddles(Ctx* c) {
   for (int ax = 0; ax < 3; ++ax) {
     const int n = c->N[ax];
-    PARO_CU(c, cudaMalloc(&c->d_tw64[ax], n * sizeof(double2)));
-    PARO_CU(c, cudaMalloc(&c->d_tw32[ax], n * sizeof(float2)));
-    PARO_CU(c, cudaMalloc(&c->d_twfx[ax], n * sizeof(fxw)));
+    PARO_CU(c, dev_malloc(c, &c->d_tw64[ax], n * sizeof(double2)));
+    PARO_CU(c, dev_malloc(c, &c->d_tw32[ax], n * sizeof(float2)));
+    PARO_CU(c, dev_malloc(c, &c->d_twfx[ax], n * sizeof(fxw)));
     k_twiddle<<<(n + 127) / 128, 128, 0, c->stream>>>(n, c->d_tw64[ax], c->d_tw32[ax],
                                                       static_cast<fxw*>(c->d_twfx[ax]));
     PARO_LAUNCH(c, "k_twiddle");
@@ -214,7 +214,7 @@ int build_vloc(Ctx* c) {
   PARO_LAUNCH(c, "k_vloc_g");
   int st = fft3d<double>(c, vg, true);
   if (st) return st;
-  if (!c->d_vloc) PARO_CU(c, cudaMalloc(&c->d_vloc, (size_t)c->ngrid * sizeof(double)));
+  if (!c->d_vloc) PARO_CU(c, dev_malloc(c, &c->d_vloc, (size_t)c->ngrid * sizeof(double)));
   k_real_part<<<(c->ngrid + 255) / 256, 256, 0, c->stream>>>(c->ngrid, vg, c->d_vloc);
   PARO_LAUNCH(c, "k_real_part");
   return PARO_OK;
@@ -403,8 +403,8 @@ int build_beta(Ctx* c) {
     }
     PARO_CU(c, cudaMemcpyAsync(kph, hk.data(), c->nat * sizeof(double2), cudaMemcpyHostToDevice, c->stream));
     if (!b.d_beta) {
-      PARO_CU(c, cudaMalloc(&b.d_beta, (size_t)c->nproj * b.npw * sizeof(double2)));
-      PARO_CU(c, cudaMalloc(&b.d_beta32, (size_t)c->nproj * b.npw * sizeof(float2)));
+      PARO_CU(c, dev_malloc(c, &b.d_beta, (size_t)c->nproj * b.npw * sizeof(double2)));
+      PARO_CU(c, dev_malloc(c, &b.d_beta32, (size_t)c->nproj * b.npw * sizeof(float2)));
     }
     for (float4** img : {&b.d_beta_img_cn, &b.d_beta_img_wx}) {  // formed again from the new projectors
       if (*img) {
@@ -496,9 +496,9 @@ __global__ void k_min_sum_final(int nblk, const double* __restrict__ part, doubl
 
 int set_veff_device(Ctx* c, const double* v_dev) {
   if (!c->d_veff) {
-    PARO_CU(c, cudaMalloc(&c->d_veff, (size_t)c->ngrid * sizeof(double)));
-    PARO_CU(c, cudaMalloc(&c->d_vplane, (size_t)c->ngrid * sizeof(double)));
-    PARO_CU(c, cudaMalloc(&c->d_vplane32, (size_t)c->ngrid * sizeof(float)));
+    PARO_CU(c, dev_malloc(c, &c->d_veff, (size_t)c->ngrid * sizeof(double)));
+    PARO_CU(c, dev_malloc(c, &c->d_vplane, (size_t)c->ngrid * sizeof(double)));
+    PARO_CU(c, dev_malloc(c, &c->d_vplane32, (size_t)c->ngrid * sizeof(float)));
   }
   if (v_dev != c->d_veff)
     PARO_CU(c, cudaMemcpyAsync(c->d_veff, v_dev, (size_t)c->ngrid * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -1311,9 +1311,9 @@ int pulay_mix(Ctx* c, const double* rho_out, int depth, double beta) {
   const int n = c->ngrid;
   if (!c->d_pulay_rho || c->pulay_cap != depth) {
     if (c->d_pulay_rho) { cudaFree(c->d_pulay_rho); cudaFree(c->d_pulay_res); }
-    PARO_CU(c, cudaMalloc(&c->d_pulay_rho, (size_t)depth * n * sizeof(double)));
-    PARO_CU(c, cudaMalloc(&c->d_pulay_res, (size_t)depth * n * sizeof(double)));
-    if (!c->d_pulay_gram) PARO_CU(c, cudaMalloc(&c->d_pulay_gram, 16 * 16 * sizeof(double)));
+    PARO_CU(c, dev_malloc(c, &c->d_pulay_rho, (size_t)depth * n * sizeof(double)));
+    PARO_CU(c, dev_malloc(c, &c->d_pulay_res, (size_t)depth * n * sizeof(double)));
+    if (!c->d_pulay_gram) PARO_CU(c, dev_malloc(c, &c->d_pulay_gram, 16 * 16 * sizeof(double)));
     c->pulay_cap = depth;
     c->pulay_n = 0;
     c->pulay_head = 0;

@@ -75,8 +75,8 @@ int beta_images(Ctx* c, int ik) {
   const size_t nwx = (size_t)ntiles * B.img_wx_nstage * 2 * kTileF4;
   float4 *cn = nullptr, *wx = nullptr;
   auto form = [&]() -> int {
-    PARO_CU(c, cudaMalloc(&cn, ncn * sizeof(float4)));
-    PARO_CU(c, cudaMalloc(&wx, nwx * sizeof(float4)));
+    PARO_CU(c, dev_malloc(c, &cn, ncn * sizeof(float4)));
+    PARO_CU(c, dev_malloc(c, &wx, nwx * sizeof(float4)));
     k_beta_img_cn<<<dim3(304, mtiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_cn_nstage, B.d_beta32, cn);
     PARO_LAUNCH(c, "k_beta_img_cn");
     k_beta_img_wx<<<dim3(8, ntiles), 256, 0, c->stream>>>(c->nproj, B.npw, B.img_wx_nstage, B.d_beta32, wx);

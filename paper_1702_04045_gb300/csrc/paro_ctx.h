@@ -187,10 +187,18 @@ void* ws_try(Ctx* c, const char* name, size_t bytes);
 void ws_drop(Ctx* c, const char* name);  // waits for the stream and frees the workspace, if there is one
 // Memory that calls do without when it is short: the digit images of the projectors and of products' operands, and
 // the blocks the adjoint projects together. What cannot have them returns kNoMemory, before any launch, and its
-// caller takes the plain form. ws_get gives them up (drop_optional) before it fails, but not inside an OptionalInUse
-// scope, whose pointers they are.
+// caller takes the plain form. ws_get and dev_malloc give them up (drop_optional) before they fail, but not inside an
+// OptionalInUse scope, whose pointers they are.
 static const int kNoMemory = 1;
 bool drop_optional(Ctx* c);
+template <typename P> cudaError_t dev_malloc(Ctx* c, P** p, size_t bytes) {
+  cudaError_t e = cudaMalloc((void**)p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_optional(c)) {
+    cudaGetLastError();
+    e = cudaMalloc((void**)p, bytes);
+  }
+  return e;
+}
 // All the dynamic shared memory a kernel can be given, set once per device: the limit is the kernel's, and a limit at one
 // call's need could be taken away by another context's call before the launch
 cudaError_t smem_all(const void* fn);

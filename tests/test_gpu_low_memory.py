@@ -62,3 +62,28 @@ def test_calls_do_without_optional_memory(call, precision, dtype, spare, tol):
     assert torch.equal(got, again)
     # with the memory back, the same context takes the usual products again
     assert torch.equal(call(ctx, x).cpu(), ref)
+
+
+def test_own_allocations_take_the_images_back():
+    """A context that holds images (342 MB for the projectors alone) and finds 48 MB free still takes orbitals, whose
+    two arrays are 110 MB, with the workspaces of their Rayleigh-Ritz step."""
+    from paper_1702_04045_gb300 import paro
+
+    def context():
+        ctx = paro.context_from_config("si64_scf", "fp64")
+        return ctx, inputs.start_vectors(144, ctx.npw(), 3)
+
+    ctx, x = context()
+    ctx.set_orbitals(x)
+    ref = ctx.eigenvalues()
+    ctx.close()
+    ctx, x = context()
+    ctx.apply_vnl(torch.from_numpy(x).cuda())
+    torch.cuda.synchronize()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - 48 * MIB, dtype=torch.uint8, device="cuda")
+    try:
+        ctx.set_orbitals(x)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert np.array_equal(ctx.eigenvalues(), ref)
